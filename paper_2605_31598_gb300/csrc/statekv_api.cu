@@ -32,7 +32,7 @@ size_t round_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 constexpr size_t kGuard = STATEKV_DEBUG_CHECKS ? kGuardBytes : 0;
 
 struct Layout {
-    size_t state_k, state_v, positions, counts, frames, text, cache_k, cache_v, partials;
+    size_t state_k, state_v, positions, counts, frames, text, tickets, cache_k, cache_v, partials;
     struct Staging {
         size_t q, k, v, out, imp;
     } stg[2];  // host-buffer calls: two frames, so copies overlap the steps
@@ -96,6 +96,7 @@ Layout make_layout(const statekv_config& c, const Derived& d)
     L.counts = take(heads * 4);
     L.frames = take(heads * 4);
     L.text = take(heads * 4);  // decode-cache rows appended after the video frames
+    L.tickets = take(heads * 4);  // decode kernel: finished CTAs per head, 0 between calls
     L.cache_k = take(heads * static_cast<size_t>(d.cap) * D * 2);
     L.cache_v = take(heads * static_cast<size_t>(d.cap) * D * 2);
     // importance partials of a frame step; a decode step's split-K partials
@@ -449,8 +450,9 @@ statekv_status run_decode(statekv_handle* h, const statekv_decode_args& a, cudaS
     ap.cap = d.cap;
     ap.status = h->status_dev;
     if (n * d.G <= kDecodeRows) {
-        // A few rows: the new tokens' K/V go into the cache first, then the
-        // one-pass split-K kernel reads every key once from the cache.
+        // A few rows: one launch of the one-pass split-K kernel, which puts the
+        // new tokens' K/V into the cache, reads every key once from it and
+        // advances the token counts.
         long long maxlen = 0;
         for (int s = a.stream_begin; s < a.stream_begin + a.stream_count; ++s)
             for (int l = a.layer_begin; l < a.layer_begin + a.layer_count; ++l) {
@@ -478,10 +480,13 @@ statekv_status run_decode(statekv_handle* h, const statekv_decode_args& a, cudaS
         }
         dp.q = static_cast<const __nv_bfloat16*>(a.q);
         dp.out = static_cast<__nv_bfloat16*>(a.out);
+        dp.k = ap.k;
+        dp.v = ap.v;
         dp.cache_k = ap.cache_k;
         dp.cache_v = ap.cache_v;
         dp.frames = frames;
         dp.text = text;
+        dp.tickets = h->at<unsigned>(h->lay.tickets);
         dp.part_o = h->at<float>(h->lay.partials);
         dp.part_ml = dp.part_o + static_cast<size_t>(U) * Hkv * dp.nchunk * kDecodeRows * D;
         dp.units = ur;
@@ -494,9 +499,7 @@ statekv_status run_decode(statekv_handle* h, const statekv_decode_args& a, cudaS
         dp.scale_log2 = d.scale * 1.4426950408889634f;
         dp.status = h->status_dev;
         dp.watchdog_ns = 1000000ull * (c.watchdog_ms ? c.watchdog_ms : 2000u);
-        if (timed(h, 0, st, [&] { return launch_append(ap, st); }) != cudaSuccess ||
-            timed(h, 1, st, [&] { return launch_decode(h->tm_dk, h->tm_dv, dp, D, U, st); }) != cudaSuccess ||
-            launch_advance(text, ur, U, Hkv, n, st) != cudaSuccess)
+        if (timed(h, 1, st, [&] { return launch_decode(h->tm_dk, h->tm_dv, dp, D, U, st); }) != cudaSuccess)
             return STATEKV_ERR_CUDA;
         for (int s = a.stream_begin; s < a.stream_begin + a.stream_count; ++s)
             for (int l = a.layer_begin; l < a.layer_begin + a.layer_count; ++l)

@@ -255,16 +255,19 @@ constexpr int kDecodeMaxChunks = 64;
 struct DecodeParams {
     const __nv_bfloat16* q;     // [U][n][Hq][D]
     __nv_bfloat16* out;         // [U][n][Hq][D]
-    const __nv_bfloat16* cache_k;  // arena [S*L][Hkv][cap][D]
-    const __nv_bfloat16* cache_v;
+    const __nv_bfloat16* k;     // [U][n][Hkv][D]: the new tokens' rows, appended to the cache
+    const __nv_bfloat16* v;
+    __nv_bfloat16* cache_k;     // arena [S*L][Hkv][cap][D]
+    __nv_bfloat16* cache_v;
     const int32_t* frames;      // arena [S*L][Hkv]: rows before = frames * T + text
-    const int32_t* text;
+    int32_t* text;              // advanced by n
+    unsigned* tickets;          // arena [S*L][Hkv]: CTAs of the head that have finished; 0 between calls
     float* part_o;              // [U][Hkv][nchunk][kDecodeRows][D]
     float* part_ml;             // [U][Hkv][nchunk][kDecodeRows][2]
     UnitRange units;
     int n, G, Hq, Hkv, T;
     long long cap;
-    int ck, nchunk;             // keys per chunk (a multiple of 256), chunks
+    int ck, nchunk;             // keys per chunk (a multiple of 128), chunks
     float scale_log2;
     int32_t* status;
     unsigned long long watchdog_ns;

@@ -106,3 +106,60 @@ def test_decode_refuses_rows_beyond_the_cache():
     q, k, v = _text_tokens(shape, 1, seed=9, device="cuda")
     assert eng.decode_step(q, k, v, torch.empty_like(q)) == 3
     assert eng.sync() == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hq,hkv,d,T,frames,layers,steps", [
+    # one head: the new tokens' rows straddle a chunk's end (rows 254..257), then start one
+    (4, 1, 128, 127, 2, 1, (4, 1, 3)),
+    (16, 1, 64, 128, 1, 2, (1, 1)),      # 16 rows per token; the new row opens a chunk
+    (2, 2, 64, 33, 1, 1, (8, 2)),        # fewer keys than a chunk
+    (14, 2, 64, 259, 7, 3, (1, 2, 1)),   # ragged lengths, several units
+    (7, 1, 128, 1024, 9, 1, (1, 1)),     # one head over all of its chunks (64)
+])
+def test_decode_token_edges(hq, hkv, d, T, frames, layers, steps):
+    """One-launch decode steps (at most 16 query rows per KV head), per layer
+    and over all layers in turn, against the oracle's exact attention."""
+    import __graft_entry__ as g
+
+    from paper_2605_31598_gb300.inputs import Shape
+
+    g.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    shape = Shape(hq, hkv, d, T, 64, frames + 1, num_layers=layers, kind="peaked")
+    eng = StateKV(make_config(shape))
+    hist = [([], []) for _ in range(layers)]
+    for n in range(1, frames + 1):
+        q, k, v = batch_qkv(shape, n, streams=[0], layers=range(layers), device="cuda")
+        assert eng.prefill_frame(q, k, v, torch.empty_like(q)) == 0
+        for l in range(layers):
+            hist[l][0].append(oracle.as_bf16_bits(k[0, l]))
+            hist[l][1].append(oracle.as_bf16_bits(v[0, l]))
+    done = frames * T
+    for i, nt in enumerate(steps):
+        q, k, v = (x * d ** 0.5 for x in _text_tokens(shape, nt, seed=300 + i, device="cuda"))
+        out = torch.full_like(q, float("nan"))
+        if i % 2:  # every layer in one call, else one call per layer
+            assert eng.decode_step(q, k, v, out) == 0
+        else:
+            for l in range(layers):
+                part = tuple(x[:, l:l + 1].contiguous() for x in (q, k, v, out))
+                assert eng.decode_step(*part, layer_begin=l, layer_count=1) == 0
+                out[:, l:l + 1] = part[3]
+        torch.cuda.synchronize()
+        for l in range(layers):
+            hist[l][0].append(oracle.as_bf16_bits(k[0, l]))
+            hist[l][1].append(oracle.as_bf16_bits(v[0, l]))
+            ks, vs = np.concatenate(hist[l][0]), np.concatenate(hist[l][1])
+            ref = oracle.full_attention(oracle.as_bf16_bits(q[0, l]), ks, vs, done, causal=True)
+            got = out[0, l].float().cpu().numpy()
+            assert np.isfinite(got).all()
+            err = float(np.abs(got - ref).max())
+            assert err <= OUT_ATOL, f"step {i} ({nt} tokens) layer {l}: max |O - O_exact| = {err}"
+            ck, cv, info = eng.cache(0, l)
+            assert info.length == done + nt
+            assert np.array_equal(oracle.as_bf16_bits(ck[:, :done + nt].transpose(0, 1)), ks)
+            assert np.array_equal(oracle.as_bf16_bits(cv[:, :done + nt].transpose(0, 1)), vs)
+        done += nt
+    assert eng.sync() == 0
