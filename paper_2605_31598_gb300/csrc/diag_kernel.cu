@@ -6,15 +6,21 @@
 //                       shared protocol sums the weights over the frame's
 //                       queries within each head, then over the heads)
 //   topb_mask           top-B membership of each row, ties to the lower
-//                       position: an MSB-first radix select over the 64-bit
-//                       key (score bits << 32 | ~position), read from global
-//                       memory on every pass, so rows may be arbitrarily long
+//                       position: an MSB-first radix select over the score
+//                       bits (11 + 11 + 9), then, among scores equal to the
+//                       threshold, the lowest positions
 //   concentration_sums  App. A.1: mass of the top-B historical keys and of
 //                       all historical keys
 //   state_metrics       App. A.2: the counts and weights behind candidate-pool
 //                       recall, weighted recall, retention and churn
-// Every reduction is one CTA per row with a fixed-order fp64 tree, so the
-// results are deterministic.
+// A few dozen rows of tens of thousands of scores are too few CTAs at one per
+// row, and each CTA then walks its row alone: 28 rows of 25k scores took 50 us
+// (top-B: up to eight passes), 27 us (concentration: two fp64 adds per score on
+// 28 SMs) and 65 us (metrics).  A row is therefore shared by the CTAs of one
+// thread-block cluster (row_cluster), which merge their histograms and sums in
+// distributed shared memory: 16, 11 and 12 us.  Sums are
+// added in one fixed order for a given cluster size, so they are deterministic.
+#include "sm103_ptx.cuh"
 #include "statekv_kernels.cuh"
 
 namespace statekv {
@@ -22,22 +28,50 @@ namespace {
 
 constexpr int kDiagThreads = 512;
 
-// Sum of one double per thread over the block; thread 0 gets the total.
-__device__ double block_sum(double x, double* sh)
+constexpr int kDiagWarps = kDiagThreads / 32;
+constexpr int kDiagBatch = 8;  // scores per thread in flight (and kept between passes)
+
+// Sums of two doubles per thread over the block; thread 0 gets them.  An fp64
+// add of a warp takes 16 cycles of the SM, so the warps reduce both values at
+// once, one in each half (5 adds where two full trees take 10).
+__device__ void block_sum2(double a, double b, double* sh, double (&out)[2])
 {
+    static_assert(kDiagWarps == 16, "one warp adds the warps' two sums");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool up = lane >= 16;
+    double x = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if (lane == 0) sh[warp] = x;
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((lane & 15) == 0) sh[(up ? kDiagWarps : 0) + warp] = x;
     __syncthreads();
-    double t = 0.0;
     if (warp == 0) {
-        t = lane < kDiagThreads / 32 ? sh[lane] : 0.0;
+        x = sh[lane];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        out[0] = x;
+        out[1] = __shfl_sync(0xffffffffu, x, 16);
     }
     __syncthreads();
-    return t;
+}
+
+// Sum of one count per thread over the block (fewer than 2^32); thread 0 gets it.
+__device__ unsigned block_count(unsigned x, unsigned* sh)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    x = __reduce_add_sync(0xffffffffu, x);
+    if (lane == 0) sh[warp] = x;
+    __syncthreads();
+    if (warp == 0) x = __reduce_add_sync(0xffffffffu, lane < kDiagWarps ? sh[lane] : 0u);
+    __syncthreads();
+    return x;
+}
+
+// The CTA's share [lo, hi) of the row's entries [0, n): rank r of C.
+__device__ __forceinline__ void row_share(long long n, int r, int C, long long& lo, long long& hi)
+{
+    const long long per = (n + C - 1) / C;
+    lo = min(n, per * r);
+    hi = min(n, lo + per);
 }
 
 __global__ void scores_reduce(const ScoresParams p)
@@ -61,146 +95,289 @@ __global__ void scores_reduce(const ScoresParams p)
     p.scores[static_cast<size_t>(u) * p.ncols + j] = s;
 }
 
-// Selection key of entry j: order-preserving bits of the (non-negative)
-// score, then the complement of the position so that the lower position wins
-// a tie.  Negative scores and NaN count as 0.
-__device__ __forceinline__ unsigned long long topb_key(const float* row, long long j)
+// Order-preserving bits of a (non-negative) score.  Negative scores and NaN
+// count as 0.
+__device__ __forceinline__ unsigned score_bits(float x)
 {
-    const float x = row[j];
-    const float c = x > 0.f ? x : 0.f;  // also maps NaN to 0
-    return (static_cast<unsigned long long>(__float_as_uint(c)) << 32) |
-           static_cast<unsigned>(0xFFFFFFFFu - static_cast<unsigned>(j));
+    return __float_as_uint(x > 0.f ? x : 0.f);  // also maps NaN to 0
 }
 
+__device__ __forceinline__ unsigned ld_dsmem_u32(uint32_t addr)
+{
+    unsigned v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_dsmem_f64(uint32_t addr)
+{
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void red_dsmem_add(uint32_t addr, unsigned v)
+{
+    asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+constexpr int kTopbBins = 2048;
+
+// One cluster of C CTAs per row.  Every pass, each CTA counts its share's digits,
+// adds the non-empty bins to the first CTA's counts of that pass, and finds the
+// bin of the k-th largest key in the merged counts.
 __global__ void __launch_bounds__(kDiagThreads) topb_mask_kernel(const float* scores, long long n,
                                                                  long long stride, long long B,
-                                                                 uint8_t* mask)
+                                                                 uint8_t* mask, int C)
 {
-    __shared__ unsigned hist[256];
-    __shared__ unsigned long long sh_prefix, sh_mask;
-    __shared__ long long sh_k;
-    __shared__ int sh_done;
-    const float* row = scores + static_cast<size_t>(blockIdx.x) * stride;
-    uint8_t* mrow = mask + static_cast<size_t>(blockIdx.x) * stride;
-    const int tid = threadIdx.x, lane = tid & 31;
-    unsigned long long prefix = 0, msk = 0;
-    bool none = B <= 0;
-    if (!none && n > B) {
-        if (tid == 0) {
-            sh_k = B;
-            sh_done = 0;
+    __shared__ __align__(16) unsigned hist[kTopbBins], merged[3][kTopbBins];
+    __shared__ unsigned wsum[kDiagWarps];
+    __shared__ unsigned sh_bin, sh_count, sh_equal;
+    __shared__ unsigned long long sh_k;
+    const int r = blockIdx.x % C, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long rowi = blockIdx.x / C;
+    const float* row = scores + static_cast<size_t>(rowi) * stride;
+    uint8_t* mrow = mask + static_cast<size_t>(rowi) * stride;
+    long long lo, hi;
+    row_share(n, r, C, lo, hi);
+    // this thread's entries base + tid + e kDiagThreads of a batch, as score bits
+    unsigned x[kDiagBatch] = {};
+    auto load = [&](long long base) {
+#pragma unroll
+        for (int e = 0; e < kDiagBatch; ++e) {
+            const long long i = base + tid + e * kDiagThreads;
+            x[e] = i < hi ? score_bits(row[i]) : 0u;
         }
-        __syncthreads();
-        for (int shift = 56; shift >= 0; shift -= 8) {
-            for (int i = tid; i < 256; i += kDiagThreads) hist[i] = 0;
-            __syncthreads();
-            for (long long i0 = 0; i0 < n; i0 += kDiagThreads) {
-                const long long i = i0 + tid;
-                int digit = -1;
-                if (i < n) {
-                    const unsigned long long k = topb_key(row, i);
-                    if ((k & msk) == prefix) digit = static_cast<int>((k >> shift) & 0xFF);
-                }
-                const unsigned peers = __match_any_sync(0xffffffffu, digit);
-                if (digit >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], __popc(peers));
-            }
-            __syncthreads();
-            if (tid < 32) {
-                // lane owns digits 255 - 8 lane - e, e = 0..7 (descending)
-                unsigned c[8], local = 0;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    c[e] = hist[255 - 8 * lane - e];
-                    local += c[e];
-                }
-                unsigned incl = local;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                const unsigned long long excl = incl - local;
-                const long long k = sh_k;
-                if (static_cast<long long>(excl) < k && static_cast<long long>(incl) >= k) {
-                    long long above = static_cast<long long>(excl);
+    };
+    constexpr long long kStep = kDiagBatch * kDiagThreads;
+    const bool cached = hi - lo <= kStep;  // the share stays in registers
+    const bool none = B <= 0, all = n <= B;
+    unsigned thr = 0, tmask = 0;           // kept: (bits & tmask) > thr, or equal and among the first `ties`
+    unsigned long long ties = ~0ull;       // equal entries to keep, in position order (~0: all)
+    if (!none && !all) {
+        if (cached) load(lo);
+        for (int i = tid; i < 3 * kTopbBins; i += kDiagThreads) (&merged[0][0])[i] = 0;
+        ptx::cluster_sync();
+        unsigned long long k = static_cast<unsigned long long>(B);
 #pragma unroll 1
-                    for (int e = 0; e < 8; ++e) {
-                        if (above + c[e] >= k) {
-                            const unsigned long long dgt = 255 - 8 * lane - e;
-                            sh_prefix = prefix | (dgt << shift);
-                            sh_mask = msk | (0xFFull << shift);
-                            sh_k = k - above;
-                            sh_done = (static_cast<long long>(c[e]) == k - above) ? 1 : 0;
-                            break;
-                        }
-                        above += c[e];
+        for (int pass = 0; pass < 3; ++pass) {
+            const int shift = pass == 0 ? 20 : pass == 1 ? 9 : 0;
+            const unsigned dmask = pass == 2 ? 0x1FFu : 0x7FFu;
+            for (int i = tid; i < kTopbBins; i += kDiagThreads) hist[i] = 0;
+            __syncthreads();
+            for (long long base = lo; base < hi; base += kStep) {
+                if (!cached) load(base);
+#pragma unroll
+                for (int e = 0; e < kDiagBatch; ++e)
+                    if (base + tid + e * kDiagThreads < hi && (x[e] & tmask) == thr)
+                        atomicAdd(&hist[(x[e] >> shift) & dmask], 1u);
+            }
+            __syncthreads();
+            const uint32_t m0 = ptx::dsmem_addr(ptx::smem_addr(merged[pass]), 0);
+            for (int i = tid; i < kTopbBins; i += kDiagThreads)
+                if (hist[i]) red_dsmem_add(m0 + 4 * i, hist[i]);
+            ptx::cluster_sync();
+            // the bin, from the largest digit down: thread t owns the four digits
+            // 2047 - 4 t - j (one 16-byte remote load: as four words, the eight
+            // CTAs' reads of one SM took 6 us a pass)
+            const float4 c4 = ptx::ld_dsmem_f4(m0 + 4 * (kTopbBins - 4 - 4 * tid));
+            const unsigned c[4] = {__float_as_uint(c4.w), __float_as_uint(c4.z), __float_as_uint(c4.y),
+                                   __float_as_uint(c4.x)};
+            const unsigned local = c[0] + c[1] + c[2] + c[3];
+            unsigned incl = local;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) wsum[warp] = incl;
+            __syncthreads();
+            unsigned long long above = incl - local;
+            for (int w = 0; w < warp; ++w) above += wsum[w];
+            if (above < k && above + local >= k) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (above < k && above + c[j] >= k) {
+                        sh_bin = kTopbBins - 1 - 4 * tid - j;
+                        sh_count = c[j];
+                        sh_k = k - above;
                     }
+                    above += c[j];
                 }
             }
             __syncthreads();
-            prefix = sh_prefix;
-            msk = sh_mask;
-            if (sh_done) break;
+            thr |= sh_bin << shift;
+            tmask |= dmask << shift;
+            k = sh_k;
+            if (sh_count == k) break;  // every entry of the bin is kept
+            if (pass == 2) ties = k;
+        }
+        if (ties != ~0ull) {
+            // the k lowest positions among the entries equal to the threshold: the
+            // CTAs' counts of them, in rank order, are in their last histograms
+            if (tid == 0) sh_equal = hist[thr & 0x1FFu];
+            ptx::cluster_sync();
+            unsigned long long before = 0;
+            for (int q = 0; q < r; ++q) before += ld_dsmem_u32(ptx::dsmem_addr(ptx::smem_addr(&sh_equal), q));
+            ties = before < ties ? ties - before : 0;
+        }
+        ptx::cluster_sync();  // no CTA leaves while others read its shared memory
+    }
+    // kept(j) <=> j < n and key(j) above the threshold, or equal and in time
+    unsigned long long seen = 0;  // equal entries of this CTA's earlier batches
+    for (long long base = lo; base < hi; base += kStep) {
+        if (!none && !all && !cached) load(base);
+#pragma unroll
+        for (int e = 0; e < kDiagBatch; ++e) {
+            const long long i = base + tid + e * kDiagThreads;
+            const unsigned d = x[e] & tmask;
+            bool keep = all || d > thr || (d == thr && ties == ~0ull);
+            if (ties != ~0ull) {  // rank of the equal entries, in position order (uniform branch)
+                const bool eq = i < hi && d == thr;
+                const unsigned bal = __ballot_sync(0xffffffffu, eq);
+                if (lane == 0) wsum[warp] = __popc(bal);
+                __syncthreads();
+                unsigned long long rank = seen + __popc(bal & ((1u << lane) - 1));
+                unsigned total = 0;
+                for (int w = 0; w < kDiagWarps; ++w) {
+                    if (w < warp) rank += wsum[w];
+                    total += wsum[w];
+                }
+                seen += total;
+                __syncthreads();
+                if (eq) keep = rank < ties;
+            }
+            if (i < hi) mrow[i] = !none && keep ? 1 : 0;
         }
     }
-    // kept(j) <=> j < n and (key(j) & mask) >= prefix (prefix 0: every entry)
-    for (long long j = tid; j < stride; j += kDiagThreads) {
-        uint8_t keep = 0;
-        if (!none && j < n) keep = (topb_key(row, j) & msk) >= prefix ? 1 : 0;
-        mrow[j] = keep;
+    long long t0, t1;  // entries past n
+    row_share(stride - n, r, C, t0, t1);
+    for (long long j = n + t0 + tid; j < n + t1; j += kDiagThreads) mrow[j] = 0;
+}
+
+// The cluster's partial sums, one set per CTA, added in rank order by the first.
+template <int K>
+__device__ void cluster_total(const double (&v)[K], double* sh, int r, int C, double* out)
+{
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int i = 0; i < K; ++i) sh[i] = v[i];
+    ptx::cluster_sync();
+    if (r == 0 && threadIdx.x < K) {
+        double t = 0.0;
+        for (int q = 0; q < C; ++q)
+            t += ld_dsmem_f64(ptx::dsmem_addr(ptx::smem_addr(sh + threadIdx.x), q));
+        out[threadIdx.x] = t;
     }
+    ptx::cluster_sync();
 }
 
 __global__ void __launch_bounds__(kDiagThreads) concentration_kernel(const float* scores,
                                                                      const uint8_t* mask,
                                                                      long long n, long long stride,
-                                                                     double* out)
+                                                                     double* out, int C)
 {
-    __shared__ double sh[kDiagThreads / 32];
-    const float* row = scores + static_cast<size_t>(blockIdx.x) * stride;
-    const uint8_t* mrow = mask + static_cast<size_t>(blockIdx.x) * stride;
-    double top = 0.0, all = 0.0;
-    for (long long j = threadIdx.x; j < n; j += kDiagThreads) {
-        const double x = row[j];
-        all += x;
-        if (mrow[j]) top += x;
+    __shared__ double sh[2 * kDiagWarps], part[2];
+    const int r = blockIdx.x % C;
+    const long long rowi = blockIdx.x / C;
+    const float* row = scores + static_cast<size_t>(rowi) * stride;
+    const uint8_t* mrow = mask + static_cast<size_t>(rowi) * stride;
+    long long lo, hi;
+    row_share(n, r, C, lo, hi);
+    double top = 0.0, rest = 0.0;  // one add per score: all = top + rest
+    for (long long base = lo; base < hi; base += kDiagBatch * kDiagThreads) {
+        float x[kDiagBatch];
+        bool in[kDiagBatch];
+#pragma unroll
+        for (int e = 0; e < kDiagBatch; ++e) {
+            const long long j = base + threadIdx.x + e * kDiagThreads;
+            x[e] = j < hi ? row[j] : 0.f;
+            in[e] = j < hi && mrow[j];
+        }
+#pragma unroll
+        for (int e = 0; e < kDiagBatch; ++e) {
+            const double t = (in[e] ? top : rest) + x[e];
+            top = in[e] ? t : top;
+            rest = in[e] ? rest : t;
+        }
     }
-    top = block_sum(top, sh);
-    all = block_sum(all, sh);
-    if (threadIdx.x == 0) {
-        out[2 * blockIdx.x] = top;
-        out[2 * blockIdx.x + 1] = all;
-    }
+    double v[2] = {};
+    block_sum2(top, rest, sh, v);
+    v[1] += v[0];
+    cluster_total(v, part, r, C, out + 2 * rowi);
 }
 
 __global__ void __launch_bounds__(kDiagThreads) state_metrics_kernel(
     const uint8_t* mask_n, const uint8_t* mask_n1, const float* w, long long n_seen, int T,
-    long long stride, double* out)
+    long long stride, double* out, int C)
 {
-    __shared__ double sh[kDiagThreads / 32];
-    const size_t base = static_cast<size_t>(blockIdx.x) * stride;
-    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (long long j = threadIdx.x; j < n_seen + T; j += kDiagThreads) {
-        const bool in_n = j < n_seen && mask_n[base + j];
-        const bool in_n1 = mask_n1[base + j] != 0;
-        const bool in_pool = in_n || j >= n_seen;  // S_n plus frame n + 1
-        const double x = w[base + j];
-        if (in_n1) {
-            v[1] += 1.0;
-            v[3] += x;
-            if (in_pool) {
-                v[0] += 1.0;
-                v[2] += x;
-            }
-            if (in_n) v[4] += 1.0;
+    __shared__ double sh[2 * kDiagWarps], part[6];
+    __shared__ unsigned shi[kDiagWarps];
+    const int r = blockIdx.x % C;
+    const long long rowi = blockIdx.x / C;
+    const size_t base0 = static_cast<size_t>(rowi) * stride;
+    long long lo, hi;
+    row_share(n_seen + T, r, C, lo, hi);
+    unsigned cnt[4] = {0, 0, 0, 0};  // |S_n1 & P|, |S_n1|, |S_n & S_n1|, |S_n| (a share has < 2^32 entries)
+    double in_p = 0.0, out_p = 0.0;  // w(S_n1 & P), w(S_n1 - P)
+    for (long long base = lo; base < hi; base += kDiagBatch * kDiagThreads) {
+        float x[kDiagBatch];
+        bool a[kDiagBatch], b[kDiagBatch], pool[kDiagBatch];
+#pragma unroll
+        for (int e = 0; e < kDiagBatch; ++e) {
+            const long long j = base + threadIdx.x + e * kDiagThreads;
+            a[e] = j < hi && j < n_seen && mask_n[base0 + j];  // in S_n
+            b[e] = j < hi && mask_n1[base0 + j] != 0;          // in S_n1
+            pool[e] = a[e] || j >= n_seen;                     // S_n plus frame n + 1
+            x[e] = j < hi ? w[base0 + j] : 0.f;
         }
-        if (in_n) v[5] += 1.0;
+#pragma unroll
+        for (int e = 0; e < kDiagBatch; ++e) {
+            cnt[0] += b[e] && pool[e];
+            cnt[1] += b[e];
+            cnt[2] += a[e] && b[e];
+            cnt[3] += a[e];
+            const double t = (pool[e] ? in_p : out_p) + (b[e] ? x[e] : 0.f);
+            in_p = pool[e] ? t : in_p;
+            out_p = pool[e] ? out_p : t;
+        }
     }
-#pragma unroll 1
-    for (int i = 0; i < 6; ++i) {
-        const double t = block_sum(v[i], sh);
-        if (threadIdx.x == 0) out[6 * blockIdx.x + i] = t;
-    }
+    double wt[2] = {};
+    block_sum2(in_p, out_p, sh, wt);
+    double v[6];
+    v[0] = block_count(cnt[0], shi);
+    v[1] = block_count(cnt[1], shi);
+    v[2] = wt[0];
+    v[3] = wt[0] + wt[1];
+    v[4] = block_count(cnt[2], shi);
+    v[5] = block_count(cnt[3], shi);
+    cluster_total(v, part, r, C, out + 6 * rowi);
+}
+
+// CTAs per row, a power of two up to 8 (the portable cluster size): no more than
+// give each about 2048 entries, and none added once the rows alone fill the SMs
+// twice.  28 rows of 25k scores: 50 us on one CTA
+// per row, 16 on eight (top-B).
+int row_cluster(int rows, long long n)
+{
+    int C = 1;
+    while (C < 8 && n / (2 * C) >= 2048 && static_cast<long long>(rows) * C < 304) C *= 2;
+    return C;
+}
+
+template <class... KArgs, class... Args>
+cudaError_t launch_rows(void (*kernel)(KArgs...), int rows, int C, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(rows) * C);
+    cfg.blockDim = dim3(kDiagThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args..., C);
 }
 
 }  // namespace
@@ -217,16 +394,14 @@ cudaError_t launch_topb_mask(const float* scores, int rows, long long n, long lo
                              long long B, uint8_t* mask, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    topb_mask_kernel<<<rows, kDiagThreads, 0, st>>>(scores, n, stride, B, mask);
-    return cudaGetLastError();
+    return launch_rows(topb_mask_kernel, rows, row_cluster(rows, n), st, scores, n, stride, B, mask);
 }
 
 cudaError_t launch_concentration(const float* scores, const uint8_t* mask, int rows, long long n,
                                  long long stride, double* out, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    concentration_kernel<<<rows, kDiagThreads, 0, st>>>(scores, mask, n, stride, out);
-    return cudaGetLastError();
+    return launch_rows(concentration_kernel, rows, row_cluster(rows, n), st, scores, mask, n, stride, out);
 }
 
 cudaError_t launch_state_metrics(const uint8_t* mask_n, const uint8_t* mask_n1, const float* w,
@@ -234,8 +409,8 @@ cudaError_t launch_state_metrics(const uint8_t* mask_n, const uint8_t* mask_n1, 
                                  cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    state_metrics_kernel<<<rows, kDiagThreads, 0, st>>>(mask_n, mask_n1, w, n_seen, T, stride, out);
-    return cudaGetLastError();
+    return launch_rows(state_metrics_kernel, rows, row_cluster(rows, n_seen + T), st, mask_n, mask_n1, w,
+                       n_seen, T, stride, out);
 }
 
 }  // namespace statekv

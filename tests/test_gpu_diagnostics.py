@@ -144,3 +144,42 @@ def test_concentration_end_to_end_on_the_toy_stream():
         _, s_ref = _oracle_scores(shape, got, hist, n)
         want = oracle.concentration(s_ref[: (n - 1) * T], budgets)
         np.testing.assert_allclose(c, want, rtol=2e-3, atol=1e-6)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,n,stride", [
+    (1, 4095, 4096),      # the last length one CTA takes alone
+    (5, 4097, 4300),      # two CTAs per row, ragged shares
+    (2, 16390, 16391),    # eight CTAs per row
+    (1, 70001, 70500),    # shares too long for the registers
+    (310, 5000, 5001),    # enough rows for one CTA each, longer than the registers
+])
+def test_row_kernels_over_cluster_sizes(rows, n, stride):
+    """Top-B masks (bit-exact, few and many ties), concentration and state
+    metrics of rows shared by one to eight CTAs, on the first, a middle and
+    the last row."""
+    _need_gpu()
+    rng = np.random.default_rng(n)
+    T = 60
+    plain = np.exp(2.0 * rng.standard_normal((rows, stride))).astype(np.float32)
+    tied = (rng.integers(0, 9, size=(rows, stride)) / 4.0).astype(np.float32)
+    tied[0, ::5] = -1.0  # ranks as 0
+    g_plain, g_tied = torch.as_tensor(plain, device="cuda"), torch.as_tensor(tied, device="cuda")
+    check = sorted({0, rows // 2, rows - 1})
+    for B in [1, n // 9, n - 1, n]:
+        for vals, g in ((plain, g_plain), (tied, g_tied)):
+            mask = diagnostics.topb_mask(g, n, B).cpu().numpy()
+            for r in check:
+                want = np.zeros(stride, np.uint8)
+                want[oracle.top_b(np.maximum(vals[r, :n], 0).astype(np.float64), B)] = 1
+                assert np.array_equal(mask[r], want), f"row {r} B {B}"
+    budgets = [max(1, n // 9), n]
+    c = diagnostics.concentration(g_plain, n, budgets)
+    m = diagnostics.state_metrics(g_plain, g_plain.flip(1).contiguous(), n - T, T, n // 9)
+    for r in check:
+        np.testing.assert_allclose(
+            c[r], oracle.concentration(plain[r, :n].astype(np.float64), budgets), rtol=1e-12)
+        want = oracle.state_metrics(plain[r, :n - T].astype(np.float64),
+                                    plain[r, ::-1][:n].astype(np.float64), n // 9)
+        for key in want:
+            assert m[key][r] == pytest.approx(want[key], rel=1e-12), (key, r)
