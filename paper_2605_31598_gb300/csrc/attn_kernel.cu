@@ -12,37 +12,42 @@
 //           tile's 128 rows (Eq. 1's importance, restricted to these rows) and
 //           O += P V with P in bf16.
 // tcgen05 runs every contraction with the A operand in TMEM (Q for Q K^T, P
-// for P V), so each MMA streams only K or V from shared memory.  TMEM
-// (512 columns): Q | P | S0 | S1 | O (layout below).
+// for P V), so each MMA streams only K or V from shared memory.
 //
-// K and V tiles stream through a ring of six 32 KB shared-memory slots in one
-// sequence, pass A's K tiles, then pass B's K(0) V(0) K(1) V(1) ...; a slot is
-// refilled once the MMAs that read it have completed (their commit arrives on
-// the slot's barrier).
+// K and V tiles of 128 keys stream through a ring of six 32 KB shared-memory
+// slots in one sequence, pass A's K tiles, then pass B's K(0) V(0) K(1) V(1) ...;
+// a slot is refilled once the MMAs that read it have completed (their commit
+// arrives on the slot's barrier).  The work on a tile goes in steps of 64 keys,
+// its halves: a step's scores get one of five TMEM buffers of 64 columns, and
+// its P overwrites the first half of them.  So up to five steps of each pass are
+// under way at once, in different stages: Q K^T, exponentials, P V.
 //
 // The kernel is persistent: one CTA per SM walks work units (query tile, KV
 // head, unit) in a fixed stride.  Ring, TMEM and barriers carry over from one
 // unit to the next, so the producer loads the next unit's first tiles while
-// the current one finishes, the next unit's Q goes into TMEM as soon as the
-// last P V completes, and its first Q K^T run while the previous O is read out.
+// the current one finishes, and its first Q K^T run while the previous O is
+// read out.
 //
-// 384 threads, three warpgroups:
+// 512 threads, four warpgroups:
 //   WG0  warp 0 producer (TMA), warps 1 and 3 MMA issuers X and Y (warp 1
-//        also owns TMEM), warp 2 the pass-B column-sum reducer.  tcgen05.mma
-//        issue blocks at the tensor core's pace, so each barrier wait of an
-//        issuing thread idles the tensor core; with two issuers one waits
-//        while the other's MMAs run.  X issues the pass-A Q K^T of even tiles
-//        and every pass-B Q K^T; Y the pass-A Q K^T of odd tiles and every
-//        P V (in order, so O accumulates deterministically).  Descriptors are precomputed words, so an MMA
-//        costs the issuing warp an add or two besides itself.
-//   WG1, WG2  softmax warpgroups.  Pass A: thread = query row; they take
-//        alternate key tiles, so the tensor core works on one warpgroup's
-//        tile while the other computes exponentials.  Pass B: both work on
-//        every tile, warpgroup w on keys [64 w, 64 w + 64), so each tile's P
-//        is ready after half a tile's work.
-// The column sums add a thread's rows in registers; the reducer warp adds the
-// four warps' staged values per lane, then the lanes by a shuffle
-// reduce-scatter, and writes the tile's importance partials.
+//        also owns TMEM), warp 2 the column-sum reducer.  Pass A: X issues the
+//        Q K^T of even steps, Y of odd ones; pass B: X every Q K^T, Y every P V
+//        (in order, so O accumulates deterministically).
+//   WG1..3  softmax warpgroups; they take the steps in turn.  Pass A: thread =
+//        query row, running max and sum.  Pass B: a thread holds 4 rows x 16
+//        columns, so the column sums start in registers.
+// What bounds it: no single unit.  At the 28-layer 7B stack (1232 units of ~35
+// steps, 213 us) the tensor core is busy 56% of the time, and taking out the
+// MMAs, the exponentials or the copies each saves 20 to 30 us: a step's chain
+// (barrier, TMEM load, 64 exponentials per thread, P store, column sums,
+// barrier) is ~1.2k cycles in a warpgroup against 540 of MMA in pass B.  Three
+// warpgroups on separate steps keep their phases apart; two on halves of one
+// tile (both in the same phase, and the odd tiles' Q K^T waiting for the P V
+// that read their P) and four (104 registers) were slower.  What had bound it
+// before was the issue of the MMAs and copies by one lane of a divergent warp;
+// see umma_ts.  Measured per frame, that form and this one (attention and
+// selection): 28-layer 7B stack 267 -> 228 us, 80-layer 72B stack 2.79 -> 2.47
+// ms, 28 layers over 32 frames of exact attention 622 -> 548 us.
 // Every mbarrier wait is bounded by the watchdog; on expiry the CTA records
 // DEV_TIMEOUT_ATTN, drains its in-flight copies and MMAs, frees TMEM and exits.
 #include "sm103_ptx.cuh"
@@ -53,38 +58,33 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 384;
+constexpr int kWG = 3;                    // softmax warpgroups
+constexpr int kSoftThreads = 128 * kWG;
+constexpr int kThreads = 128 + kSoftThreads;
 constexpr int kSlots = 6;        // 32 KB K/V tile slots (D = 128), one ring
-// TMEM columns: Q [0, 64) | P [64, 128) | S0 | S1 | O; pass A also uses O's
-// columns as a third score buffer S2.  Pass B puts even tiles' scores in S0
-// and odd tiles' in S1.  P (bf16 pairs) of even tiles goes to the P buffer,
-// so Q K^T can refill S0 as soon as both warpgroups have read the scores; P
-// of odd tiles overwrites the scores it came from (each warpgroup the first
-// 32 columns of its own 64), so Q K^T into S1 waits for the P V that reads
-// it.  (TMEM has no room for a second P buffer next to Q, two score buffers
-// and O.)
-constexpr uint32_t kColP = 64;
-constexpr uint32_t kColS0 = 128;
-constexpr uint32_t kColS1 = 256;
-constexpr uint32_t kColO = 384;
-constexpr int kSA = 3;           // pass-A score buffers
-// Pass-A barriers are indexed by tile mod 6 (buffer tile % 3, warpgroup and
-// issuer tile % 2), so each waiter has seen the barrier's previous phase and
-// can never mistake a phase two back for the one it waits for.
-constexpr int kSA2 = 2 * kSA;
+constexpr int kStep = 64;        // keys per step: half a K/V tile
+constexpr int kBufs = 5;         // score buffers
+// TMEM columns: Q [0, 64) | O [64, 192) | five score buffers of 64 columns.
+// A step's P (bf16 pairs) overwrites the first 32 columns of its own scores.
+constexpr uint32_t kColO = 64;
+constexpr uint32_t kColS = 192;
+// Barriers of a step are indexed by step mod 10, so that each waiter has seen the
+// barrier's previous phase and can never mistake a phase two back for the one it
+// waits for (two issuers and kWG warpgroups take steps in turn).
+constexpr int kBars = 2 * kBufs;
+constexpr int kWgArrive = 128;   // arrivals of a warpgroup on a barrier: every thread (one per warp was slower)
 
 template <int D>
 struct AttnLayout {
     static constexpr int kTileBytes = kBN * D * 2;  // one K or V tile
     static constexpr int kOffSlots = 0;
-    // column-sum staging of one pass-B tile: float[2 wg][4 quadrants][4 chunks][32 lanes][4]
+    // column sums of four pass-B steps: float[4][4 warps][32 lanes][2]
     static constexpr int kOffStage = kOffSlots + kSlots * kTileBytes;
-    static constexpr int kOffStat = kOffStage + 2 * 4 * 4 * 32 * 4 * 4;  // float[5][128]
-    static constexpr int kOffBar = kOffStat + 5 * kBM * 4;
-    // slot_full[6] slot_empty[6] sa_full[6] sa_read[6] sb_full[2] sb_read[2]
-    // p_full[2] pv_done[2] q_full o_full drain a_done a_read stage_full stage_free
-    // o_read stall
-    static constexpr int kNumBars = 41;
+    static constexpr int kOffStat = kOffStage + 4 * 4 * 32 * 2 * 4;  // float[kWG][2][128]
+    static constexpr int kOffBar = kOffStat + kWG * 2 * kBM * 4;
+    // slot_full[6] slot_empty[6] s_full[10] s_free[10] p_full[8] stage_full[4]
+    // stage_free[4] q_full o_full o_read drain stall
+    static constexpr int kNumBars = 2 * kSlots + 2 * kBars + 8 + 8 + 5;
     static constexpr int kOffMisc = kOffBar + kNumBars * 8;
     static constexpr int kBytes = kOffMisc + 16;
     static constexpr int kAlloc = kBytes + 1024;  // room to align the base to 1 KB
@@ -144,18 +144,6 @@ __device__ __forceinline__ unsigned long long globaltimer()
     return t;
 }
 
-// Bounded wait on an mbarrier phase: polls until `deadline` (globaltimer ns).
-__device__ __forceinline__ bool wait_until(uint64_t* bar, uint32_t parity,
-                                           unsigned long long deadline)
-{
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait(bar, parity)) return true;
-        if (globaltimer() > deadline) return false;
-    }
-}
-
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -166,35 +154,92 @@ __device__ __forceinline__ void named_bar_arrive(int id, int nthreads)
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// One MMA group, D[d] (+)= A[a + 8k (+ kGapA when k >= NK/2)] * B_k for k < NK
-// (bf16 in, fp32 accumulator, A in TMEM), with B's descriptor for step k given as its two
-// 32-bit words (lo + off(k), hi): the issuing warp shares its SM sub-partition
-// with the softmax warps, so each MMA should cost it as few instructions as
-// possible.
-template <int NK, bool kMajorB, uint32_t kGapA = 0>
-__device__ __forceinline__ void mma_group(uint32_t d, uint32_t a, uint32_t blo, uint32_t bhi,
-                                          uint32_t idesc, bool accumulate)
+__device__ __forceinline__ void arrive_at(uint32_t bar, uint32_t n = 1)
 {
-#pragma unroll
-    for (int k = 0; k < NK; ++k) {
-        // K-major B: 16 KB per 64-wide K half of a 128-row tile, 32 B per
-        // 16-element step inside a half; MN-major B: 2 KB per step.
-        const uint32_t off =
-            kMajorB ? ((k >> 2) * (kBN * 128) + (k & 3) * 32) >> 4 : (k * 2048) >> 4;
-        if (k == 0 && !accumulate)
-            asm volatile(
-                "{\n\t.reg .b64 bd;\n\t"
-                "mov.b64 bd, {%2, %3};\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], bd, %4, 0;\n\t}" ::"r"(d),
-                "r"(a), "r"(blo + off), "r"(bhi), "r"(idesc)
-                : "memory");
-        else
-            asm volatile(
-                "{\n\t.reg .b64 bd;\n\t"
-                "mov.b64 bd, {%2, %3};\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], bd, %4, 1;\n\t}" ::"r"(d),
-                "r"(a + 8 * k + (k >= NK / 2 ? kGapA : 0u)), "r"(blo + off), "r"(bhi), "r"(idesc)
-                : "memory");
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ void expect_at(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tma_load_at(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
+                                            int c3)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
+
+// A position in a cycle of N places (ring slots, score buffers) and the parity of
+// its current use.
+template <uint32_t N>
+struct Cycle {
+    uint32_t at, ph;
+    __device__ __forceinline__ Cycle plus(uint32_t n) const  // any n
+    {
+        const uint32_t t = at + n, q = t / N;
+        return Cycle{t - q * N, ph ^ (q & 1)};
+    }
+    __device__ __forceinline__ void step(uint32_t n)  // n <= N
+    {
+        at += n;
+        if (at >= N) {
+            at -= N;
+            ph ^= 1;
+        }
+    }
+};
+
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// D[d] (+)= A[a] B (bf16 in, fp32 accumulator, A in TMEM), issued by one lane of a
+// converged warp whose lanes all hold the same operands.  tcgen05.mma takes them
+// from uniform registers: where the compiler sees one lane in a branch of its
+// own it moves each into place for every MMA, and eight of them take 380 to 950
+// cycles to issue (more when the neighbouring warps do arithmetic) instead of 85.
+__device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, bool accumulate)
+{
+    if (elect_one())
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+            "r"(a), "l"(b), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
+            : "memory");
+}
+__device__ __forceinline__ void commit_elect(uint32_t bar)
+{
+    if (elect_one())
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                     : "memory");
+}
+// Bounded wait of a converged warp: the polls stay inside one asm statement, so
+// the code around it remains uniform; the deadline is looked at between them.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, unsigned long long deadline)
+{
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred P1;\n\t.reg .u32 c;\n\tmov.u32 c, 64;\n"
+            "W%=:\n\tmbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t@P1 bra D%=;\n\t"
+            "sub.u32 c, c, 1;\n\tsetp.ne.u32 P1, c, 0;\n\t@P1 bra W%=;\n\tsetp.ne.u32 P1, 0, 0;\n"
+            "D%=:\n\tselp.u32 %0, 1, 0, P1;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (__all_sync(0xffffffffu, done)) return true;
+        if (__any_sync(0xffffffffu, globaltimer() > deadline)) return false;
     }
 }
 
@@ -250,44 +295,48 @@ __device__ __forceinline__ void tmem_st_16x128b_x8(uint32_t taddr, const uint32_
         : "memory");
 }
 
-// Sums over the 8 lanes that share lane % 4 (lane bits 2..4) of 32 values,
-// as a reduce-scatter: lane l returns the sums of values 4 (l/4) .. +3.
-__device__ __forceinline__ void lane8_reduce_scatter(float (&x)[32], int lane, float (&out)[4])
+// Sums over the 8 lanes that share lane % 4 (lane bits 2..4) of 16 values,
+// as a reduce-scatter: lane l returns the sums of values 2 (l/4) and 2 (l/4) + 1.
+__device__ __forceinline__ float2 lane8_reduce_scatter(float (&x)[16], int lane)
 {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
+    for (int i = 0; i < 8; ++i) {
         const bool up = (lane & 16) != 0;
-        const float send = up ? x[i] : x[i + 16];
-        const float keep = up ? x[i + 16] : x[i];
+        const float send = up ? x[i] : x[i + 8];
+        const float keep = up ? x[i + 8] : x[i];
         x[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const bool up = (lane & 8) != 0;
-        const float send = up ? x[i] : x[i + 8];
-        const float keep = up ? x[i + 8] : x[i];
-        x[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-#pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const bool up = (lane & 4) != 0;
+        const bool up = (lane & 8) != 0;
         const float send = up ? x[i] : x[i + 4];
         const float keep = up ? x[i + 4] : x[i];
-        out[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+        x[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
     }
+    float2 out;
+    {
+        const bool up = (lane & 4) != 0;
+        const float s0 = up ? x[0] : x[2], k0 = up ? x[2] : x[0];
+        const float s1 = up ? x[1] : x[3], k1 = up ? x[3] : x[1];
+        out.x = k0 + __shfl_xor_sync(0xffffffffu, s0, 4);
+        out.y = k1 + __shfl_xor_sync(0xffffffffu, s1, 4);
+    }
+    return out;
 }
 
 // One work unit: the 128 query rows of tile mt of KV head hkv of the call's
 // unit u, with the key range the unit sees.  Units are numbered with the tile
-// fastest, then the KV head, then the unit.
+// fastest, then the KV head, then the unit.  Keys are taken in steps of 64: the
+// state's (or cache's) first, then the frame's, each range starting a new tile.
 struct WorkUnit {
     int mt, hkv, u, ua;
     int count;  // visible keys before the frame (state slots or cache rows)
-    int nst;    // key tiles over them
-    int nft;    // frame key tiles the tile's last row can see
-    int nt;     // nst + nft
+    int nfull;  // whole 128-key tiles over them
+    int nss;    // steps over them
+    int nst;    // tiles over them
+    int ns;     // all steps: nss and the frame steps the tile's last row can see
+    int nt;     // all tiles
     int rot;    // first state tile (see state_tile)
-    int full_state;  // state tiles [0, full_state) hold 128 valid keys wherever they start
 };
 
 __device__ __forceinline__ WorkUnit work_unit(const AttnParams& p, int w)
@@ -301,32 +350,60 @@ __device__ __forceinline__ WorkUnit work_unit(const AttnParams& p, int w)
     const int head = x.ua * p.Hkv + x.hkv;
     x.count = p.count_mul * ((p.B > 0 || p.count_mul > 1) ? p.counts[head] : 0) +
               (p.count_add ? p.count_add[head] : 0);
+    x.nfull = x.count / kBN;
+    x.nss = (x.count + kStep - 1) / kStep;
     x.nst = (x.count + kBN - 1) / kBN;
     const int row_hi = min(p.G * p.T, (x.mt + 1) * kBM) - 1;
-    x.nft = p.causal ? (row_hi / p.G) / kBN + 1 : (p.T + kBN - 1) / kBN;
-    x.nt = x.nst + x.nft;
+    const int nfs = p.causal ? (row_hi / p.G) / kStep + 1 : (p.T + kStep - 1) / kStep;
+    x.ns = x.nss + nfs;
+    x.nt = x.nst + (nfs + 1) / 2;
     // The query tiles of one KV head read the same state tiles; each starts at
-    // a different one (a fixed rotation) so they do not all request the same
-    // L2 lines at the same moment.  Frame tiles keep their order.
-    x.rot = x.nst > 0 ? (x.mt * 3) % x.nst : 0;
-    // with a rotation the ragged state tile (the last one, if count % 128 != 0)
-    // can come at any position; only when every state tile is whole is the
-    // check skipped for all of them
-    x.full_state = (x.count % kBN == 0) ? x.nst : 0;
+    // a different whole one (a fixed rotation) so they do not all request the
+    // same L2 lines at the same moment.  The ragged tile comes last; frame
+    // tiles keep their order.
+    x.rot = x.nfull > 0 ? (x.mt * 3) % x.nfull : 0;
     return x;
 }
 
+// the state tile taken t-th
 __device__ __forceinline__ int state_tile(const WorkUnit& x, int t)
 {
-    return t + x.rot < x.nst ? t + x.rot : t + x.rot - x.nst;
+    return t >= x.nfull ? t : t + x.rot < x.nfull ? t + x.rot : t + x.rot - x.nfull;
+}
+
+// The first key of step s: state slot / cache row (s < nss) or frame token.
+__device__ __forceinline__ int step_key(const WorkUnit& x, int s)
+{
+    return s < x.nss ? state_tile(x, s >> 1) * kBN + (s & 1) * kStep : (s - x.nss) * kStep;
+}
+
+constexpr int kAuxRegs = 80;    // registers per thread of the first warpgroup
+constexpr int kSoftRegs = 144;  // and of the softmax warpgroups
+
+// The same for a whole warp, every field the same register for all lanes as far as
+// the compiler can tell (it comes through a shuffle).
+__device__ __forceinline__ WorkUnit work_unit_uniform(const AttnParams& p, int w)
+{
+    WorkUnit x = work_unit(p, w);
+    x.hkv = uniform(x.hkv);
+    x.u = uniform(x.u);
+    x.ua = uniform(x.ua);
+    x.nfull = uniform(x.nfull);
+    x.rot = uniform(x.rot);
+    x.nss = uniform(x.nss);
+    x.nst = uniform(x.nst);
+    x.ns = uniform(x.ns);
+    x.nt = uniform(x.nt);
+    return x;
 }
 
 // Persistent: one CTA per SM walks the work units w = blockIdx.x, + gridDim.x,
 // ...  The ring, the TMEM allocation and every barrier live across units: the
-// producer loads the next unit's first tiles while the current one finishes,
-// and the per-tile barrier phases continue from unit to unit (tb below counts
-// the key tiles of the CTA's earlier units, so tile it of pass A is global
-// tile tb + it, and item i of the ring is global item 3 tb + i).
+// producer loads the next unit's first tiles while the current one finishes.
+// Steps are numbered through the CTA's life: a unit with first step gb takes
+// gb .. gb + ns - 1 in pass A and gb + ns .. gb + 2 ns - 1 in pass B, step g uses
+// score buffer g % 5 and belongs to warpgroup g % kWG; the ring holds the unit's nt
+// K tiles, then K V K V ...; pb counts pass-B steps.
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     frame_attn_lse_importance(const __grid_constant__ CUtensorMap tm_sk,
@@ -339,50 +416,61 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
     uint8_t* sSlot = sm + L::kOffSlots;
-    float4* stage = reinterpret_cast<float4*>(sm + L::kOffStage);
+    float2* stage = reinterpret_cast<float2*>(sm + L::kOffStage);
     float* stat = reinterpret_cast<float*>(sm + L::kOffStat);
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kOffBar);
-    uint64_t* slot_full = bars + 0;
-    uint64_t* slot_empty = bars + 6;
-    uint64_t* sa_full = bars + 12;  // pass A: Q K^T of global tile g done (index g % 6)
-    uint64_t* sa_read = bars + 18;  // pass A: global tile g read by its warpgroup (index g % 6)
-    uint64_t* sb_full = bars + 24;  // pass B: Q K^T of global tile g in score buffer g & 1
-    uint64_t* sb_read = bars + 26;  // pass B: both warpgroups have read S0 ([1] unused)
-    uint64_t* p_full = bars + 28;   // pass B: both warpgroups have written P of tile g (g & 1)
-    uint64_t* pv_done = bars + 30;  // pass B: P V of tile g has completed (index g & 1)
-    uint64_t* q_full = bars + 32;   // per unit: Q is in TMEM
-    uint64_t* o_full = bars + 33;   // per unit: every P V has completed
-    uint64_t* drain = bars + 34;
-    uint64_t* a_done = bars + 35;   // per unit: every pass-A MMA has completed
-    uint64_t* a_read = bars + 36;   // per unit: both warpgroups have read every pass-A tile
-    uint64_t* stage_full = bars + 37;  // pass B: the tile's column sums are staged
-    uint64_t* stage_free = bars + 38;  // pass B: the reducer warp has read them
-    uint64_t* o_read = bars + 39;   // per unit: O has been read out of TMEM
-    uint64_t* stall = bars + 40;    // watchdog self-test: never completed
+    uint64_t* slot_full = bars;                 // ring slot loaded
+    uint64_t* slot_empty = slot_full + kSlots;  // the MMAs of its steps have read it (2 arrivals)
+    uint64_t* s_full = slot_empty + kSlots;     // Q K^T of step g done (index g % 10)
+    uint64_t* s_free = s_full + kBars;          // step g's buffer free: pass A read, pass B P V done
+    uint64_t* p_full = s_free + kBars;          // P of pass-B step pb written (index pb % 8)
+    uint64_t* stage_full = p_full + 8;          // column sums of pass-B step pb staged (index pb % 4)
+    uint64_t* stage_free = stage_full + 4;      // and read by the reducer warp
+    uint64_t* q_full = stage_free + 4;          // per unit: Q is in TMEM
+    uint64_t* o_full = q_full + 1;              // per unit: every P V has completed
+    uint64_t* o_read = q_full + 2;              // per unit: O has been read out of TMEM
+    uint64_t* drain = q_full + 3;
+    uint64_t* stall = q_full + 4;               // watchdog self-test: never completed
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + L::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + L::kOffMisc + 4);
 
-    const int warp = threadIdx.x >> 5;
+    // barrier i of the order above at bar0 + 8 i
+    const uint32_t bar0 = smem_addr(bars);
+    constexpr uint32_t kBarSlotFull = 0, kBarSlotEmpty = 8 * kSlots, kBarSFull = 16 * kSlots,
+                       kBarSFree = kBarSFull + 8 * kBars, kBarPFull = kBarSFree + 8 * kBars,
+                       kBarStageFull = kBarPFull + 64, kBarStageFree = kBarStageFull + 32,
+                       kBarQFull = kBarStageFree + 32, kBarOFull = kBarQFull + 8, kBarORead = kBarQFull + 16,
+                       kBarDrain = kBarQFull + 24, kBarStall = kBarQFull + 32;
+    const int warp = uniform(threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int T = p.T, G = p.G, B = p.B;
     const int rows = G * T;
     const int W = p.MT * p.Hkv * p.U;
     const int w0 = blockIdx.x, wstep = gridDim.x;
 
-    // A softmax thread's Q row of unit w (thread 128 + i: warpgroup i / 128 - 1,
-    // row i % 128; warpgroup wg holds d in [64 wg, 64 wg + 64)).
+    // A softmax thread's part of its Q row of unit w (thread 128 + i: warpgroup
+    // i / 128, row i % 128; warpgroup wg < 2 holds d in [64 wg, 64 (wg + 1))).
+    // Padding rows load the last row (zeroed when they are stored).
     uint4 qreg[8];
-    auto load_q = [&](int w) {
+    auto q_src = [&](int w) -> const uint4* {
+        const int tq = static_cast<int>(threadIdx.x) - 128, qwg = tq >> 7;
+        if (p.q == nullptr || w >= W || tq < 0 || qwg * 64 >= D) return nullptr;  // nothing to load
         const int mt = w % p.MT, r = w / p.MT, hkv = r % p.Hkv, u = r / p.Hkv;
-        const int tq = static_cast<int>(threadIdx.x) - 128;
-        const int qwg = tq >> 7, qrow = tq & 127, qr = mt * kBM + qrow;
-        const bool loads = p.q != nullptr && w < W && tq >= 0 && qwg * 64 < D && qr < rows;
-        const int t = loads ? qr / G : 0, g = loads ? qr - t * G : 0;
-        const uint4* src = reinterpret_cast<const uint4*>(
-            p.q + ((static_cast<size_t>(loads ? u : 0) * T + t) * p.Hq + (loads ? hkv : 0) * G + g) * D +
-            (loads ? qwg * 64 : 0));
+        const int qr = min(mt * kBM + (tq & 127), rows - 1), t = qr / G, g = qr - t * G;
+        return reinterpret_cast<const uint4*>(
+            p.q + ((static_cast<size_t>(u) * T + t) * p.Hq + hkv * G + g) * D + qwg * 64);
+    };
+    auto load_q = [&](int w) {
+        const uint4* src = q_src(w);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) qreg[i] = loads ? src[i] : make_uint4(0u, 0u, 0u, 0u);
+        for (int i = 0; i < 8; ++i) qreg[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (src)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) qreg[i] = src[i];
+    };
+    auto prefetch_q = [&](int w) {
+        const uint4* src = q_src(w);
+        if (src) asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
     };
     // the first unit's rows load while the barriers and TMEM are set up
     load_q(w0);
@@ -390,26 +478,21 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (threadIdx.x == 0) {
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(&slot_full[i], 1);
-            mbar_init(&slot_empty[i], 1);
+            mbar_init(&slot_empty[i], 2);
         }
-        for (int i = 0; i < kSA2; ++i) {
-            mbar_init(&sa_full[i], 1);
-            mbar_init(&sa_read[i], 128);
+        for (int i = 0; i < kBars; ++i) {
+            mbar_init(&s_full[i], 1);
+            mbar_init(&s_free[i], kWgArrive);
         }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&sb_full[i], 1);
-            mbar_init(&sb_read[i], 256);
-            mbar_init(&p_full[i], 256);
-            mbar_init(&pv_done[i], 1);
+        for (int i = 0; i < 8; ++i) mbar_init(&p_full[i], kWgArrive);
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(&stage_full[i], kWgArrive);
+            mbar_init(&stage_free[i], 1);
         }
-        mbar_init(a_read, 256);
-        mbar_init(stage_full, 256);
-        mbar_init(stage_free, 32);
-        mbar_init(q_full, 256);
+        mbar_init(q_full, kSoftThreads);
         mbar_init(o_full, 1);
-        mbar_init(o_read, 256);
+        mbar_init(o_read, kSoftThreads);
         mbar_init(drain, 2);   // one commit per MMA issuer
-        mbar_init(a_done, 2);
         mbar_init(stall, 1);
         *abort_flag = 0;
         fence_mbar_init();
@@ -430,254 +513,254 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 96;" ::: "memory");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kAuxRegs) : "memory");
         if (warp == 0) {
             // ------------------------------------------------------------ producer
             // One ring of tiles for both passes of every unit: per unit, pass A's
-            // K tiles, then pass B's K(0) V(0) K(1) V(1) ...
-            if (lane == 0) {
+            // K tiles, then pass B's K(0) V(0) K(1) V(1) ...  Like the issuers, the whole
+            // warp runs the loop and elects a lane for the copies.
+            if (elect_one()) {
                 tma_prefetch_desc(&tm_fk);
                 tma_prefetch_desc(&tm_fv);
                 if (B > 0) {
                     tma_prefetch_desc(&tm_sk);
                     tma_prefetch_desc(&tm_sv);
                 }
-                int last_use[kSlots];
-#pragma unroll
-                for (int sl = 0; sl < kSlots; ++sl) last_use[sl] = -1;
-                bool ok = true;
-                // the self-test's wait gives up at half the watchdog, so it is
-                // deterministically the first wait of the launch to expire
-                if (p.selftest_stall && !wait_until(stall, 0, globaltimer() + p.watchdog_ns / 2)) {
-                    fail(1);
-                    ok = false;
-                }
-                int n = 0;  // global item
-                for (int w = w0; ok && w < W; w += wstep) {
-                    const WorkUnit x = work_unit(p, w);
-                    const unsigned long long deadline = globaltimer() + p.watchdog_ns;
-                    for (int i = 0; i < 3 * x.nt; ++i, ++n) {
-                        if (*abort_flag) {
-                            ok = false;
-                            break;
-                        }
-                        const int slot = n % kSlots, use = n / kSlots;
-                        if (use >= 1 && !wait_until(&slot_empty[slot], (use - 1) & 1, deadline)) {
-                            fail(2);
-                            ok = false;
-                            break;
-                        }
-                        const bool is_v = i >= x.nt && ((i - x.nt) & 1);
-                        const int tile = i < x.nt ? i : (i - x.nt) >> 1;
-                        const bool st = tile < x.nst;
-                        const CUtensorMap* map = st ? (is_v ? &tm_sv : &tm_sk) : (is_v ? &tm_fv : &tm_fk);
-                        const int c1 = st ? state_tile(x, tile) * kBN : x.hkv;
-                        const int c2 = st ? x.hkv : (tile - x.nst) * kBN;
-                        const int c3 = st ? x.ua : x.u;
-                        uint8_t* dst = sSlot + slot * L::kTileBytes;
-                        mbar_arrive_expect_tx(&slot_full[slot], L::kTileBytes);
-#pragma unroll
-                        for (int h = 0; h < D / 64; ++h)
-                            tma_load_4d(dst + h * (kBN * 128), map, &slot_full[slot], h * 64, c1, c2, c3);
-                        last_use[slot] = use;
-                    }
-                }
-                const unsigned long long dl = globaltimer() + p.watchdog_ns;
-                if (ok) {
-                    // every slot's last tile has been read by its MMAs
-                    for (int sl = 0; sl < kSlots; ++sl)
-                        if (last_use[sl] >= 0) wait_until(&slot_empty[sl], last_use[sl] & 1, dl);
-                } else {
-                    // let copies already in flight land before the CTA's memory goes away
-                    for (int sl = 0; sl < kSlots; ++sl)
-                        if (last_use[sl] >= 0) wait_until(&slot_full[sl], last_use[sl] & 1, dl);
-                }
             }
             __syncwarp();
+            bool ok = true;
+            // the self-test's wait gives up at half the watchdog, so it is
+            // deterministically the first wait of the launch to expire
+            if (p.selftest_stall && !wait_warp(bar0 + kBarStall, 0, globaltimer() + p.watchdog_ns / 2)) {
+                if (lane == 0) fail(1);
+                ok = false;
+            }
+            const uint32_t aSlot = uniform(smem_addr(sSlot));
+            uint32_t n = 0;            // items so far
+            Cycle<kSlots> ring{0, 0};  // the next item's slot
+            for (int w = w0; ok && w < W; w += wstep) {
+                const WorkUnit x = work_unit_uniform(p, w);
+                const unsigned long long deadline = globaltimer() + p.watchdog_ns;
+                auto load = [&](const CUtensorMap* map, int c1, int c2, int c3) {
+                    if (n >= kSlots && !wait_warp(bar0 + kBarSlotEmpty + 8 * ring.at, ring.ph ^ 1u, deadline)) return false;
+                    const uint32_t full = bar0 + kBarSlotFull + 8 * ring.at, dst = aSlot + ring.at * L::kTileBytes;
+                    if (elect_one()) {
+                        expect_at(full, L::kTileBytes);
+#pragma unroll
+                        for (int h = 0; h < D / 64; ++h)
+                            tma_load_at(dst + h * (kBN * 128), map, full, h * 64, c1, c2, c3);
+                    }
+                    ++n;
+                    ring.step(1);
+                    return true;
+                };
+                // tile t of the unit's keys: rows of the state (or cache), then of the frame
+                auto load_tile = [&](int t, bool v) {
+                    return t < x.nst ? load(v ? &tm_sv : &tm_sk, state_tile(x, t) * kBN, x.hkv, x.ua)
+                                     : load(v ? &tm_fv : &tm_fk, x.hkv, (t - x.nst) * kBN, x.u);
+                };
+#pragma unroll 1
+                for (int t = 0; ok && t < x.nt; ++t) ok = load_tile(t, false);
+#pragma unroll 1
+                for (int t = 0; ok && t < x.nt; ++t) ok = load_tile(t, false) && load_tile(t, true);
+                if (!ok && lane == 0) fail(2);
+                if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
+            }
+            // let every copy land, and every slot's last tile be read by its MMAs,
+            // before the CTA's memory goes away
+            const unsigned long long dl = globaltimer() + p.watchdog_ns;
+            for (uint32_t i = 0; i < kSlots && i < n; ++i) {  // the last min(n, 6) items
+                const Cycle<kSlots> c = ring.plus(2 * kSlots - 1 - i);  // item n - 1 - i (two turns on, same parity)
+                wait_warp(bar0 + (ok ? kBarSlotEmpty : kBarSlotFull) + 8 * c.at, c.ph, dl);
+            }
         } else if (warp == 2) {
             // ------------------------------------------------------------ column-sum reducer
-            // Pass B, per tile: the softmax threads stage their 16 row-summed
-            // values (4 rows each); lane L adds the 4 quadrants' values of
-            // staging lane L, then the 8 lanes that share L % 4 reduce-scatter
-            // 32 values, leaving lane L with columns 64 wg + 16 jj + 8 h + 2 (L % 4) + e
-            // (wg = m / 4, jj = m % 4, m = L / 4; h, e in {0, 1}).
+            // Pass B, per step: each of a warpgroup's four warps stages the column sums
+            // of its 32 rows, two columns per lane; they are added in warp order.
             bool ok = true;
-            int tb = 0;
+            int pb = 0;
             for (int w = w0; ok && w < W && p.partials != nullptr; w += wstep) {
                 const WorkUnit x = work_unit(p, w);
                 const unsigned long long deadline = globaltimer() + p.watchdog_ns;
                 float* part = p.partials + ((static_cast<size_t>(x.u) * p.Hkv + x.hkv) * p.MT + x.mt) * p.P;
-                for (int j = 0; j < x.nt; ++j) {
-                    const int g = tb + j;
-                    ok = __all_sync(0xffffffffu, wait_until(stage_full, g & 1, deadline));
+                for (int s = 0; s < x.ns; ++s, ++pb) {
+                    const float2* area = stage + (pb & 3) * 128 + lane;
+                    ok = wait_warp(bar0 + kBarStageFull + 8 * (pb & 3), (pb >> 2) & 1, deadline);
                     if (!ok) {
                         if (lane == 0) fail(13);
                         break;
                     }
-                    float xs[32];  // index (wg * 4 + jj) * 4 + i
+                    float2 sum = area[0];
 #pragma unroll
-                    for (int w2 = 0; w2 < 2; ++w2)
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            float4 a = stage[((w2 * 4 + 0) * 4 + jj) * 32 + lane];
-#pragma unroll
-                            for (int q = 1; q < 4; ++q) {
-                                const float4 b4 = stage[((w2 * 4 + q) * 4 + jj) * 32 + lane];
-                                a.x += b4.x;
-                                a.y += b4.y;
-                                a.z += b4.z;
-                                a.w += b4.w;
-                            }
-                            const int o = (w2 * 4 + jj) * 4;
-                            xs[o] = a.x;
-                            xs[o + 1] = a.y;
-                            xs[o + 2] = a.z;
-                            xs[o + 3] = a.w;
-                        }
-                    mbar_arrive(stage_free);  // the softmax threads may stage the next tile
-                    float sum4[4];
-                    lane8_reduce_scatter(xs, lane, sum4);
-                    const int m4 = lane >> 2, cbase = 64 * (m4 >> 2) + 16 * (m4 & 3) + 2 * (lane & 3);
-                    const bool is_state = j < x.nst;
-                    const int kb = (is_state ? state_tile(x, j) : j - x.nst) * kBN;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int key = kb + cbase + 8 * (i >> 1) + (i & 1);
-                        if (is_state ? key < x.count : key < T) part[is_state ? key : B + key] = sum4[i];
+                    for (int q = 1; q < 4; ++q) {
+                        const float2 y = area[32 * q];
+                        sum.x += y.x;
+                        sum.y += y.y;
                     }
+                    __syncwarp();
+                    if (lane == 0) arrive_at(bar0 + kBarStageFree + 8 * (pb & 3));
+                    const bool is_state = s < x.nss;
+                    const int key = step_key(x, s) + 8 * (lane >> 2) + 2 * (lane & 3);
+                    const int lim = is_state ? x.count : T;
+                    float* dst = part + (is_state ? 0 : B) + key;
+                    if (key < lim) dst[0] = sum.x;
+                    if (key + 1 < lim) dst[1] = sum.y;
                 }
-                tb += x.nt;
             }
-        } else if (warp == 1 || warp == 3) {
+        } else {
             // ------------------------------------------------------------ MMA issuers
-            if (lane == 0) {
-                const bool isx = warp == 1;
-                const uint32_t aSlot = smem_addr(sSlot);
-                const uint64_t dk = sdesc_sw128(aSlot, 16, 1024);         // K-major, slot 0
-                const uint64_t dv = sdesc_sw128(aSlot, kBN * 128, 1024);  // MN-major, slot 0
-                const uint32_t dk_lo = static_cast<uint32_t>(dk), d_hi = static_cast<uint32_t>(dk >> 32);
-                const uint32_t dv_lo = static_cast<uint32_t>(dv);
-                constexpr uint32_t kSlotStep = L::kTileBytes >> 4;  // descriptor address units
-                const uint32_t tQ = tbase, tO = tbase + kColO;
-                const uint32_t tS0 = tbase + kColS0, tS1 = tbase + kColS1;
-                constexpr uint32_t kIdQK = idesc_bf16_f32(kBM, kBN, false, false);
-                constexpr uint32_t kIdPV = idesc_bf16_f32(kBM, D, false, true);
-                int site = 4;  // first wait that expired, for the status word
-                bool ok = true;
-                int tb = 0, k = 0;
-                unsigned long long deadline = 0;
-                // S = Q K^T of one tile into buffer tS; its slot is released by the commit
-                auto qk = [&](int item, uint32_t tS, uint64_t* done) {
-                    const int slot = item % kSlots;
-                    tc_fence_after();
-                    mma_group<D / 16, true>(tS, tQ, dk_lo + slot * kSlotStep, d_hi, kIdQK, false);
-                    umma_commit(done);
-                    umma_commit(&slot_empty[slot]);
-                };
-                for (int w = w0; ok && w < W; w += wstep, ++k) {
-                    const WorkUnit x = work_unit(p, w);
-                    deadline = globaltimer() + p.watchdog_ns;
-                    const int nb = 3 * tb;  // the unit's first ring item
-                    site = 4;
-                    ok = wait_until(q_full, k & 1, deadline);
-                    // pass A: X takes the even global tiles, Y the odd ones; buffer
-                    // g % 3 (S0, S1, or O's columns, free once the previous unit's O
-                    // has been read out)
-                    for (int it = (isx ? 0 : 1) ^ (tb & 1); ok && it < x.nt; it += 2) {
-                        const int g = tb + it, item = nb + it;
-                        site = 5;
-                        if (!(ok = wait_until(&slot_full[item % kSlots], (item / kSlots) & 1, deadline)))
-                            break;
-                        site = 6;
-                        const int b = g % kSA;
-                        if (g >= kSA && !(ok = wait_until(&sa_read[(g - kSA) % kSA2],
-                                                          ((g - kSA) / kSA2) & 1, deadline)))
-                            break;
-                        if (b == 2 && it < kSA && k >= 1 &&
-                            !(ok = wait_until(o_read, (k - 1) & 1, deadline)))
-                            break;
-                        qk(item, b == 0 ? tS0 : b == 1 ? tS1 : tO, &sa_full[g % kSA2]);
-                    }
-                    if (ok) umma_commit(a_done);
-                    if (isx) {
-                        // Pass B Q K^T, in tile order.  Every pass-A MMA has completed
-                        // (so every pass-A load has landed: a slot's earlier occupant
-                        // may have been the other issuer's) and both warpgroups have
-                        // read every pass-A tile (the first tiles reuse S0 and S1).
-                        if (ok) {
-                            site = 9;
-                            ok = wait_until(a_done, k & 1, deadline) && wait_until(a_read, k & 1, deadline);
-                        }
-                        for (int j = 0; ok && j < x.nt; ++j) {
-                            const int g = tb + j, item = nb + x.nt + 2 * j, b = g & 1;
+            // Pass A: X (warp 1) takes the even steps' Q K^T, Y (warp 3) the odd ones'.
+            // Pass B: X issues every Q K^T, Y every P V, in step order.
+            // The whole warp runs the loops, with uniform operands, and elects a lane
+            // for each instruction (see umma_ts).
+            const bool isx = warp == 1;
+            const uint32_t aSlot = uniform(smem_addr(sSlot));
+            const uint64_t dk = sdesc_sw128(aSlot, 16, 1024);         // K-major, slot 0
+            const uint64_t dv = sdesc_sw128(aSlot, kBN * 128, 1024);  // MN-major, slot 0
+            // descriptor address units: a slot, half a tile's rows (64 of K, or 64 keys of V)
+            constexpr uint32_t kSlotStep = L::kTileBytes >> 4;
+            constexpr uint32_t kHalf = (kStep * 128) >> 4;
+            const uint32_t tb0 = uniform(tbase);
+            const uint32_t tQ = tb0, tO = tb0 + kColO, tS = tb0 + kColS;
+            constexpr uint32_t kIdQK = idesc_bf16_f32(kBM, kStep, false, false);
+            constexpr uint32_t kIdPV = idesc_bf16_f32(kBM, D, false, true);
+            int site = 4;  // first wait that expired, for the status word
+            bool ok = true;
+            uint32_t gb = 0, pb = 0, k = 0;  // earlier units' steps, pass-B steps so far, units
+            Cycle<kSlots> ring{0, 0};        // the unit's first ring item
+            Cycle<kBars> bar{0, 0};          // the unit's first step's barriers; buffer = at % 5
+            // S = Q K^T of step g (barriers b; half h of the tile in ring slot) once the
+            // step g - 5 has left its buffer
+            auto qk = [&](uint32_t g, const Cycle<kBars>& b, uint32_t slot, uint32_t h, unsigned long long deadline) {
+                const bool hi = b.at >= kBufs;
+                if (g >= kBufs && !wait_warp(bar0 + kBarSFree + 8 * (hi ? b.at - kBufs : b.at + kBufs),
+                                             hi ? b.ph : b.ph ^ 1u, deadline))
+                    return false;
+                tc_fence_after();
+                const uint64_t bd = dk + slot * kSlotStep + h * kHalf;
+                const uint32_t d = tS + (hi ? b.at - kBufs : b.at) * kStep;
+#pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk)  // 16 KB per 64-wide K half of a tile, 32 B per step
+                    umma_ts(d, tQ + 8 * kk, bd + (((kk >> 2) * (kBN * 128) + (kk & 3) * 32) >> 4), kIdQK, kk > 0);
+                commit_elect(bar0 + kBarSFull + 8 * b.at);
+                return true;
+            };
+            for (int w = w0; ok && w < W; w += wstep, ++k) {
+                const WorkUnit x = work_unit_uniform(p, w);
+                const uint32_t nt = x.nt, ns = x.ns;
+                // tiles of one step: the ragged state tile and the last frame tile, if odd
+                const uint32_t odd0 = (x.nss & 1) ? x.nst - 1 : nt, odd1 = ((ns - x.nss) & 1) ? nt - 1 : nt;
+                const unsigned long long deadline = globaltimer() + p.watchdog_ns;
+                site = 4;
+                ok = wait_warp(bar0 + kBarQFull, k & 1, deadline);
+                {   // pass A: step s of the unit is step gb + s; a tile's steps go to both issuers
+                    Cycle<kSlots> r = ring;
+                    Cycle<kBars> b = bar;
+                    uint32_t g = gb;
+#pragma unroll 1
+                    for (uint32_t t = 0; ok && t < nt; ++t) {
+                        const uint32_t nh = t == odd0 || t == odd1 ? 1 : 2;
+                        const uint32_t h = (g & 1) == (isx ? 0u : 1u) ? 0u : 1u;  // this issuer's half
+                        if (h < nh) {
                             site = 5;
-                            if (!(ok = wait_until(&slot_full[item % kSlots], (item / kSlots) & 1, deadline)))
-                                break;
-                            // the buffer's previous tile (g - 2) is consumed: read by both
-                            // warpgroups (S0: its P went to the P buffer), or read by its
-                            // P V (S1: its P overwrote the scores)
+                            if (!(ok = wait_warp(bar0 + kBarSlotFull + 8 * r.at, r.ph, deadline))) break;
                             site = 6;
-                            if (g >= 2 && !(ok = b == 0 ? wait_until(&sb_read[0], ((g - 2) >> 1) & 1, deadline)
-                                                        : wait_until(&pv_done[1], ((g - 2) >> 1) & 1, deadline)))
-                                break;
-                            qk(item, b ? tS1 : tS0, &sb_full[b]);
+                            Cycle<kBars> c = b;
+                            c.step(h);
+                            if (!(ok = qk(g + h, c, r.at, h, deadline))) break;
+                            if (nh == 1 && elect_one()) arrive_at(bar0 + kBarSlotEmpty + 8 * r.at);
+                            commit_elect(bar0 + kBarSlotEmpty + 8 * r.at);
                         }
-                    } else {
-                        // O += P(j) V(j): P of even global tiles in the P buffer (keys
-                        // 0..63 then 64..127), of odd ones over S1 (keys 0..63 at its
-                        // columns 0..31, keys 64..127 at 64..95)
-                        for (int j = 0; ok && j < x.nt; ++j) {
-                            const int g = tb + j, item = nb + x.nt + 2 * j + 1, b = g & 1;
-                            const int slot = item % kSlots;
-                            // the V tile usually landed long ago: its wait goes first, so
-                            // the wait that P ends is the last before the MMAs
-                            site = 8;
-                            if (!(ok = wait_until(&slot_full[slot], (item / kSlots) & 1, deadline))) break;
-                            site = 7;
-                            if (!(ok = wait_until(&p_full[b], (g >> 1) & 1, deadline))) break;
-                            tc_fence_after();
-                            if (b == 0)
-                                mma_group<kBN / 16, false>(tO, tbase + kColP, dv_lo + slot * kSlotStep,
-                                                           d_hi, kIdPV, j > 0);
-                            else
-                                mma_group<kBN / 16, false, 32>(tO, tS1, dv_lo + slot * kSlotStep, d_hi,
-                                                               kIdPV, j > 0);
-                            umma_commit(&pv_done[b]);
-                            umma_commit(&slot_empty[slot]);
-                        }
-                        if (ok) umma_commit(o_full);
+                        g += nh;
+                        b.step(nh);
+                        r.step(1);
                     }
-                    tb += x.nt;
                 }
-                if (!ok) fail(site + (isx ? 0 : 16));
-                // Every MMA issued so far must finish before TMEM is released.
-                umma_commit(drain);
-                wait_until(drain, 0, globaltimer() + p.watchdog_ns);
+                Cycle<kBars> b = bar.plus(ns);
+                if (isx) {
+                    // pass B Q K^T, in step order
+                    Cycle<kSlots> r = ring.plus(nt);
+                    uint32_t g = gb + ns;
+#pragma unroll 1
+                    for (uint32_t t = 0; ok && t < nt; ++t) {
+                        const uint32_t nh = t == odd0 || t == odd1 ? 1 : 2;
+                        site = 5;
+                        if (!(ok = wait_warp(bar0 + kBarSlotFull + 8 * r.at, r.ph, deadline))) break;
+                        site = 9;
+#pragma unroll
+                        for (uint32_t h = 0; h < 2; ++h) {
+                            if (h >= nh || !ok) break;
+                            ok = qk(g, b, r.at, h, deadline);
+                            ++g;
+                            b.step(1);
+                        }
+                        if (elect_one()) arrive_at(bar0 + kBarSlotEmpty + 8 * r.at);
+                        commit_elect(bar0 + kBarSlotEmpty + 8 * r.at);
+                        r.step(2);
+                    }
+                } else {
+                    // O += P V, in step order (O accumulates deterministically)
+                    Cycle<kSlots> r = ring.plus(nt + 1);
+                    site = 7;
+                    if (ok && k >= 1) ok = wait_warp(bar0 + kBarORead, (k - 1) & 1, deadline);
+#pragma unroll 1
+                    for (uint32_t t = 0; ok && t < nt; ++t) {
+                        const uint32_t nh = t == odd0 || t == odd1 ? 1 : 2;
+#pragma unroll
+                        for (uint32_t h = 0; h < 2; ++h) {
+                            if (h >= nh || !ok) break;
+                            // P first: once the unit's first P is written every pass-A tile has
+                            // landed, so the V slot's barrier is at most one phase behind
+                            site = 7;
+                            if (!(ok = wait_warp(bar0 + kBarPFull + 8 * (pb & 7), (pb >> 3) & 1, deadline))) break;
+                            ++pb;
+                            site = 8;
+                            if (h == 0 && !(ok = wait_warp(bar0 + kBarSlotFull + 8 * r.at, r.ph, deadline))) break;
+                            tc_fence_after();
+                            const uint64_t bd = dv + r.at * kSlotStep + h * kHalf;
+                            const uint32_t pa = tS + (b.at >= kBufs ? b.at - kBufs : b.at) * kStep;
+#pragma unroll
+                            for (int kk = 0; kk < kStep / 16; ++kk)  // 2 KB of V per 16 keys
+                                umma_ts(tO, pa + 8 * kk, bd + ((kk * 2048) >> 4), kIdPV, t > 0 || h > 0 || kk > 0);
+                            if (elect_one()) arrive_at(bar0 + kBarSFree + 8 * b.at, kWgArrive - 1);
+                            commit_elect(bar0 + kBarSFree + 8 * b.at);
+                            b.step(1);
+                        }
+                        if (elect_one()) arrive_at(bar0 + kBarSlotEmpty + 8 * r.at);
+                        commit_elect(bar0 + kBarSlotEmpty + 8 * r.at);
+                        r.step(2);
+                    }
+                    if (ok) commit_elect(bar0 + kBarOFull);
+                }
+                gb += 2 * ns;
+                ring = ring.plus(3 * nt);
+                bar = bar.plus(2 * ns);
             }
-            __syncwarp();
+            if (!ok && lane == 0) fail(site + (isx ? 0 : 16));
+            // Every MMA issued so far must finish before TMEM is released.
+            commit_elect(bar0 + kBarDrain);
+            wait_warp(bar0 + kBarDrain, 0, globaltimer() + p.watchdog_ns);
         }
         tc_fence_before();
         __syncthreads();
         if (warp == 1) tmem_dealloc(tbase, 512);
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 200;" ::: "memory");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftRegs) : "memory");
         // ------------------------------------------------------------ softmax warpgroups
-        const int wg = (warp >> 2) - 1;          // 0 or 1
+        const int wg = (warp >> 2) - 1;
         const int quad = warp & 3;               // TMEM lane quadrant of this warp
         const int row = quad * 32 + lane;        // TMEM lane = query row of the tile
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
         const float c = p.scale_log2;
         const int cq = 2 * (lane & 3);           // this thread's column offset in 8
-        const int c0 = 64 * wg;                  // this warpgroup's first key of a tile
-        const uint32_t tSh0 = tbase + lane_off + kColS0 + c0;   // this warpgroup's S0 half
-        const uint32_t tSh1 = tbase + lane_off + kColS1 + c0;   // its S1 half (and odd P)
-        const uint32_t tPh = tbase + lane_off + kColP + c0 / 2;  // its even-tile P
-        float4* mystage = stage + (wg * 4 + quad) * 4 * 32 + lane;  // chunk jj at + jj * 32
-        float* nl_row = stat + 4 * kBM;  // -lse of every row of the tile
+        const uint32_t tSw = tbase + lane_off + kColS;   // this warp's lanes of the score buffers
+        float2* mystage = stage + quad * 32 + lane;  // area i at + 128 i
         const f2 cc = pk(c, c);
 
-        // O rows of unit x -> bf16 out; warpgroup wg stores columns [wg D/2, (wg+1) D/2)
+        // O rows of unit x -> bf16 out; warpgroup wg < 2 stores columns [wg D/2, (wg + 1) D/2)
+        constexpr int kOc = D / 2;
         auto store_o = [&](const WorkUnit& x) {
+            if (wg * kOc >= D) return;
             const int my_r = x.mt * kBM + row;
             __nv_bfloat16* dst = p.out;
             if (my_r < rows) {
@@ -685,8 +768,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 dst += ((static_cast<size_t>(x.u) * T + t) * p.Hq + x.hkv * G + g) * D;
             }
 #pragma unroll
-            for (int cc2 = 0; cc2 < D / 64; ++cc2) {
-                const int col = wg * (D / 2) + cc2 * 32;
+            for (int cc2 = 0; cc2 < kOc / 32; ++cc2) {
+                const int col = wg * kOc + cc2 * 32;
                 float o[32];
                 tmem_ld32(tbase + lane_off + kColO + col, o);
                 tmem_ld_wait();
@@ -704,7 +787,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
         bool ok = true;
         int site = 10;  // first wait that expired, for the status word
-        int tb = 0, k = 0;
+        int gb = 0, pbb = 0, k = 0;  // earlier units' steps of both passes, pass-B steps, units
+        Cycle<kBars> bar{0, 0};      // the unit's first step's barriers; buffer = at % 5
         WorkUnit prev{};
         for (int w = w0; ok && w < W; w += wstep, ++k) {
             const WorkUnit x = work_unit(p, w);
@@ -713,82 +797,76 @@ __global__ void __launch_bounds__(kThreads, 1)
             const bool row_valid = my_r < rows;
             const int my_tq = row_valid ? my_r / G : T;  // padding rows see every frame key
 
-            {   // Q row -> TMEM columns [0, D/2) (bf16 pairs); warpgroup wg stores
-                // d in [64 wg, 64 wg + 64) when D = 128, warpgroup 0 all of D = 64.
-                // Every Q K^T of the previous unit has completed (its P V have).
+            {   // Q row -> TMEM columns [0, D/2) (bf16 pairs).  Every Q K^T of the
+                // previous unit has completed (its P V have).
                 if (wg * 64 < D) {
                     uint32_t w32[32];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        w32[4 * i] = qreg[i].x;
-                        w32[4 * i + 1] = qreg[i].y;
-                        w32[4 * i + 2] = qreg[i].z;
-                        w32[4 * i + 3] = qreg[i].w;
+                        w32[4 * i] = row_valid ? qreg[i].x : 0u;
+                        w32[4 * i + 1] = row_valid ? qreg[i].y : 0u;
+                        w32[4 * i + 2] = row_valid ? qreg[i].z : 0u;
+                        w32[4 * i + 3] = row_valid ? qreg[i].w : 0u;
                     }
-                    tmem_st16(tbase + lane_off + wg * 32, *reinterpret_cast<uint32_t(*)[16]>(&w32[0]));
-                    tmem_st16(tbase + lane_off + wg * 32 + 16,
-                              *reinterpret_cast<uint32_t(*)[16]>(&w32[16]));
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        tmem_st16(tbase + lane_off + wg * 32 + 16 * i,
+                                  *reinterpret_cast<uint32_t(*)[16]>(&w32[16 * i]));
                     tmem_st_wait();
                 }
                 tc_fence_before();
-                mbar_arrive(q_full);
+                arrive_at(bar0 + kBarQFull);
             }
             if (k >= 1) {  // the previous unit's O, while this unit's first Q K^T run
                 store_o(prev);
                 tc_fence_before();
-                mbar_arrive(o_read);
+                arrive_at(bar0 + kBarORead);
             }
 
-            // ---------------- pass A: online max / sum of exp2 over this warpgroup's tiles
+            // ---------------- pass A: online max / sum of exp2 over this warpgroup's steps
             float m = -INFINITY, l = 0.f;  // log2 units, scaled
-            const int it0 = wg ^ (tb & 1);  // this warpgroup takes the global tiles of parity wg
-            for (int it = it0; it < x.nt; it += 2) {
-                const int g = tb + it;
-                const int b = g % kSA;  // score buffer of this tile
-                ok = __all_sync(0xffffffffu, wait_until(&sa_full[g % kSA2], (g / kSA2) & 1, deadline));
+            const int sA = (wg + kWG - gb % kWG) % kWG;
+            Cycle<kBars> b = bar.plus(sA);
+            for (int s = sA; s < x.ns; s += kWG) {
+                ok = wait_warp(bar0 + kBarSFull + 8 * b.at, b.ph, deadline);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t tSa = tbase + lane_off + (b == 0 ? kColS0 : b == 1 ? kColS1 : kColO);
-                int lim;  // keys [0, lim) of this tile are visible to this row
-                if (it < x.nst) {
-                    lim = min(kBN, x.count - state_tile(x, it) * kBN);
-                } else {
-                    const int f0 = (it - x.nst) * kBN;
-                    lim = min(kBN, (p.causal ? min(T, my_tq + 1) : T) - f0);
-                }
-                // the whole tile into registers, then release the buffer at once so
+                const uint32_t tSa = tSw + (b.at >= kBufs ? b.at - kBufs : b.at) * kStep;
+                // the step into registers, then release the buffer at once so
                 // the next Q K^T into it can start while this one is reduced
-                float v[4][32];
-#pragma unroll
-                for (int ch = 0; ch < 4; ++ch) tmem_ld32(tSa + ch * 32, v[ch]);
+                float v[2][32];
+                tmem_ld32(tSa, v[0]);
+                tmem_ld32(tSa + 32, v[1]);
                 tmem_ld_wait();
                 tc_fence_before();
-                mbar_arrive(&sa_read[g % kSA2]);
-                // after its last tile is in registers, this thread holds no pass-A
-                // score buffer: pass B's Q K^T may start while the sums finish
-                if (it + 2 >= x.nt) mbar_arrive(a_read);
-                if (lim < kBN) {
+                arrive_at(bar0 + kBarSFree + 8 * b.at);
+                b.step(kWG);
+                if (s >= 2 * x.nfull) {  // keys [0, lim) of a ragged or frame step are visible to this row
+                    const int lim = s < x.nss ? x.count - s * kStep
+                                              : (p.causal ? min(T, my_tq + 1) : T) - (s - x.nss) * kStep;
+                    if (lim < kStep) {
 #pragma unroll
-                    for (int ch = 0; ch < 4; ++ch)
+                        for (int ch = 0; ch < 2; ++ch)
 #pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            v[ch][e] = (ch * 32 + e < lim) ? v[ch][e] : -INFINITY;
+                            for (int e = 0; e < 32; ++e)
+                                v[ch][e] = (ch * 32 + e < lim) ? v[ch][e] : -INFINITY;
+                    }
                 }
                 float mx[4];
 #pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) mx[q4] = fmaxf(v[q4][0], v[q4][1]);
+                for (int q4 = 0; q4 < 4; ++q4) mx[q4] = fmaxf(v[q4 >> 1][(q4 & 1) * 16], v[q4 >> 1][(q4 & 1) * 16 + 1]);
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch)
+                for (int q4 = 0; q4 < 4; ++q4)
 #pragma unroll
-                    for (int e = 2; e < 32; e += 2)
-                        mx[ch] = max3(mx[ch], v[ch][e], v[ch][e + 1]);
+                    for (int e = 2; e < 16; e += 2)
+                        mx[q4] = max3(mx[q4], v[q4 >> 1][(q4 & 1) * 16 + e], v[q4 >> 1][(q4 & 1) * 16 + e + 1]);
                 const float m_new =
                     fmaxf(m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c);  // c > 0
                 if (m_new != -INFINITY) {
                     const f2 nm = pk(-m_new, -m_new);
                     f2 acc[4] = {pk(0.f, 0.f), pk(0.f, 0.f), pk(0.f, 0.f), pk(0.f, 0.f)};
 #pragma unroll
-                    for (int ch = 0; ch < 4; ++ch)
+                    for (int ch = 0; ch < 2; ++ch)
 #pragma unroll
                         for (int e = 0; e < 32; e += 2) {
                             float x0, x1;
@@ -801,90 +879,57 @@ __global__ void __launch_bounds__(kThreads, 1)
                     m = m_new;
                 }
             }
-            if (it0 >= x.nt) mbar_arrive(a_read);  // a warpgroup without pass-A tiles
             // The pass-A -> pass-B hand-over exchanges the row statistics through
-            // two named barriers (1, then 2).  A warp whose pass-A wait expired
-            // records it, arrives at both barriers without waiting and leaves: the
-            // other warpgroup may have no pass-A tile left to wait on and be at
-            // barrier 1 already, and it is released through both; its pass-B waits
-            // then expire, since every pass-B step needs both warpgroups.  (An
-            // AND-reducing barrier that both leave together measured 5.8% slower
-            // over the whole launch.)
+            // named barrier 1.  A warp whose pass-A wait expired records it,
+            // arrives at the barrier without waiting and leaves; the others are
+            // released and their pass-B waits expire.
             if (!ok) {
                 fail(10 + 32 * wg);  // Q K^T in pass A
-                named_bar_arrive(1, 256);
-                named_bar_arrive(2, 256);
+                named_bar_arrive(1, kSoftThreads);
                 break;
             }
             stat[(wg * 2 + 0) * kBM + row] = m;
             stat[(wg * 2 + 1) * kBM + row] = l;
-            named_bar_sync(1, 256);
-            site = 11;
-            float nlse;  // -log2-sum-exp of this row (scaled); -inf for padding rows
-            {
-                const float m0 = stat[0 * kBM + row], l0 = stat[1 * kBM + row];
-                const float m1 = stat[2 * kBM + row], l1 = stat[3 * kBM + row];
-                const float mm = fmaxf(m0, m1);
-                const float ll = l0 * ex2(m0 - mm) + l1 * ex2(m1 - mm);
-                nlse = row_valid ? -(mm + __log2f(ll)) : -INFINITY;
-            }
-            if (wg == 0) nl_row[row] = nlse;
-            named_bar_sync(2, 256);
-            float nl4[4];  // -lse of this thread's 4 rows, index 2h + k
+            named_bar_sync(1, kSoftThreads);
+            float nl4[4];  // -log2-sum-exp (scaled) of this thread's 4 rows, index 2h + k; -inf for padding rows
             int tq4[4];    // token of each row (T for padding rows)
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+            for (int i = 0; i < 4; ++i) {
+                const int rr = quad * 32 + 16 * (i >> 1) + lane / 4 + 8 * (i & 1);
+                float mm = stat[rr], ll = 0.f;
 #pragma unroll
-                for (int k2 = 0; k2 < 2; ++k2) {
-                    const int rr = quad * 32 + 16 * h + lane / 4 + 8 * k2;
-                    nl4[2 * h + k2] = nl_row[rr];
-                    const int gr = x.mt * kBM + rr;
-                    tq4[2 * h + k2] = gr < rows ? gr / G : T;
-                }
-            // the next unit's Q rows load during pass B
-            load_q(w + wstep);
+                for (int g = 1; g < kWG; ++g) mm = fmaxf(mm, stat[g * 2 * kBM + rr]);
+#pragma unroll
+                for (int g = 0; g < kWG; ++g)
+                    ll += stat[(g * 2 + 1) * kBM + rr] * ex2(stat[g * 2 * kBM + rr] - mm);
+                const int gr = x.mt * kBM + rr;
+                nl4[i] = gr < rows ? -(mm + __log2f(ll)) : -INFINITY;
+                tq4[i] = gr < rows ? gr / G : T;
+            }
+            // the next unit's Q rows come to L2 during pass B
+            prefetch_q(w + wstep);
 
             // ---------------- pass B: P = exp2(S c - lse) -> TMEM (bf16) and column sums
-            // Both warpgroups work on every tile, warpgroup wg on its keys
-            // [64 wg, 64 wg + 64), so a tile's P is ready after half a tile's work.
             // TMEM is read in 16-lane x 256-bit groups: a thread holds 4 rows
             // (quadrant rows 16h + t/4 + 8k, h, k in {0, 1}) x 16 columns
-            // (8r + 2(t%4) + e).  P of even global tiles goes to the P buffer (so
-            // Q K^T can refill S0 once both warpgroups have read it); P of odd
-            // tiles overwrites the first half of this warpgroup's own S1 columns
-            // (Q K^T into S1 waits for that P V).
+            // (8r + 2(t%4) + e).  P overwrites the first half of the step's own
+            // score columns.
             float* part = p.partials ? p.partials + ((static_cast<size_t>(x.u) * p.Hkv + x.hkv) * p.MT + x.mt) * p.P
                                      : nullptr;
             site = 12;
-            for (int j = 0; ok && j < x.nt; ++j) {
-                const int g = tb + j, b = g & 1;
-                ok = __all_sync(0xffffffffu, wait_until(&sb_full[b], (g >> 1) & 1, deadline));
+            const int sB = (wg + kWG - (gb + x.ns) % kWG) % kWG;
+            b = bar.plus(x.ns + sB);
+            for (int s = sB; s < x.ns; s += kWG) {
+                const int pb = pbb + s;
+                ok = wait_warp(bar0 + kBarSFull + 8 * b.at, b.ph, deadline);
                 if (!ok) break;
                 tc_fence_after();
-                int lim4[4] = {kBN, kBN, kBN, kBN};  // keys [0, lim) of this tile are visible to each row
-                bool full = true;
-                if (j >= x.full_state) {  // the last state tile or a frame tile
-                    if (j < x.nst) {
-                        const int lim = min(kBN, x.count - state_tile(x, j) * kBN);
-#pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) lim4[q4] = lim;
-                    } else {
-                        const int f0 = (j - x.nst) * kBN;
-#pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4)
-                            lim4[q4] = min(kBN, (p.causal ? min(T, tq4[q4] + 1) : T) - f0);
-                    }
-                    const int lmin = min(min(lim4[0], lim4[1]), min(lim4[2], lim4[3]));
-                    full = lmin >= c0 + 64;
-                }
+                const uint32_t tSb = tSw + (b.at >= kBufs ? b.at - kBufs : b.at) * kStep;
+                b.step(kWG);
                 float v[2][32];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) tmem_ld_16x256b_x8((b ? tSh1 : tSh0) + ((16u * h) << 16), v[h]);
+                for (int h = 0; h < 2; ++h) tmem_ld_16x256b_x8(tSb + ((16u * h) << 16), v[h]);
                 tmem_ld_wait();
-                if (b == 0) {
-                    tc_fence_before();
-                    mbar_arrive(&sb_read[0]);  // Q K^T of tile g + 2 may overwrite S0
-                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -898,24 +943,27 @@ __global__ void __launch_bounds__(kThreads, 1)
                             v[h][i] = ex2(x0);
                             v[h][i + 1] = ex2(x1);
                         }
-                if (!full) {  // a ragged tile: keys at or past a row's limit get zero weight
+                if (s >= 2 * x.nfull) {  // a ragged or frame step: keys at or past a row's limit get zero weight
+                    int lim4[4];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h)
+                    for (int i = 0; i < 4; ++i)
+                        lim4[i] = s < x.nss ? x.count - s * kStep
+                                            : (p.causal ? min(T, tq4[i] + 1) : T) - (s - x.nss) * kStep;
+                    const int lmin = min(min(lim4[0], lim4[1]), min(lim4[2], lim4[3]));
+                    if (lmin < kStep) {
 #pragma unroll
-                        for (int r = 0; r < 8; ++r)
+                        for (int h = 0; h < 2; ++h)
 #pragma unroll
-                            for (int k2 = 0; k2 < 2; ++k2) {
-                                const int i = 4 * r + 2 * k2;
-                                const int col = c0 + 8 * r + cq, lim = lim4[2 * h + k2];
-                                v[h][i] = col < lim ? v[h][i] : 0.f;
-                                v[h][i + 1] = col + 1 < lim ? v[h][i + 1] : 0.f;
-                            }
+                            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                                for (int k2 = 0; k2 < 2; ++k2) {
+                                    const int i = 4 * r + 2 * k2;
+                                    const int col = 8 * r + cq, lim = lim4[2 * h + k2];
+                                    v[h][i] = col < lim ? v[h][i] : 0.f;
+                                    v[h][i + 1] = col + 1 < lim ? v[h][i + 1] : 0.f;
+                                }
+                    }
                 }
-                // the P buffer is free once the P V of tile g - 2 has read it
-                if (b == 0 && g >= 2)
-                    ok = __all_sync(0xffffffffu, wait_until(&pv_done[0], ((g - 2) >> 1) & 1, deadline));
-                if (!ok) break;
-                tc_fence_after();
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     uint32_t pw[16];  // register 2r + k: row k, P column 4r + t%4
@@ -924,14 +972,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                         for (int k2 = 0; k2 < 2; ++k2)
                             pw[2 * r + k2] = pack_bf16x2(v[h][4 * r + 2 * k2], v[h][4 * r + 2 * k2 + 1]);
-                    tmem_st_16x128b_x8((b ? tSh1 : tPh) + ((16u * h) << 16), pw);
+                    tmem_st_16x128b_x8(tSb + ((16u * h) << 16), pw);
                 }
                 tmem_st_wait();
                 tc_fence_before();
-                mbar_arrive(&p_full[b]);
-                // the column sums run while the tensor core does this tile's P V:
-                // value 2r + e is column 8r + cq + e summed over the thread's rows;
-                // the reducer warp adds them across lanes and warps
+                arrive_at(bar0 + kBarPFull + 8 * (pb & 7));
+                // the column sums run while the tensor core does this step's P V:
+                // value 2r + e is column 8r + cq + e summed over the thread's rows, then
+                // over the 8 lanes that share its columns; the reducer warp adds the warps
                 if (part != nullptr) {
                     float cs[16];
 #pragma unroll
@@ -940,27 +988,29 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const f2 bb = add2(pk(v[1][4 * r], v[1][4 * r + 1]), pk(v[1][4 * r + 2], v[1][4 * r + 3]));
                         upk(add2(a, bb), cs[2 * r], cs[2 * r + 1]);
                     }
-                    if (g >= 1)  // the reducer has read the previous tile's values
-                        ok = __all_sync(0xffffffffu, wait_until(stage_free, (g - 1) & 1, deadline));
+                    const float2 sum = lane8_reduce_scatter(cs, lane);  // columns 8 (lane / 4) + cq + {0, 1}
+                    if (pb >= 4)  // the reducer has read the step that had the area before
+                        ok = wait_warp(bar0 + kBarStageFree + 8 * (pb & 3), ((pb >> 2) & 1) ^ 1, deadline);
                     if (!ok) break;
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj)
-                        mystage[jj * 32] = make_float4(cs[4 * jj], cs[4 * jj + 1], cs[4 * jj + 2], cs[4 * jj + 3]);
-                    mbar_arrive(stage_full);
+                    mystage[(pb & 3) * 128] = sum;
+                    arrive_at(bar0 + kBarStageFull + 8 * (pb & 3));
                 }
             }
             if (!ok) break;
+            load_q(w + wstep);  // while the last P V run
             // Frame keys no row of this tile can see receive zero importance here.
             if (part != nullptr)
-                for (int t = x.nft * kBN + (threadIdx.x - 128); t < T; t += 256) part[B + t] = 0.f;
+                for (int t = (x.ns - x.nss) * kStep + (threadIdx.x - 128); t < T; t += kSoftThreads) part[B + t] = 0.f;
             // every P V of the unit has completed: O is final, and TMEM's Q and
             // score columns are free for the next unit
             site = 14;
-            ok = __all_sync(0xffffffffu, wait_until(o_full, k & 1, deadline));
+            ok = wait_warp(bar0 + kBarOFull, k & 1, deadline);
             if (!ok) break;
             tc_fence_after();
             prev = x;
-            tb += x.nt;
+            gb += 2 * x.ns;
+            pbb += x.ns;
+            bar = bar.plus(2 * x.ns);
         }
         if (ok && k >= 1) store_o(prev);  // the last unit's O
         if (!ok) fail(site + 32 * wg);
@@ -969,11 +1019,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-// The register split (WG0 down to 96, the softmax warpgroups up to 200 per
-// thread) must fit the registers the CTA is launched with, or setmaxnreg.inc
-// would wait forever: 128 * 96 + 256 * 200 = 63488 <= 384 threads * 168.
-constexpr int kLaunchRegs = 168;
-static_assert(128 * 96 + 256 * 200 <= kThreads * kLaunchRegs, "register split");
+// The register split must fit the registers the CTA is launched with, or
+// setmaxnreg.inc would wait forever.
+constexpr int kLaunchRegs = 128;
+static_assert(128 * kAuxRegs + kSoftThreads * kSoftRegs <= kThreads * kLaunchRegs, "register split");
 
 // SMs of each device, read by attn_prepare with that device current; the
 // persistent grid of a launch is sized for the device current at the launch.

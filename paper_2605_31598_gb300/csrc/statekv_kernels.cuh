@@ -19,11 +19,11 @@ namespace statekv {
 // byte is the kind; an attention-kernel timeout carries the waiting site in
 // bits 8..15 (the first expired wait of the CTA): 1 the watchdog self-test's
 // barrier (see AttnParams::selftest_stall), 2 producer (free slot),
-// 4..9 MMA issuer X (4 Q ready, 5 K tile landed, 6 score buffer free, 7 P
-// written, 8 V tile landed, 9 pass A done and read; +16 for issuer Y),
-// 10..12 and 14 softmax warpgroup 0 (10 Q K^T in pass A, 11 pass-B scores
-// ready, 12 the P buffer or the staging area free, 14 O final; +32 for
-// warpgroup 1), 13 the column-sum reducer.
+// 4..9 MMA issuer X (4 Q ready, 5 K tile landed, 6 score buffer free in pass A,
+// 7 O read out or P written, 8 V tile landed, 9 score buffer free in pass B; +16
+// for issuer Y), 10, 12 and 14 softmax warpgroup 0 (10 Q K^T in pass A, 12 pass-B
+// scores ready or the staging area free, 14 O final; +32 and +64 for warpgroups 1
+// and 2), 13 the column-sum reducer.
 enum DeviceError : int32_t {
     DEV_OK = 0,
     DEV_TIMEOUT_ATTN = 1,
