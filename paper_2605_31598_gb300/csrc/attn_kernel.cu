@@ -48,6 +48,15 @@
 // see umma_ts.  Measured per frame, that form and this one (attention and
 // selection): 28-layer 7B stack 267 -> 228 us, 80-layer 72B stack 2.79 -> 2.47
 // ms, 28 layers over 32 frames of exact attention 622 -> 548 us.
+//
+// Few units (one layer of a 7B model has 44 for 152 SMs): the split form.  A
+// thread-block cluster of S CTAs shares a unit, each CTA with a run of its key
+// tiles: pass A over them, then the CTAs exchange their rows' (max, sum) in
+// distributed shared memory, pass B over the same tiles (the importance columns
+// are its own), and last the S partial O are added in rank order, each CTA
+// finishing 1/S of the rows.  Per frame (attention and selection): one 7B layer (15
+// key tiles, S = 3) 35.2 -> 32.5 us, with a state of 16,384 (130 tiles) 184 ->
+// 111 us.
 // Every mbarrier wait is bounded by the watchdog; on expiry the CTA records
 // DEV_TIMEOUT_ATTN, drains its in-flight copies and MMAs, frees TMEM and exits.
 #include "sm103_ptx.cuh"
@@ -63,6 +72,8 @@ constexpr int kSoftThreads = 128 * kWG;
 constexpr int kThreads = 128 + kSoftThreads;
 constexpr int kSlots = 6;        // 32 KB K/V tile slots (D = 128), one ring
 constexpr int kStep = 64;        // keys per step: half a K/V tile
+constexpr int kMaxSplit = 8;     // CTAs that may share a unit (the portable cluster size)
+constexpr int kMinSplitTiles = 3;  // key tiles a CTA of a shared unit has at least
 constexpr int kBufs = 5;         // score buffers
 // TMEM columns: Q [0, 64) | O [64, 192) | five score buffers of 64 columns.
 // A step's P (bf16 pairs) overwrites the first 32 columns of its own scores.
@@ -81,7 +92,10 @@ struct AttnLayout {
     // column sums of four pass-B steps: float[4][4 warps][32 lanes][2]
     static constexpr int kOffStage = kOffSlots + kSlots * kTileBytes;
     static constexpr int kOffStat = kOffStage + 4 * 4 * 32 * 2 * 4;  // float[kWG][2][128]
-    static constexpr int kOffBar = kOffStat + kWG * 2 * kBM * 4;
+    static constexpr int kOffXStat = kOffStat + kWG * 2 * kBM * 4;  // split form: float2[8 ranks][128]
+    static constexpr int kOffBar = kOffXStat + kMaxSplit * kBM * 8;
+    static constexpr int kOStageLd = D + 4;  // split form: O staged over the ring, rows padded by a float4
+    static_assert(kBM * kOStageLd * 4 <= kSlots * kTileBytes, "O staging");
     // slot_full[6] slot_empty[6] s_full[10] s_free[10] p_full[8] stage_full[4]
     // stage_free[4] q_full o_full o_read drain stall
     static constexpr int kNumBars = 2 * kSlots + 2 * kBars + 8 + 8 + 5;
@@ -334,11 +348,14 @@ struct WorkUnit {
     int nfull;  // whole 128-key tiles over them
     int nss;    // steps over them
     int nst;    // tiles over them
-    int ns;     // all steps: nss and the frame steps the tile's last row can see
-    int nt;     // all tiles
+    int nfs;    // frame steps the tile's last row can see
+    int s0, t0; // this CTA's first step and tile (0 unless it shares the unit)
+    int ns;     // and how many of each it takes
+    int nt;
     int rot;    // first state tile (see state_tile)
 };
 
+template <bool kSplit>
 __device__ __forceinline__ WorkUnit work_unit(const AttnParams& p, int w)
 {
     WorkUnit x;
@@ -354,9 +371,19 @@ __device__ __forceinline__ WorkUnit work_unit(const AttnParams& p, int w)
     x.nss = (x.count + kStep - 1) / kStep;
     x.nst = (x.count + kBN - 1) / kBN;
     const int row_hi = min(p.G * p.T, (x.mt + 1) * kBM) - 1;
-    const int nfs = p.causal ? (row_hi / p.G) / kStep + 1 : (p.T + kStep - 1) / kStep;
-    x.ns = x.nss + nfs;
-    x.nt = x.nst + (nfs + 1) / 2;
+    x.nfs = p.causal ? (row_hi / p.G) / kStep + 1 : (p.T + kStep - 1) / kStep;
+    x.s0 = x.t0 = 0;
+    x.ns = x.nss + x.nfs;
+    x.nt = x.nst + (x.nfs + 1) / 2;
+    if (kSplit) {  // rank r of S takes tiles [nt r / S, nt (r + 1) / S)
+        const int r = static_cast<int>(cluster_ctarank()), nt = x.nt, ns = x.ns;
+        auto first_step = [&](int t) { return t >= nt ? ns : t <= x.nst ? min(2 * t, x.nss) : x.nss + 2 * (t - x.nst); };
+        const int t1 = nt * (r + 1) / p.split;
+        x.t0 = nt * r / p.split;
+        x.s0 = first_step(x.t0);
+        x.nt = t1 - x.t0;
+        x.ns = first_step(t1) - x.s0;
+    }
     // The query tiles of one KV head read the same state tiles; each starts at
     // a different whole one (a fixed rotation) so they do not all request the
     // same L2 lines at the same moment.  The ragged tile comes last; frame
@@ -382,9 +409,10 @@ constexpr int kSoftRegs = 144;  // and of the softmax warpgroups
 
 // The same for a whole warp, every field the same register for all lanes as far as
 // the compiler can tell (it comes through a shuffle).
+template <bool kSplit>
 __device__ __forceinline__ WorkUnit work_unit_uniform(const AttnParams& p, int w)
 {
-    WorkUnit x = work_unit(p, w);
+    WorkUnit x = work_unit<kSplit>(p, w);
     x.hkv = uniform(x.hkv);
     x.u = uniform(x.u);
     x.ua = uniform(x.ua);
@@ -392,6 +420,9 @@ __device__ __forceinline__ WorkUnit work_unit_uniform(const AttnParams& p, int w
     x.rot = uniform(x.rot);
     x.nss = uniform(x.nss);
     x.nst = uniform(x.nst);
+    x.nfs = uniform(x.nfs);
+    x.s0 = kSplit ? uniform(x.s0) : 0;
+    x.t0 = kSplit ? uniform(x.t0) : 0;
     x.ns = uniform(x.ns);
     x.nt = uniform(x.nt);
     return x;
@@ -404,7 +435,8 @@ __device__ __forceinline__ WorkUnit work_unit_uniform(const AttnParams& p, int w
 // gb .. gb + ns - 1 in pass A and gb + ns .. gb + 2 ns - 1 in pass B, step g uses
 // score buffer g % 5 and belongs to warpgroup g % kWG; the ring holds the unit's nt
 // K tiles, then K V K V ...; pb counts pass-B steps.
-template <int D>
+// The split form's CTA has one unit, blockIdx.x / S.
+template <int D, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
     frame_attn_lse_importance(const __grid_constant__ CUtensorMap tm_sk,
                               const __grid_constant__ CUtensorMap tm_sv,
@@ -418,6 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* sSlot = sm + L::kOffSlots;
     float2* stage = reinterpret_cast<float2*>(sm + L::kOffStage);
     float* stat = reinterpret_cast<float*>(sm + L::kOffStat);
+    float2* xstat = reinterpret_cast<float2*>(sm + L::kOffXStat);
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kOffBar);
     uint64_t* slot_full = bars;                 // ring slot loaded
     uint64_t* slot_empty = slot_full + kSlots;  // the MMAs of its steps have read it (2 arrivals)
@@ -446,7 +479,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int T = p.T, G = p.G, B = p.B;
     const int rows = G * T;
     const int W = p.MT * p.Hkv * p.U;
-    const int w0 = blockIdx.x, wstep = gridDim.x;
+    const int w0 = kSplit ? blockIdx.x / p.split : blockIdx.x, wstep = kSplit ? W : gridDim.x;
 
     // A softmax thread's part of its Q row of unit w (thread 128 + i: warpgroup
     // i / 128, row i % 128; warpgroup wg < 2 holds d in [64 wg, 64 (wg + 1))).
@@ -502,6 +535,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_relinquish();
     }
     __syncthreads();
+    // Split form: every thread of the cluster passes four phases of its barrier, on
+    // every path: 0 all CTAs run, 1 row statistics exchanged, 2 O staged, 3 O read.
+    if (kSplit) cluster_sync();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
 
@@ -514,6 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kAuxRegs) : "memory");
+        if (kSplit) cluster_arrive();  // phase 1: nothing of this warpgroup's to wait for
         if (warp == 0) {
             // ------------------------------------------------------------ producer
             // One ring of tiles for both passes of every unit: per unit, pass A's
@@ -539,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t n = 0;            // items so far
             Cycle<kSlots> ring{0, 0};  // the next item's slot
             for (int w = w0; ok && w < W; w += wstep) {
-                const WorkUnit x = work_unit_uniform(p, w);
+                const WorkUnit x = work_unit_uniform<kSplit>(p, w);
                 const unsigned long long deadline = globaltimer() + p.watchdog_ns;
                 auto load = [&](const CUtensorMap* map, int c1, int c2, int c3) {
                     if (n >= kSlots && !wait_warp(bar0 + kBarSlotEmpty + 8 * ring.at, ring.ph ^ 1u, deadline)) return false;
@@ -555,7 +592,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     return true;
                 };
                 // tile t of the unit's keys: rows of the state (or cache), then of the frame
-                auto load_tile = [&](int t, bool v) {
+                auto load_tile = [&](int tl, bool v) {
+                    const int t = tl + x.t0;
                     return t < x.nst ? load(v ? &tm_sv : &tm_sk, state_tile(x, t) * kBN, x.hkv, x.ua)
                                      : load(v ? &tm_fv : &tm_fk, x.hkv, (t - x.nst) * kBN, x.u);
                 };
@@ -580,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             int pb = 0;
             for (int w = w0; ok && w < W && p.partials != nullptr; w += wstep) {
-                const WorkUnit x = work_unit(p, w);
+                const WorkUnit x = work_unit<kSplit>(p, w);
                 const unsigned long long deadline = globaltimer() + p.watchdog_ns;
                 float* part = p.partials + ((static_cast<size_t>(x.u) * p.Hkv + x.hkv) * p.MT + x.mt) * p.P;
                 for (int s = 0; s < x.ns; ++s, ++pb) {
@@ -599,8 +637,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     __syncwarp();
                     if (lane == 0) arrive_at(bar0 + kBarStageFree + 8 * (pb & 3));
-                    const bool is_state = s < x.nss;
-                    const int key = step_key(x, s) + 8 * (lane >> 2) + 2 * (lane & 3);
+                    const int sg = s + x.s0;  // the unit's step
+                    const bool is_state = sg < x.nss;
+                    const int key = step_key(x, sg) + 8 * (lane >> 2) + 2 * (lane & 3);
                     const int lim = is_state ? x.count : T;
                     float* dst = part + (is_state ? 0 : B) + key;
                     if (key < lim) dst[0] = sum.x;
@@ -646,10 +685,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 return true;
             };
             for (int w = w0; ok && w < W; w += wstep, ++k) {
-                const WorkUnit x = work_unit_uniform(p, w);
+                const WorkUnit x = work_unit_uniform<kSplit>(p, w);
                 const uint32_t nt = x.nt, ns = x.ns;
                 // tiles of one step: the ragged state tile and the last frame tile, if odd
-                const uint32_t odd0 = (x.nss & 1) ? x.nst - 1 : nt, odd1 = ((ns - x.nss) & 1) ? nt - 1 : nt;
+                // (counted from this CTA's first; one that is not its own compares unequal)
+                const uint32_t odd0 = (x.nss & 1) ? x.nst - 1 - x.t0 : ~0u,
+                               odd1 = (x.nfs & 1) ? x.nst + x.nfs / 2 - x.t0 : ~0u;
                 const unsigned long long deadline = globaltimer() + p.watchdog_ns;
                 site = 4;
                 ok = wait_warp(bar0 + kBarQFull, k & 1, deadline);
@@ -741,6 +782,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             commit_elect(bar0 + kBarDrain);
             wait_warp(bar0 + kBarDrain, 0, globaltimer() + p.watchdog_ns);
         }
+        if (kSplit) {
+            __syncwarp();
+            cluster_wait();  // phase 1
+            cluster_sync();  // phase 2
+            cluster_sync();  // phase 3
+        }
         tc_fence_before();
         __syncthreads();
         if (warp == 1) tmem_dealloc(tbase, 512);
@@ -787,11 +834,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 
         bool ok = true;
         int site = 10;  // first wait that expired, for the status word
+        bool exchanged = false;  // split form: past phase 1
         int gb = 0, pbb = 0, k = 0;  // earlier units' steps of both passes, pass-B steps, units
         Cycle<kBars> bar{0, 0};      // the unit's first step's barriers; buffer = at % 5
         WorkUnit prev{};
         for (int w = w0; ok && w < W; w += wstep, ++k) {
-            const WorkUnit x = work_unit(p, w);
+            const WorkUnit x = work_unit<kSplit>(p, w);
             const unsigned long long deadline = globaltimer() + p.watchdog_ns;
             const int my_r = x.mt * kBM + row;
             const bool row_valid = my_r < rows;
@@ -841,9 +889,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tc_fence_before();
                 arrive_at(bar0 + kBarSFree + 8 * b.at);
                 b.step(kWG);
-                if (s >= 2 * x.nfull) {  // keys [0, lim) of a ragged or frame step are visible to this row
-                    const int lim = s < x.nss ? x.count - s * kStep
-                                              : (p.causal ? min(T, my_tq + 1) : T) - (s - x.nss) * kStep;
+                const int sg = s + x.s0;
+                if (sg >= 2 * x.nfull) {  // keys [0, lim) of a ragged or frame step are visible to this row
+                    const int lim = sg < x.nss ? x.count - sg * kStep
+                                               : (p.causal ? min(T, my_tq + 1) : T) - (sg - x.nss) * kStep;
                     if (lim < kStep) {
 #pragma unroll
                         for (int ch = 0; ch < 2; ++ch)
@@ -891,17 +940,41 @@ __global__ void __launch_bounds__(kThreads, 1)
             stat[(wg * 2 + 0) * kBM + row] = m;
             stat[(wg * 2 + 1) * kBM + row] = l;
             named_bar_sync(1, kSoftThreads);
+            if (kSplit) {
+                // this CTA's (max, sum) of every row to every CTA of the cluster
+                if (wg == 0) {
+                    float mm = stat[row], ll = 0.f;
+#pragma unroll
+                    for (int g = 1; g < kWG; ++g) mm = fmaxf(mm, stat[g * 2 * kBM + row]);
+                    if (mm != -INFINITY)
+#pragma unroll
+                        for (int g = 0; g < kWG; ++g)
+                            ll += stat[(g * 2 + 1) * kBM + row] * ex2(stat[g * 2 * kBM + row] - mm);
+                    const uint32_t a = smem_addr(xstat + cluster_ctarank() * kBM + row);
+                    for (int q = 0; q < p.split; ++q) st_dsmem_f2(dsmem_addr(a, q), mm, ll);
+                }
+                cluster_arrive();  // phase 1
+                cluster_wait();
+                exchanged = true;
+            }
             float nl4[4];  // -log2-sum-exp (scaled) of this thread's 4 rows, index 2h + k; -inf for padding rows
             int tq4[4];    // token of each row (T for padding rows)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int rr = quad * 32 + 16 * (i >> 1) + lane / 4 + 8 * (i & 1);
-                float mm = stat[rr], ll = 0.f;
+                float mm, ll = 0.f;
+                if (kSplit) {  // every CTA adds the ranks in the same order
+                    mm = xstat[rr].x;
+                    for (int q = 1; q < p.split; ++q) mm = fmaxf(mm, xstat[q * kBM + rr].x);
+                    for (int q = 0; q < p.split; ++q) ll += xstat[q * kBM + rr].y * ex2(xstat[q * kBM + rr].x - mm);
+                } else {
+                    mm = stat[rr];
 #pragma unroll
-                for (int g = 1; g < kWG; ++g) mm = fmaxf(mm, stat[g * 2 * kBM + rr]);
+                    for (int g = 1; g < kWG; ++g) mm = fmaxf(mm, stat[g * 2 * kBM + rr]);
 #pragma unroll
-                for (int g = 0; g < kWG; ++g)
-                    ll += stat[(g * 2 + 1) * kBM + rr] * ex2(stat[g * 2 * kBM + rr] - mm);
+                    for (int g = 0; g < kWG; ++g)
+                        ll += stat[(g * 2 + 1) * kBM + rr] * ex2(stat[g * 2 * kBM + rr] - mm);
+                }
                 const int gr = x.mt * kBM + rr;
                 nl4[i] = gr < rows ? -(mm + __log2f(ll)) : -INFINITY;
                 tq4[i] = gr < rows ? gr / G : T;
@@ -943,12 +1016,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                             v[h][i] = ex2(x0);
                             v[h][i + 1] = ex2(x1);
                         }
-                if (s >= 2 * x.nfull) {  // a ragged or frame step: keys at or past a row's limit get zero weight
+                const int sg = s + x.s0;
+                if (sg >= 2 * x.nfull) {  // a ragged or frame step: keys at or past a row's limit get zero weight
                     int lim4[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        lim4[i] = s < x.nss ? x.count - s * kStep
-                                            : (p.causal ? min(T, tq4[i] + 1) : T) - (s - x.nss) * kStep;
+                        lim4[i] = sg < x.nss ? x.count - sg * kStep
+                                             : (p.causal ? min(T, tq4[i] + 1) : T) - (sg - x.nss) * kStep;
                     const int lmin = min(min(lim4[0], lim4[1]), min(lim4[2], lim4[3]));
                     if (lmin < kStep) {
 #pragma unroll
@@ -999,8 +1073,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) break;
             load_q(w + wstep);  // while the last P V run
             // Frame keys no row of this tile can see receive zero importance here.
-            if (part != nullptr)
-                for (int t = (x.ns - x.nss) * kStep + (threadIdx.x - 128); t < T; t += kSoftThreads) part[B + t] = 0.f;
+            if (part != nullptr && (!kSplit || cluster_ctarank() == 0))
+                for (int t = x.nfs * kStep + (threadIdx.x - 128); t < T; t += kSoftThreads) part[B + t] = 0.f;
             // every P V of the unit has completed: O is final, and TMEM's Q and
             // score columns are free for the next unit
             site = 14;
@@ -1012,7 +1086,65 @@ __global__ void __launch_bounds__(kThreads, 1)
             pbb += x.ns;
             bar = bar.plus(2 * x.ns);
         }
-        if (ok && k >= 1) store_o(prev);  // the last unit's O
+        if (kSplit) {
+            __syncwarp();
+            if (!exchanged) {
+                cluster_arrive();  // phase 1
+                cluster_wait();
+            }
+            // this CTA's O (fp32; zero if it had no keys) over the idle ring, thread = row
+            float* ost = reinterpret_cast<float*>(sSlot);
+            if (ok && wg * kOc < D)
+#pragma unroll
+                for (int c2 = 0; c2 < kOc / 32; ++c2) {
+                    const int col = wg * kOc + c2 * 32;
+                    float o[32];
+                    if (prev.ns > 0) {
+                        tmem_ld32(tbase + lane_off + kColO + col, o);
+                        tmem_ld_wait();
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) o[e] = 0.f;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        *reinterpret_cast<float4*>(ost + row * L::kOStageLd + col + 4 * e) =
+                            make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+                }
+            __syncwarp();
+            cluster_sync();  // phase 2
+            if (ok) {
+                const int rank = static_cast<int>(cluster_ctarank());
+                const int r0 = kBM * rank / p.split, r1 = kBM * (rank + 1) / p.split;
+                const uint32_t a0 = smem_addr(ost);
+                for (int i = threadIdx.x - 128; i < (r1 - r0) * (D / 4); i += kSoftThreads) {
+                    const int rr = r0 + i / (D / 4), c4 = 4 * (i % (D / 4)), my_r = prev.mt * kBM + rr;
+                    const uint32_t a = a0 + static_cast<uint32_t>(rr * L::kOStageLd + c4) * 4u;
+                    float4 v[kMaxSplit];
+#pragma unroll
+                    for (int q = 0; q < kMaxSplit; ++q)
+                        if (q < p.split) v[q] = ld_dsmem_f4(dsmem_addr(a, q));
+#pragma unroll
+                    for (int q = 1; q < kMaxSplit; ++q)
+                        if (q < p.split) {
+                            v[0].x += v[q].x;
+                            v[0].y += v[q].y;
+                            v[0].z += v[q].z;
+                            v[0].w += v[q].w;
+                        }
+                    if (my_r < rows) {
+                        const int t = my_r / G, g = my_r - t * G;
+                        *reinterpret_cast<uint2*>(
+                            p.out + ((static_cast<size_t>(prev.u) * T + t) * p.Hq + prev.hkv * G + g) * D + c4) =
+                            make_uint2(pack_bf16x2(v[0].x, v[0].y), pack_bf16x2(v[0].z, v[0].w));
+                    }
+                }
+            }
+            __syncwarp();
+            cluster_sync();  // phase 3
+        } else if (ok && k >= 1) {
+            store_o(prev);  // the last unit's O
+        }
         if (!ok) fail(site + 32 * wg);
         tc_fence_before();
         __syncthreads();
@@ -1036,25 +1168,76 @@ int current_device_sms()
     return g_num_sms[dev] > 0 ? g_num_sms[dev] : 1;
 }
 
+// Clusters of each size that a device holds at once with the split form's shared
+// memory, measured by attn_prepare (0: not measured, or none).
+int g_attn_clusters[kMaxDevices][2][kMaxSplit + 1] = {};
+
+template <int D>
+cudaLaunchConfig_t split_config(int units, int S, cudaStream_t st, cudaLaunchAttribute* attr)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(units) * S);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = AttnLayout<D>::kAlloc;
+    cfg.stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = S;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+template <int D, bool kSplit>
+cudaError_t prepare_form()
+{
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, frame_attn_lse_importance<D, kSplit>);
+    if (e != cudaSuccess) return e;
+    if (fa.numRegs < kLaunchRegs) return cudaErrorInvalidConfiguration;
+    return cudaFuncSetAttribute(frame_attn_lse_importance<D, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                AttnLayout<D>::kAlloc);
+}
+
 template <int D>
 cudaError_t prepare_one()
 {
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, frame_attn_lse_importance<D>);
-    if (e != cudaSuccess) return e;
-    if (fa.numRegs < kLaunchRegs) return cudaErrorInvalidConfiguration;
     int dev = 0, sms = 0;
+    cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if ((e = prepare_form<D, false>()) != cudaSuccess || (e = prepare_form<D, true>()) != cudaSuccess) return e;
+    for (int S = 2; S <= kMaxSplit; ++S) {
+        cudaLaunchAttribute attr[1];
+        const cudaLaunchConfig_t cfg = split_config<D>(1, S, nullptr, attr);
+        int n = 0;
+        if ((e = cudaOccupancyMaxActiveClusters(&n, frame_attn_lse_importance<D, true>, &cfg)) != cudaSuccess)
+            return e;
+        g_attn_clusters[dev][D == 128][S] = n;
+    }
     g_num_sms[dev] = sms;
-    return cudaFuncSetAttribute(frame_attn_lse_importance<D>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                AttnLayout<D>::kAlloc);
+    return cudaSuccess;
 }
 
-// One CTA per SM (at most one per work unit); each walks its units in order.
+// CTAs per unit: as many as let every unit's cluster be resident at once (so the
+// split form runs where the units leave half of the SMs idle or more) and leave
+// every CTA kMinSplitTiles key tiles; the two exchanges cost about as much as two
+// tiles.  At 15 tiles and S = 3 (5 each) 32.5 us per frame against 36.1 whole.
+template <int D>
+int split_for(long long W, int tiles)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 1;
+    for (int S = kMaxSplit; S >= 2; --S)
+        if (W <= g_attn_clusters[dev][D == 128][S] && tiles >= kMinSplitTiles * S) return S;
+    return 1;
+}
+
+// One CTA per SM (at most one per work unit), each walking its units in order; or
+// a cluster per unit.
 template <int D>
 cudaError_t launch_one(const CUtensorMap& tm_sk, const CUtensorMap& tm_sv, const CUtensorMap& tm_fk,
                        const CUtensorMap& tm_fv, const AttnParams& p0, int U, cudaStream_t st)
@@ -1064,10 +1247,16 @@ cudaError_t launch_one(const CUtensorMap& tm_sk, const CUtensorMap& tm_sv, const
     const long long W = static_cast<long long>(p.MT) * p.Hkv * U;
     if (W <= 0) return cudaSuccess;
     if (W > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+    p.split = p.selftest_stall ? 1 : split_for<D>(W, (p.keys_hint + kBN - 1) / kBN + (p.T + kBN - 1) / kBN);
+    if (p.split > 1) {
+        cudaLaunchAttribute attr[1];
+        const cudaLaunchConfig_t cfg = split_config<D>(static_cast<int>(W), p.split, st, attr);
+        return cudaLaunchKernelEx(&cfg, frame_attn_lse_importance<D, true>, tm_sk, tm_sv, tm_fk, tm_fv, p);
+    }
     const int sms = current_device_sms();
     const int grid = static_cast<int>(W < sms ? W : sms);
-    frame_attn_lse_importance<D><<<grid, kThreads, AttnLayout<D>::kAlloc, st>>>(tm_sk, tm_sv, tm_fk,
-                                                                              tm_fv, p);
+    frame_attn_lse_importance<D, false><<<grid, kThreads, AttnLayout<D>::kAlloc, st>>>(tm_sk, tm_sv, tm_fk,
+                                                                                     tm_fv, p);
     return cudaSuccess;
 }
 

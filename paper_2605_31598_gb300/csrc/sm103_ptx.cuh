@@ -84,6 +84,9 @@ __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// its two halves
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // the address of shared-memory location `saddr` in the CTA of cluster rank `rank`
 __device__ __forceinline__ uint32_t dsmem_addr(uint32_t saddr, uint32_t rank)
 {
@@ -99,6 +102,11 @@ __device__ __forceinline__ float4 ld_dsmem_f4(uint32_t addr)
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
     return v;
+}
+
+__device__ __forceinline__ void st_dsmem_f2(uint32_t addr, float x, float y)
+{
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
 }
 
 // ---------------------------------------------------------------- L2 prefetch

@@ -244,6 +244,19 @@ statekv_status check_args(const statekv_handle* h, const statekv_frame_args* a, 
     return STATEKV_OK;
 }
 
+// The most frames any (stream, layer) of the range has seen, and decoded tokens.
+long long most_rows(const statekv_handle* h, int stream_begin, int stream_count, int layer_begin, int layer_count)
+{
+    long long rows = 0;
+    for (int s = stream_begin; s < stream_begin + stream_count; ++s)
+        for (int l = layer_begin; l < layer_begin + layer_count; ++l) {
+            const size_t unit = static_cast<size_t>(s) * h->cfg.num_layers + l;
+            rows = std::max(rows, static_cast<long long>(h->frames_host[unit]) * h->cfg.tokens_per_frame +
+                                      h->text_host[unit]);
+        }
+    return rows;
+}
+
 template <class F>
 cudaError_t timed(statekv_handle* h, int kind, cudaStream_t st, F&& launch)
 {
@@ -320,6 +333,8 @@ statekv_status run_step(statekv_handle* h, const statekv_frame_args& a, cudaStre
     pa.MT = d.MT;
     pa.causal = c.causal_in_frame;
     pa.count_mul = 1;
+    pa.keys_hint = static_cast<int>(std::min<long long>(
+        c.state_capacity, most_rows(h, a.stream_begin, a.stream_count, a.layer_begin, a.layer_count)));
     pa.scale_log2 = d.scale * 1.4426950408889634f;
     pa.watchdog_ns = 1000000ull * (c.watchdog_ms ? c.watchdog_ms : 2000u);
     const cudaError_t ek =
@@ -414,6 +429,7 @@ statekv_status run_full(statekv_handle* h, const statekv_frame_args& a, cudaStre
     pa.MT = d.MT;
     pa.causal = c.causal_in_frame;
     pa.count_mul = T;
+    pa.keys_hint = static_cast<int>(most_rows(h, a.stream_begin, a.stream_count, a.layer_begin, a.layer_count));
     pa.scale_log2 = d.scale * 1.4426950408889634f;
     pa.watchdog_ns = 1000000ull * (c.watchdog_ms ? c.watchdog_ms : 2000u);
     if (timed(h, 1, st, [&] { return launch_attn(D, h->tm_ck, h->tm_cv, tm_fk, tm_fv, pa, U, st); }) !=
@@ -453,13 +469,7 @@ statekv_status run_decode(statekv_handle* h, const statekv_decode_args& a, cudaS
         // A few rows: one launch of the one-pass split-K kernel, which puts the
         // new tokens' K/V into the cache, reads every key once from it and
         // advances the token counts.
-        long long maxlen = 0;
-        for (int s = a.stream_begin; s < a.stream_begin + a.stream_count; ++s)
-            for (int l = a.layer_begin; l < a.layer_begin + a.layer_count; ++l) {
-                const size_t unit = static_cast<size_t>(s) * c.num_layers + l;
-                maxlen = std::max(maxlen, static_cast<long long>(h->frames_host[unit]) * T +
-                                              h->text_host[unit] + n);
-            }
+        const long long maxlen = most_rows(h, a.stream_begin, a.stream_count, a.layer_begin, a.layer_count) + n;
         // chunk count: the one whose waves of CTAs (one per SM) take the least
         // time, counting each CTA's fixed cost as ~512 keys of streaming
         DecodeParams dp{};
@@ -535,6 +545,7 @@ statekv_status run_decode(statekv_handle* h, const statekv_decode_args& a, cudaS
     pa.MT = static_cast<int>((static_cast<long long>(d.G) * n + kBM - 1) / kBM);
     pa.causal = 1;
     pa.count_mul = T;
+    pa.keys_hint = static_cast<int>(most_rows(h, a.stream_begin, a.stream_count, a.layer_begin, a.layer_count));
     pa.scale_log2 = d.scale * 1.4426950408889634f;
     pa.watchdog_ns = 1000000ull * (c.watchdog_ms ? c.watchdog_ms : 2000u);
     if (timed(h, 1, st, [&] { return launch_attn(D, h->tm_ck, h->tm_cv, tm_nk, tm_nv, pa, U, st); }) !=

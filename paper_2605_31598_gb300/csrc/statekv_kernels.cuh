@@ -79,6 +79,9 @@ struct AttnParams {
     UnitRange units;
     int T, Hq, Hkv, G, B, P, MT;
     int U;                    // units of the call (set by launch_attn)
+    int split;                // CTAs that share a work unit's keys, a cluster (set by launch_attn)
+    int keys_hint;            // about how many keys before the frame the units have, at most (host
+                              //   counters): launch_attn splits long ones when there are few
     int causal;
     int count_mul;            // 1: counts are state sizes; T: counts are frame counters
     float scale_log2;         // softmax scale * log2(e)

@@ -13,7 +13,7 @@ import torch
 from paper_2605_31598_gb300 import StateKV, make_config
 from paper_2605_31598_gb300.inputs import WORKLOADS, Shape, batch_qkv
 
-from .parity import run_free_running, run_parity
+from .parity import IMP_ATOL, IMP_RTOL, OUT_ATOL, run_free_running, run_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -318,3 +318,44 @@ def test_streams_at_different_frames_in_one_launch():
         run([0, 1])
     assert done == [8, 5]
     assert eng.sync() == 0
+
+
+# few work units over many key tiles: the attention kernel's split form (a cluster
+# of CTAs per unit), from two CTAs to eight, with ragged last tiles
+SPLIT = {
+    "one_unit_d128": (Shape(2, 1, 128, 64, 1100, 22), 22),
+    "three_units_ragged_d64": (Shape(6, 3, 64, 37, 700, 24), 24),
+    "long_frame_b0_like": (Shape(1, 1, 128, 300, 2500, 10), 10),
+    "frame_tiles_only": (Shape(1, 1, 64, 900, 0, 2), 2),
+}
+
+
+@pytest.mark.parametrize("name", sorted(SPLIT))
+@pytest.mark.parametrize("causal", [True, False])
+def test_split_attention_parity(name, causal):
+    shape, frames = SPLIT[name]
+    run_parity(shape, frames, kind="peaked", causal=causal,
+               check_frames=[f for f in (1, 2, frames // 2, frames) if f <= frames])
+
+
+def test_split_attention_with_streams_at_different_frames():
+    """A stream that has seen 16 frames and one at its first share a call: the
+    CTAs per unit follow the longer one, so some of the other's CTAs hold no key
+    tile.  The short stream's outputs equal those of a call of its own."""
+    shape = Shape(4, 1, 128, 64, 1000, 20, num_streams=2, kind="peaked")
+    B, T = shape.state_capacity, shape.tokens_per_frame
+    both, own = StateKV(make_config(shape)), StateKV(make_config(shape))
+    for n in range(1, 17):
+        q, k, v = batch_qkv(shape, n, streams=[0], layers=[0], device="cuda")
+        assert both.prefill_frame(q, k, v, torch.empty_like(q), stream_begin=0, stream_count=1) == 0
+    q, k, v = batch_qkv(shape, [17, 1], streams=[0, 1], layers=[0], device="cuda")
+    out, imp = torch.full_like(q, float("nan")), torch.full((2, 1, 1, B + T), float("nan"), device="cuda")
+    assert both.prefill_frame(q, k, v, out, imp) == 0
+    out1, imp1 = torch.empty_like(q[1:]), torch.empty((1, 1, 1, B + T), device="cuda")
+    assert own.prefill_frame(q[1:].contiguous(), k[1:].contiguous(), v[1:].contiguous(), out1, imp1,
+                             stream_begin=1, stream_count=1) == 0
+    torch.cuda.synchronize()
+    assert both.sync() == 0 and own.sync() == 0
+    assert torch.isfinite(out).all() and torch.isfinite(imp).all()
+    assert (out[1:].float() - out1.float()).abs().max().item() <= OUT_ATOL
+    torch.testing.assert_close(imp[1:], imp1, rtol=IMP_RTOL, atol=IMP_ATOL)
