@@ -371,19 +371,19 @@ def run_ours(args, world, rank, local):
     s_launches, s_ms = prof[2]
     d = shape.head_dim
     append_bytes = 2 * 2 * S * L * Hkv * T * d * 2  # read + write K and V rows
-    # The append runs on a side stream next to the attention kernel (it takes
-    # the SMs the attention grid's last wave leaves idle), so its event span
-    # includes waiting for SMs and it is off the critical path; the shares are
+    # The append shares the selection's launch (with the recency window it is a
+    # launch of its own on a side stream, off the critical path); the shares are
     # of the two kernels in series.
     kernels = {
         "frame_attn_lse_importance": {"avg_us": 1e6 * k1_avg_s, "tflops": achieved,
                                       "share": k1_ms / max(1e-9, k1_ms + s_ms)},
-        "decode_cache_append": {"span_us": 1e3 * a_ms / max(a_launches, 1),
-                                "bytes": append_bytes,
-                                "concurrent_with": "frame_attn_lse_importance (side stream)"},
+        "decode_cache_append": {"bytes": append_bytes, "launched_with": "state_select_gather"},
         "state_select_gather": {"avg_us": 1e3 * s_ms / max(s_launches, 1),
                                 "share": s_ms / max(1e-9, k1_ms + s_ms)},
     }
+    if a_launches:
+        kernels["decode_cache_append"] = {"span_us": 1e3 * a_ms / a_launches, "bytes": append_bytes,
+                                          "concurrent_with": "frame_attn_lse_importance (side stream)"}
     value = world * S * args.steps / (total_ms_max * 1e-3)
     ps = sorted(per_step)
     # flat per-frame cost: slope of a linear fit of per-frame time against the
@@ -436,7 +436,7 @@ def run_ours(args, world, rank, local):
                      "flops_per_launch": flops},
         "kernels": kernels,
         "flatness": flatness,
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": (4 if a_launches else 2) * args.steps,
     }
     line["config"]["kernel_timing"] = (f"kernel durations from a second pass of {kpass} steps over the same "
                                        "inputs with per-launch CUDA events on the launching streams; the "

@@ -357,6 +357,7 @@ statekv_status statekv_cache_view(const statekv_handle* h, int32_t stream, int32
 /* Optional per-kernel timing with CUDA events recorded on the call's stream
  * around each launch.  enable != 0 starts a new record; read synchronises on
  * the recorded events and returns, per kernel kind (0 = decode-cache append,
+ * where it is a launch of its own,
  * 1 = frame attention + importance, 2 = state select/gather, 3 = the block's
  * projection GEMMs, 4 = the block's RMSNorm / RoPE / SiLU kernels), the
  * number of launches and their summed device milliseconds. */

@@ -505,9 +505,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint4* src = q_src(w);
         if (src) asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
     };
-    // the first unit's rows load while the barriers and TMEM are set up
-    load_q(w0);
-
     if (threadIdx.x == 0) {
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(&slot_full[i], 1);
@@ -534,6 +531,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
+    // Launched programmatically: everything above overlaps the end of the stream's
+    // previous kernel, and nothing it wrote is read before this wait.  Then the next
+    // kernel (the selection) may come in as SMs fall idle.
+    pdl_wait();
+    pdl_launch_dependents();
+    load_q(w0);  // the first unit's rows
     __syncthreads();
     // Split form: every thread of the cluster passes four phases of its barrier, on
     // every path: 0 all CTAs run, 1 row statistics exchanged, 2 O staged, 3 O read.
@@ -1172,20 +1175,23 @@ int current_device_sms()
 // memory, measured by attn_prepare (0: not measured, or none).
 int g_attn_clusters[kMaxDevices][2][kMaxSplit + 1] = {};
 
+// attr: two entries
 template <int D>
-cudaLaunchConfig_t split_config(int units, int S, cudaStream_t st, cudaLaunchAttribute* attr)
+cudaLaunchConfig_t launch_config(int grid, int S, cudaStream_t st, cudaLaunchAttribute* attr)
 {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(units) * S);
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = AttnLayout<D>::kAlloc;
     cfg.stream = st;
-    attr->id = cudaLaunchAttributeClusterDimension;
-    attr->val.clusterDim.x = S;
-    attr->val.clusterDim.y = 1;
-    attr->val.clusterDim.z = 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = S;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = S > 1 ? 2 : 1;
     return cfg;
 }
 
@@ -1211,8 +1217,10 @@ cudaError_t prepare_one()
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if ((e = prepare_form<D, false>()) != cudaSuccess || (e = prepare_form<D, true>()) != cudaSuccess) return e;
     for (int S = 2; S <= kMaxSplit; ++S) {
-        cudaLaunchAttribute attr[1];
-        const cudaLaunchConfig_t cfg = split_config<D>(1, S, nullptr, attr);
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = launch_config<D>(S, S, nullptr, attr);
+        cfg.attrs = attr + 1;  // the cluster size alone
+        cfg.numAttrs = 1;
         int n = 0;
         if ((e = cudaOccupancyMaxActiveClusters(&n, frame_attn_lse_importance<D, true>, &cfg)) != cudaSuccess)
             return e;
@@ -1248,16 +1256,12 @@ cudaError_t launch_one(const CUtensorMap& tm_sk, const CUtensorMap& tm_sv, const
     if (W <= 0) return cudaSuccess;
     if (W > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     p.split = p.selftest_stall ? 1 : split_for<D>(W, (p.keys_hint + kBN - 1) / kBN + (p.T + kBN - 1) / kBN);
-    if (p.split > 1) {
-        cudaLaunchAttribute attr[1];
-        const cudaLaunchConfig_t cfg = split_config<D>(static_cast<int>(W), p.split, st, attr);
-        return cudaLaunchKernelEx(&cfg, frame_attn_lse_importance<D, true>, tm_sk, tm_sv, tm_fk, tm_fv, p);
-    }
     const int sms = current_device_sms();
-    const int grid = static_cast<int>(W < sms ? W : sms);
-    frame_attn_lse_importance<D, false><<<grid, kThreads, AttnLayout<D>::kAlloc, st>>>(tm_sk, tm_sv, tm_fk,
-                                                                                     tm_fv, p);
-    return cudaSuccess;
+    const int grid = p.split > 1 ? static_cast<int>(W) * p.split : static_cast<int>(W < sms ? W : sms);
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = launch_config<D>(grid, p.split, st, attr);
+    return p.split > 1 ? cudaLaunchKernelEx(&cfg, frame_attn_lse_importance<D, true>, tm_sk, tm_sv, tm_fk, tm_fv, p)
+                       : cudaLaunchKernelEx(&cfg, frame_attn_lse_importance<D, false>, tm_sk, tm_sv, tm_fk, tm_fv, p);
 }
 
 }  // namespace

@@ -1,9 +1,9 @@
 // Host runtime behind include/statekv.h: configuration checks, arena
 // carve-up, TMA descriptor encoding, launch sequencing and profiling.
 //
-// Per call, in stream order:  K4 append -> K1 attention -> K3 select/gather.
-// K4 reads the per-head frame counter before K3 advances it; K1 reads the
-// state before K3 rewrites it.
+// Per call, in stream order:  K1 attention -> K3 select/gather with the decode-
+// cache append (recency window: K4 append on a side stream beside K1, then the
+// scatter).  K1 reads the state before K3 rewrites it.
 #include "../../include/statekv.h"
 #include "statekv_kernels.cuh"
 
@@ -96,7 +96,7 @@ Layout make_layout(const statekv_config& c, const Derived& d)
     L.counts = take(heads * 4);
     L.frames = take(heads * 4);
     L.text = take(heads * 4);  // decode-cache rows appended after the video frames
-    L.tickets = take(heads * 4);  // decode kernel: finished CTAs per head, 0 between calls
+    L.tickets = take(heads * 4);  // select and decode kernels: finished CTAs, 0 between calls
     L.cache_k = take(heads * static_cast<size_t>(d.cap) * D * 2);
     L.cache_v = take(heads * static_cast<size_t>(d.cap) * D * 2);
     // importance partials of a frame step; a decode step's split-K partials
@@ -173,8 +173,8 @@ struct statekv_handle {
     bool prof_on;
     size_t prof_used;
     std::vector<ProfRec> prof;
-    // The decode-cache append runs on a side stream forked from the call's
-    // stream and joined before the selection: it depends on nothing the
+    // Recency window: the decode-cache append runs on a side stream forked from the
+    // call's stream and joined before the state update: it depends on nothing the
     // attention kernel writes, so it fills SMs the attention grid leaves idle.
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -309,12 +309,13 @@ statekv_status run_step(statekv_handle* h, const statekv_frame_args& a, cudaStre
     ap.row_mul = T;
     ap.cap = d.cap;
     ap.status = h->status_dev;
-    // append on the side stream; it reads the frame counters, so the join
-    // comes before the selection kernel advances them
-    if (cudaEventRecord(h->ev_fork, st) != cudaSuccess ||
+    // recency window: append on the side stream; it reads the frame counters, so the
+    // join comes before the scatter advances them
+    if (c.selection == 1 &&
+        (cudaEventRecord(h->ev_fork, st) != cudaSuccess ||
         cudaStreamWaitEvent(h->side, h->ev_fork, 0) != cudaSuccess ||
         timed(h, 0, h->side, [&] { return launch_append(ap, h->side); }) != cudaSuccess ||
-        cudaEventRecord(h->ev_join, h->side) != cudaSuccess)
+        cudaEventRecord(h->ev_join, h->side) != cudaSuccess))
         return STATEKV_ERR_CUDA;
 
     AttnParams pa{};
@@ -339,10 +340,10 @@ statekv_status run_step(statekv_handle* h, const statekv_frame_args& a, cudaStre
     pa.watchdog_ns = 1000000ull * (c.watchdog_ms ? c.watchdog_ms : 2000u);
     const cudaError_t ek =
         timed(h, 1, st, [&] { return launch_attn(D, h->tm_sk, h->tm_sv, tm_fk, tm_fv, pa, U, st); });
-    const cudaError_t ej = cudaStreamWaitEvent(st, h->ev_join, 0);  // the append is done
-    if (ek != cudaSuccess || ej != cudaSuccess) return STATEKV_ERR_CUDA;
+    if (ek != cudaSuccess) return STATEKV_ERR_CUDA;
 
     if (c.selection == 1) {
+        if (cudaStreamWaitEvent(st, h->ev_join, 0) != cudaSuccess) return STATEKV_ERR_CUDA;  // the append is done
         RecencyParams pr{};
         pr.k = ap.k;
         pr.v = ap.v;
@@ -379,6 +380,10 @@ statekv_status run_step(statekv_handle* h, const statekv_frame_args& a, cudaStre
     ps.P = d.P;
     ps.MT = d.MT;
     ps.shared = c.selection == 2 ? 1 : 0;
+    ps.cache_k = ap.cache_k;
+    ps.cache_v = ap.cache_v;
+    ps.tickets = h->at<unsigned>(h->lay.tickets);
+    ps.cap = d.cap;
     if (timed(h, 2, st, [&] { return launch_select(ps, U, st); }) != cudaSuccess)
         return STATEKV_ERR_CUDA;
     }

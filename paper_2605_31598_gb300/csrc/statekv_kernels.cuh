@@ -106,6 +106,11 @@ struct SelectParams {
     UnitRange units;
     int T, Hkv, D, B, P, MT;
     int shared;                 // 1: rank by the importance summed over every KV head
+    __nv_bfloat16* cache_k;     // arena [S*L][Hkv][cap][D]: the frame's rows are appended
+    __nv_bfloat16* cache_v;
+    unsigned* tickets;          // arena [S*L][Hkv]: a unit's finished CTAs at its first head; 0 between calls
+    long long cap;
+    int U, appenders;           // units of the call, append CTAs per unit (set by launch_select)
 };
 
 struct AppendParams {
