@@ -73,7 +73,6 @@ constexpr int kThreads = 128 + kSoftThreads;
 constexpr int kSlots = 6;        // 32 KB K/V tile slots (D = 128), one ring
 constexpr int kStep = 64;        // keys per step: half a K/V tile
 constexpr int kMaxSplit = 8;     // CTAs that may share a unit (the portable cluster size)
-constexpr int kMinSplitTiles = 3;  // key tiles a CTA of a shared unit has at least
 constexpr int kBufs = 5;         // score buffers
 // TMEM columns: Q [0, 64) | O [64, 192) | five score buffers of 64 columns.
 // A step's P (bf16 pairs) overwrites the first 32 columns of its own scores.
@@ -151,13 +150,6 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b)
     return d;
 }
 
-__device__ __forceinline__ unsigned long long globaltimer()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -166,25 +158,6 @@ __device__ __forceinline__ void named_bar_sync(int id, int nthreads)
 __device__ __forceinline__ void named_bar_arrive(int id, int nthreads)
 {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
-__device__ __forceinline__ void arrive_at(uint32_t bar, uint32_t n = 1)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
-}
-
-__device__ __forceinline__ void expect_at(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_load_at(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
-                                            int c3)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
 }
 
 // A position in a cycle of N places (ring slots, score buffers) and the parity of
@@ -206,56 +179,6 @@ struct Cycle {
         }
     }
 };
-
-__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
-
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile(
-        "{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}"
-        : "=r"(p));
-    return p != 0;
-}
-
-// D[d] (+)= A[a] B (bf16 in, fp32 accumulator, A in TMEM), issued by one lane of a
-// converged warp whose lanes all hold the same operands.  tcgen05.mma takes them
-// from uniform registers: where the compiler sees one lane in a branch of its
-// own it moves each into place for every MMA, and eight of them take 380 to 950
-// cycles to issue (more when the neighbouring warps do arithmetic) instead of 85.
-__device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, bool accumulate)
-{
-    if (elect_one())
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
-            "r"(a), "l"(b), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
-            : "memory");
-}
-__device__ __forceinline__ void commit_elect(uint32_t bar)
-{
-    if (elect_one())
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                     : "memory");
-}
-// Bounded wait of a converged warp: the polls stay inside one asm statement, so
-// the code around it remains uniform; the deadline is looked at between them.
-__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, unsigned long long deadline)
-{
-    for (;;) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred P1;\n\t.reg .u32 c;\n\tmov.u32 c, 64;\n"
-            "W%=:\n\tmbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t@P1 bra D%=;\n\t"
-            "sub.u32 c, c, 1;\n\tsetp.ne.u32 P1, c, 0;\n\t@P1 bra W%=;\n\tsetp.ne.u32 P1, 0, 0;\n"
-            "D%=:\n\tselp.u32 %0, 1, 0, P1;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (__all_sync(0xffffffffu, done)) return true;
-        if (__any_sync(0xffffffffu, globaltimer() > deadline)) return false;
-    }
-}
 
 // 16 consecutive 32-bit TMEM columns of this thread's lane <- registers.
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16])
@@ -1231,16 +1154,18 @@ cudaError_t prepare_one()
 }
 
 // CTAs per unit: as many as let every unit's cluster be resident at once (so the
-// split form runs where the units leave half of the SMs idle or more) and leave
-// every CTA kMinSplitTiles key tiles; the two exchanges cost about as much as two
-// tiles.  At 15 tiles and S = 3 (5 each) 32.5 us per frame against 36.1 whole.
+// split form runs where the units leave half of the SMs idle or more), if each CTA
+// then has kMinSaved tiles fewer than the unit: the two exchanges cost ~4.4 us, a
+// tile 0.8.  Per launch (ncu): 7 tiles whole ~17 us, on two CTAs 21.5; 15 tiles
+// whole 23.5 us, on three 20.
+constexpr int kMinSaved = 7;
 template <int D>
 int split_for(long long W, int tiles)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 1;
     for (int S = kMaxSplit; S >= 2; --S)
-        if (W <= g_attn_clusters[dev][D == 128][S] && tiles >= kMinSplitTiles * S) return S;
+        if (W <= g_attn_clusters[dev][D == 128][S] && tiles - (tiles + S - 1) / S >= kMinSaved) return S;
     return 1;
 }
 

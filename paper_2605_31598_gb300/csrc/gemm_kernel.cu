@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     volatile int* last_flag = reinterpret_cast<volatile int*>(sm + L::kOffMisc + 8);
     const bool split = BN == 128 && p.splits > 1;  // the plan splits K only with 128-wide tiles
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kGStages; ++i) {
             mbar_init(&full[i], 1);
@@ -266,90 +266,93 @@ __global__ void __launch_bounds__(kGThreads, 1)
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        // (the whole warp runs the loop, with uniform operands, and elects a lane for
+        // the copies; the MMA issuer likewise)
+        if (elect_one()) {
             tma_prefetch_desc(&tm_x);
             tma_prefetch_desc(&tm_w);
-            int last_use[kGStages];
-#pragma unroll
-            for (int s = 0; s < kGStages; ++s) last_use[s] = -1;
-            bool ok = true;
-            int n = 0;
-            for (int w = blockIdx.x; ok && w < p.units; w += gridDim.x) {
-                const GemmUnit x = gemm_unit<BN>(p, w);
-                const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
-                for (int ks = x.ks0; ks < x.ks1; ++ks, ++n) {
-                    if (*abort_flag) {
-                        ok = false;
-                        break;
-                    }
-                    const int s = n % kGStages, use = n / kGStages;
-                    if (use >= 1 && !g_wait(&empty[s], (use - 1) & 1, deadline)) {
-                        fail(2);
-                        ok = false;
-                        break;
-                    }
-                    uint8_t* base = sm + s * kGStageBytes;
-                    mbar_arrive_expect_tx(&full[s], (x.two ? 2 : 1) * kGTileA + kGTileB);
-                    const int kc = ks * kGemmBK;
-                    tma_load_4d(base, &tm_x, &full[s], kc, x.m0, 0, 0);
-                    if (x.two) tma_load_4d(base + kGTileA, &tm_x, &full[s], kc, x.m0 + kGemmBM, 0, 0);
-                    if (p.paired_I) {  // BN / 2 gate rows, then the same up rows
-                        tma_load_4d(base + 2 * kGTileA, &tm_w, &full[s], kc, x.n0, 0, 0);
-                        tma_load_4d(base + 2 * kGTileA + kGTileB / 2, &tm_w, &full[s], kc, x.n0, 1, 0);
-                    } else {
-                        tma_load_4d(base + 2 * kGTileA, &tm_w, &full[s], kc, x.n0, 0, 0);
-                    }
-                    last_use[s] = use;
-                }
-            }
-            // let every copy land before the CTA's memory goes away
-            const unsigned long long dl = g_globaltimer() + p.watchdog_ns;
-            for (int s = 0; s < kGStages; ++s)
-                if (last_use[s] >= 0) g_wait(&full[s], last_use[s] & 1, dl);
         }
         __syncwarp();
+        const uint32_t s0 = uniform(smem_addr(sm)), bfull = smem_addr(full), bempty = smem_addr(empty);
+        bool ok = true;
+        uint32_t n = 0, s = 0, ph = 0;  // steps loaded, the next one's stage and its turn's parity
+        for (int w = blockIdx.x; ok && w < p.units; w += gridDim.x) {
+            const GemmUnit x = gemm_unit<BN>(p, w);
+            const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
+#pragma unroll 1
+            for (int ks = x.ks0; ks < x.ks1; ++ks, ++n) {
+                if (n >= kGStages && !wait_warp(bempty + 8 * s, ph ^ 1u, deadline)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t base = s0 + s * kGStageBytes, bar = bfull + 8 * s;
+                if (elect_one()) {
+                    expect_at(bar, (x.two ? 2 : 1) * kGTileA + kGTileB);
+                    const int kc = ks * kGemmBK;
+                    tma_load_at(base, &tm_x, bar, kc, x.m0, 0, 0);
+                    if (x.two) tma_load_at(base + kGTileA, &tm_x, bar, kc, x.m0 + kGemmBM, 0, 0);
+                    if (p.paired_I) {  // BN / 2 gate rows, then the same up rows
+                        tma_load_at(base + 2 * kGTileA, &tm_w, bar, kc, x.n0, 0, 0);
+                        tma_load_at(base + 2 * kGTileA + kGTileB / 2, &tm_w, bar, kc, x.n0, 1, 0);
+                    } else {
+                        tma_load_at(base + 2 * kGTileA, &tm_w, bar, kc, x.n0, 0, 0);
+                    }
+                }
+                if (++s == kGStages) s = 0, ph ^= 1;
+            }
+            if (!ok && lane == 0) fail(2);
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
+        }
+        // let every copy land before the CTA's memory goes away: the last min(n, stages)
+        const unsigned long long dl = g_globaltimer() + p.watchdog_ns;
+        for (uint32_t i = 0; i < kGStages && i < n; ++i) {
+            const bool wrap = s == 0;
+            s = wrap ? kGStages - 1 : s - 1;
+            ph ^= wrap ? 1u : 0u;
+            wait_warp(bfull + 8 * s, ph, dl);
+        }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t kId = idesc_bf16_f32(kGemmBM, BN, false, false);
-            const uint32_t s0 = smem_addr(sm);
-            bool ok = true;
-            int n = 0, u = 0, site = 3;
-            for (int w = blockIdx.x; ok && w < p.units; w += gridDim.x, ++u) {
-                const GemmUnit x = gemm_unit<BN>(p, w);
-                const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
-                const int buf = u % NB;
-                site = 4;
-                if (u >= NB && !(ok = g_wait(&acc_empty[buf], ((u - NB) / NB) & 1, deadline))) break;
+        constexpr uint32_t kId = idesc_bf16_f32(kGemmBM, BN, false, false);
+        const uint32_t s0 = uniform(smem_addr(sm)), t0 = uniform(tbase);
+        const uint32_t bfull = smem_addr(full), bempty = smem_addr(empty), baf = smem_addr(acc_full),
+                       bae = smem_addr(acc_empty);
+        bool ok = true;
+        uint32_t s = 0, ph = 0, u = 0;
+        int site = 3;
+        for (int w = blockIdx.x; ok && w < p.units; w += gridDim.x, ++u) {
+            const GemmUnit x = gemm_unit<BN>(p, w);
+            const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
+            const uint32_t buf = u % NB;
+            site = 4;
+            if (u >= NB && !(ok = wait_warp(bae + 8 * buf, ((u - NB) / NB) & 1, deadline))) break;
+            const uint32_t acc0 = t0 + buf * L::kSetStride, acc1 = acc0 + L::kMtStride;
+#pragma unroll 1
+            for (int ks = x.ks0; ks < x.ks1; ++ks) {
+                site = 3;
+                if (!(ok = wait_warp(bfull + 8 * s, ph, deadline))) break;
                 tc_fence_after();
-                const uint32_t acc0 = tbase + buf * L::kSetStride, acc1 = acc0 + L::kMtStride;
-                for (int ks = x.ks0; ks < x.ks1; ++ks, ++n) {
-                    const int s = n % kGStages;
-                    site = 3;
-                    if (!(ok = g_wait(&full[s], (n / kGStages) & 1, deadline))) break;
-                    tc_fence_after();
-                    const uint32_t sa = s0 + s * kGStageBytes;
-                    const uint64_t da0 = sdesc_sw128(sa, 16, 1024);
-                    const uint64_t da1 = sdesc_sw128(sa + kGTileA, 16, 1024);
-                    const uint64_t db = sdesc_sw128(sa + 2 * kGTileA, 16, 1024);
+                const uint32_t sa = s0 + s * kGStageBytes;
+                const uint64_t da0 = sdesc_sw128(sa, 16, 1024);
+                const uint64_t da1 = sdesc_sw128(sa + kGTileA, 16, 1024);
+                const uint64_t db = sdesc_sw128(sa + 2 * kGTileA, 16, 1024);
 #pragma unroll
-                    for (int kk = 0; kk < kGemmBK / 16; ++kk) {
-                        // 16 K-elements = 32 bytes further along each 128-byte row
-                        const uint32_t acc = (ks > x.ks0 || kk > 0) ? 1u : 0u;
-                        umma_bf16(acc0, da0 + 2 * kk, db + 2 * kk, kId, acc);
-                        if (x.two) umma_bf16(acc1, da1 + 2 * kk, db + 2 * kk, kId, acc);
-                    }
-                    umma_commit(&empty[s]);
+                for (int kk = 0; kk < kGemmBK / 16; ++kk) {
+                    // 16 K-elements = 32 bytes further along each 128-byte row
+                    const bool acc = ks > x.ks0 || kk > 0;
+                    umma_ss(acc0, da0 + 2 * kk, db + 2 * kk, kId, acc);
+                    if (x.two) umma_ss(acc1, da1 + 2 * kk, db + 2 * kk, kId, acc);
                 }
-                if (!ok) break;
-                umma_commit(&acc_full[buf]);
+                commit_elect(bempty + 8 * s);
+                if (++s == kGStages) s = 0, ph ^= 1;
             }
-            if (!ok) fail(site);
-            // every MMA issued so far must finish before TMEM is released
-            umma_commit(drain);
-            g_wait(drain, 0, g_globaltimer() + p.watchdog_ns);
+            if (!ok) break;
+            commit_elect(baf + 8 * buf);
         }
-        __syncwarp();
+        if (!ok && lane == 0) fail(site);
+        // every MMA issued so far must finish before TMEM is released
+        commit_elect(smem_addr(drain));
+        wait_warp(smem_addr(drain), 0, g_globaltimer() + p.watchdog_ns);
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..5)
         const int quad = warp & 3;  // TMEM lane quadrant: rows 32 quad .. 32 quad + 31 of a tile
@@ -735,7 +738,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     }
     const int nacc = nv1 > 0 ? 2 : 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int i = 0; i < S; ++i) {
             mbar_init(&full[i], 1);
@@ -765,73 +768,75 @@ __global__ void __launch_bounds__(kGThreads, 1)
     bool ok = true;
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             tma_prefetch_desc(&tm_x);
             tma_prefetch_desc(&tm_w);
-            const uint32_t tx = nacc * kTTileW + p.Mp * kGemmBK * 2;
-            // The weights do not depend on the previous kernel of the stream:
-            // the first ring's worth of W tiles is requested before waiting
-            // for it (a no-op unless launched programmatically), X after.
-            const int pre = min(S, ks1 - ks0);
-            for (int n = 0; n < pre; ++n) {
-                uint8_t* base = sm + n * stage_bytes;
-                mbar_arrive_expect_tx(&full[n], tx);
-                const int kc = (ks0 + n) * kGemmBK;
-                tma_load_4d(base, &tm_w, &full[n], kc, wb0, 0, 0);
-                if (nacc == 2) tma_load_4d(base + kTTileW, &tm_w, &full[n], kc, wb1, 0, 0);
-            }
-            pdl_wait();
-            for (int n = 0; n < pre; ++n)
-                tma_load_4d(sm + n * stage_bytes + x_off, &tm_x, &full[n], (ks0 + n) * kGemmBK, 0, 0, 0);
-            int n = pre;
-            for (int ks = ks0 + pre; ks < ks1; ++ks, ++n) {
-                if (*abort_flag) break;
-                const int s = n % S, use = n / S;
-                if (use >= 1 && !g_wait(&empty[s], (use - 1) & 1, deadline)) {
-                    fail(6);
-                    break;
-                }
-                uint8_t* base = sm + s * stage_bytes;
-                mbar_arrive_expect_tx(&full[s], tx);
-                const int kc = ks * kGemmBK;
-                tma_load_4d(base, &tm_w, &full[s], kc, wb0, 0, 0);
-                if (nacc == 2) tma_load_4d(base + kTTileW, &tm_w, &full[s], kc, wb1, 0, 0);
-                tma_load_4d(base + x_off, &tm_x, &full[s], kc, 0, 0, 0);
-            }
-            // let every copy land before the stages are reused or the CTA's
-            // memory goes away: the last use of stage s is the largest one issued
-            const unsigned long long dl = g_globaltimer() + p.watchdog_ns;
-            for (int s = 0; s < S && s < n; ++s) g_wait(&full[s], ((n - 1 - s) / S) & 1, dl);
         }
         __syncwarp();
+        const uint32_t tx = nacc * kTTileW + p.Mp * kGemmBK * 2;
+        const uint32_t s0 = uniform(smem_addr(sm)), bfull = smem_addr(full), bempty = smem_addr(empty);
+        const uint32_t nk = ks1 - ks0, pre = min(static_cast<uint32_t>(S), nk);
+        auto load_w = [&](uint32_t s, uint32_t n) {  // K step n's W tiles into stage s, by one lane
+            const uint32_t base = s0 + s * stage_bytes, bar = bfull + 8 * s;
+            const int kc = (ks0 + n) * kGemmBK;
+            expect_at(bar, tx);
+            tma_load_at(base, &tm_w, bar, kc, wb0, 0, 0);
+            if (nacc == 2) tma_load_at(base + kTTileW, &tm_w, bar, kc, wb1, 0, 0);
+        };
+        // The weights do not depend on the previous kernel of the stream:
+        // the first ring's worth of W tiles is requested before waiting
+        // for it (a no-op unless launched programmatically), X after.
+        for (uint32_t n = 0; n < pre; ++n)
+            if (elect_one()) load_w(n, n);
+        pdl_wait();
+        for (uint32_t n = 0; n < pre; ++n)
+            if (elect_one())
+                tma_load_at(s0 + n * stage_bytes + x_off, &tm_x, bfull + 8 * n, (ks0 + n) * kGemmBK, 0, 0, 0);
+        uint32_t n = pre, s = pre == static_cast<uint32_t>(S) ? 0 : pre, ph = s == 0 ? 1 : 0;
+#pragma unroll 1
+        for (; n < nk; ++n) {
+            if (!wait_warp(bempty + 8 * s, ph ^ 1u, deadline)) {
+                if (lane == 0) fail(6);
+                break;
+            }
+            if (elect_one()) {
+                load_w(s, n);
+                tma_load_at(s0 + s * stage_bytes + x_off, &tm_x, bfull + 8 * s, (ks0 + n) * kGemmBK, 0, 0, 0);
+            }
+            if (++s == static_cast<uint32_t>(S)) s = 0, ph ^= 1;
+        }
+        // let every copy land before the stages are reused or the CTA's
+        // memory goes away: the last use of stage s is the largest one issued
+        const unsigned long long dl = g_globaltimer() + p.watchdog_ns;
+        for (uint32_t q = 0; q < static_cast<uint32_t>(S) && q < n; ++q)
+            wait_warp(bfull + 8 * q, ((n - 1 - q) / S) & 1, dl);
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t id = idesc_bf16_f32(128, p.Mp, false, false);
-            const uint32_t s0 = smem_addr(sm);
-            int n = 0;
-            for (int ks = ks0; ks < ks1; ++ks, ++n) {
-                const int s = n % S;
-                if (!(ok = g_wait(&full[s], (n / S) & 1, deadline))) break;
-                tc_fence_after();
-                const uint32_t sa = s0 + s * stage_bytes;
-                const uint64_t da0 = sdesc_sw128(sa, 16, 1024);
-                const uint64_t da1 = sdesc_sw128(sa + kTTileW, 16, 1024);
-                const uint64_t dx = sdesc_sw128(sa + x_off, 16, 1024);
+        const uint32_t id = idesc_bf16_f32(128, p.Mp, false, false);
+        const uint32_t s0 = uniform(smem_addr(sm)), t0 = uniform(tbase), bfull = smem_addr(full),
+                       bempty = smem_addr(empty);
+        uint32_t s = 0, ph = 0;
+#pragma unroll 1
+        for (int ks = ks0; ks < ks1; ++ks) {
+            if (!(ok = wait_warp(bfull + 8 * s, ph, deadline))) break;
+            tc_fence_after();
+            const uint32_t sa = s0 + s * stage_bytes;
+            const uint64_t da0 = sdesc_sw128(sa, 16, 1024);
+            const uint64_t da1 = sdesc_sw128(sa + kTTileW, 16, 1024);
+            const uint64_t dx = sdesc_sw128(sa + x_off, 16, 1024);
 #pragma unroll
-                for (int kk = 0; kk < kGemmBK / 16; ++kk) {
-                    const uint32_t acc = (ks > ks0 || kk > 0) ? 1u : 0u;
-                    umma_bf16(tbase, da0 + 2 * kk, dx + 2 * kk, id, acc);
-                    if (nacc == 2) umma_bf16(tbase + 256, da1 + 2 * kk, dx + 2 * kk, id, acc);
-                }
-                umma_commit(&empty[s]);
+            for (int kk = 0; kk < kGemmBK / 16; ++kk) {
+                const bool acc = ks > ks0 || kk > 0;
+                umma_ss(t0, da0 + 2 * kk, dx + 2 * kk, id, acc);
+                if (nacc == 2) umma_ss(t0 + 256, da1 + 2 * kk, dx + 2 * kk, id, acc);
             }
-            if (ok) umma_commit(acc_full);
-            else fail(7);
-            umma_commit(drain);
-            g_wait(drain, 0, g_globaltimer() + p.watchdog_ns);
+            commit_elect(bempty + 8 * s);
+            if (++s == static_cast<uint32_t>(S)) s = 0, ph ^= 1;
         }
-        __syncwarp();
+        if (ok) commit_elect(smem_addr(acc_full));
+        else if (lane == 0) fail(7);
+        commit_elect(smem_addr(drain));
+        wait_warp(smem_addr(drain), 0, g_globaltimer() + p.watchdog_ns);
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..5), part 1
         // thread = W row (TMEM lane); each 32-column TMEM load holds 32 rows of X

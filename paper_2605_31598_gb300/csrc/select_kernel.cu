@@ -427,22 +427,34 @@ __global__ void __launch_bounds__(kSelThreads)
     const int npairs = min(nadm, nfree);
     if (tid == 0 && nadm > nfree) *reinterpret_cast<volatile int32_t*>(p.status) = DEV_BAD_SELECT;
 
-    // 4. gather: 16-byte vector copies of the admitted K and V rows
-    const int chunks = D / 8;
+    // 4. gather: 16-byte vector copies of the admitted K and V rows, kGatherBatch of a
+    // thread's loads in flight before its first store (196 rows of 256 bytes twice
+    // are ten copies per thread: one at a time, each waits for its load)
+    constexpr int kGatherBatch = 8;
+    const int cs = D == 128 ? 4 : 3, chunks = 1 << cs;  // 16-byte chunks per row
     const size_t src_stride = static_cast<size_t>(p.Hkv) * D;
     const __nv_bfloat16* ksrc = p.k + (static_cast<size_t>(u) * T * p.Hkv + hkv) * D;
     const __nv_bfloat16* vsrc = p.v + (static_cast<size_t>(u) * T * p.Hkv + hkv) * D;
     __nv_bfloat16* kdst = p.state_k + head * B * D;
     __nv_bfloat16* vdst = p.state_v + head * B * D;
-    for (int w = tid; w < npairs * chunks * 2; w += kSelThreads) {
-        const int which = w / (npairs * chunks);
-        const int r = w % (npairs * chunks);
-        const int i = r / chunks, ch = r % chunks;
-        const int t = adm_tok[i], s = free_slot[i];
-        if (!SKV_CHECK(t >= 0 && t < T && s >= 0 && s < B, p.status, 2)) continue;
-        const __nv_bfloat16* src = (which ? vsrc : ksrc) + t * src_stride + ch * 8;
-        __nv_bfloat16* dst = (which ? vdst : kdst) + static_cast<size_t>(s) * D + ch * 8;
-        *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(src);
+    for (int w0 = tid; w0 < npairs << (cs + 1); w0 += kGatherBatch * kSelThreads) {
+        uint4 x[kGatherBatch];
+#pragma unroll
+        for (int e = 0; e < kGatherBatch; ++e) {  // copy w: chunk w % chunks of K (even) or V (odd) of a pair
+            const int w = w0 + e * kSelThreads, i = w >> (cs + 1);
+            if (i < npairs)
+                x[e] = *reinterpret_cast<const uint4*>((((w >> cs) & 1) ? vsrc : ksrc) + adm_tok[i] * src_stride +
+                                                       (w & (chunks - 1)) * 8);
+        }
+#pragma unroll
+        for (int e = 0; e < kGatherBatch; ++e) {
+            const int w = w0 + e * kSelThreads, i = w >> (cs + 1);
+            if (i >= npairs) break;
+            const int s = free_slot[i];
+            if (!SKV_CHECK(adm_tok[i] >= 0 && adm_tok[i] < T && s >= 0 && s < B, p.status, 2)) continue;
+            *reinterpret_cast<uint4*>((((w >> cs) & 1) ? vdst : kdst) + static_cast<size_t>(s) * D +
+                                      (w & (chunks - 1)) * 8) = x[e];
+        }
     }
     for (int i = tid; i < npairs; i += kSelThreads)
         if (SKV_CHECK(free_slot[i] >= 0 && free_slot[i] < B, p.status, 3)) pos[free_slot[i]] = L + adm_tok[i];

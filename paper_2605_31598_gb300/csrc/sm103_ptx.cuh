@@ -256,6 +256,87 @@ __device__ __forceinline__ void tmem_ld_wait()
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// ---------------------------------------------------------------- uniform issue
+__device__ __forceinline__ unsigned long long globaltimer()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ __forceinline__ void arrive_at(uint32_t bar, uint32_t n = 1)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ void expect_at(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tma_load_at(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
+                                            int c3)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
+
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// D[d] (+)= A B (bf16 in, fp32 accumulator; umma_ts: A in TMEM, umma_ss: both operands
+// in shared memory), issued by one lane of a converged warp whose lanes all hold the same operands.  tcgen05.mma takes them
+// from uniform registers: where the compiler sees one lane in a branch of its
+// own it moves each into place for every MMA, and eight of them take 380 to 950
+// cycles to issue (more when the neighbouring warps do arithmetic) instead of 85.
+__device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, bool accumulate)
+{
+    if (elect_one())
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+            "r"(a), "l"(b), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
+            : "memory");
+}
+__device__ __forceinline__ void umma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate)
+{
+    if (elect_one()) umma_bf16(d, a, b, idesc, accumulate);
+}
+__device__ __forceinline__ void commit_elect(uint32_t bar)
+{
+    if (elect_one())
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                     : "memory");
+}
+// Bounded wait of a converged warp: the polls stay inside one asm statement, so
+// the code around it remains uniform; the deadline is looked at between them.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, unsigned long long deadline)
+{
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred P1;\n\t.reg .u32 c;\n\tmov.u32 c, 64;\n"
+            "W%=:\n\tmbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t@P1 bra D%=;\n\t"
+            "sub.u32 c, c, 1;\n\tsetp.ne.u32 P1, c, 0;\n\t@P1 bra W%=;\n\tsetp.ne.u32 P1, 0, 0;\n"
+            "D%=:\n\tselp.u32 %0, 1, 0, P1;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (__all_sync(0xffffffffu, done)) return true;
+        if (__any_sync(0xffffffffu, globaltimer() > deadline)) return false;
+    }
+}
+
 // ---------------------------------------------------------------- descriptors
 // Shared-memory matrix descriptor for tcgen05.mma, 128-byte swizzle.
 //   K-major operand: rows of 128 B (64 bf16 along K) in 8-row atoms of
