@@ -17,10 +17,8 @@
 //     not depend on timing;
 //   - one CTA per SM walks the units; TMEM holds two accumulator sets, so the
 //     epilogue of one unit overlaps the main loop of the next;
-//   - GEMMs whose 128-wide tiles would take several rounds on the SMs use W
-//     tiles of 192 or 256 rows when fewer rounds of those cost less (every
-//     projection at eight streams, gate/up from two): one accumulator set, and
-//     each staged byte feeds up to 1.5x the MMA work.
+//   - GEMMs whose tiles fill the SMs anyway run on pairs of CTAs instead
+//     (gemm_pair_tc below: every projection at eight streams, gate/up from two).
 // 192 threads: warp 0 issues the TMA loads (a four-stage ring of 48 KB: X rows
 // m0..m0+127, X rows m0+128..m0+255, W rows n0..n0+127, 64 K-columns each,
 // 128-byte swizzle), warp 1 allocates TMEM and issues tcgen05.mma
@@ -44,22 +42,18 @@ constexpr int kGTileA = kGemmBM * kGemmBK * 2;        // 16 KB: 128 rows of X x 
 // rows padded by one float4 against bank conflicts) turns thread-per-row TMEM
 // reads into row-contiguous global stores
 constexpr int kGStageLd = 36;
+constexpr double kNarrowCycles = 872;  // per K step of a 256 x 128 tile, measured
 constexpr int kRG = 8;  // rows per group of the split-K reduction (2 kRG loads in flight)
 
-// Shared memory and TMEM plan for a tile of 256 rows of X x BN rows of W.
-// BN = 128: a four-stage ring of 48 KB and two accumulator sets (2 x 128
-// TMEM columns each), so a unit's epilogue overlaps the next unit's main loop.
-// BN = 192 / 256: a three-stage ring of 56 / 64 KB and one set, its two
-// 128-row accumulators at TMEM columns 0 and 256; each byte staged feeds up to
-// 1.5x the MMA work of BN = 128, and the wider tiles change how many rounds a
-// GEMM's tiles take on the SMs.
-template <int BN>
+// Shared memory and TMEM plan for a tile of 256 rows of X x 128 rows of W: a
+// four-stage ring of 48 KB and two accumulator sets (2 x 128 TMEM columns each),
+// so a unit's epilogue overlaps the next unit's main loop.
 struct GLayout {
-    static constexpr int kStages = BN == 128 ? 4 : 3;
-    static constexpr int kAccSets = BN == 128 ? 2 : 1;
-    static constexpr int kMtStride = BN == 128 ? 128 : 256;  // TMEM columns between the two row tiles
-    static constexpr int kSetStride = 256;                   // TMEM columns between accumulator sets
-    static constexpr int kTileB = BN * kGemmBK * 2;
+    static constexpr int kStages = 4;
+    static constexpr int kAccSets = 2;
+    static constexpr int kMtStride = 128;   // TMEM columns between the two row tiles
+    static constexpr int kSetStride = 256;  // TMEM columns between accumulator sets
+    static constexpr int kTileB = kGemmBN * kGemmBK * 2;
     static constexpr int kStageBytes = 2 * kGTileA + kTileB;
     static constexpr int kOffEpi = kStages * kStageBytes;
     static constexpr int kOffBar = kOffEpi + 4 * 32 * kGStageLd * 4;
@@ -67,10 +61,7 @@ struct GLayout {
     static constexpr int kOffMisc = kOffBar + kNumBars * 8;
     static constexpr int kBytes = kOffMisc + 16;
     static constexpr int kAlloc = kBytes + 1024;      // room to align the base to 1 KB
-    // the epilogue reads the accumulators in 32-column chunks (paired: 32 gate and 32 up
-    // columns at a time), so BN is a multiple of 64
-    static_assert(BN == 128 || BN == 192 || BN == 256, "tile width");
-    static_assert((kAccSets - 1) * kSetStride + kMtStride + BN <= 512, "TMEM columns");
+    static_assert((kAccSets - 1) * kSetStride + kMtStride + kGemmBN <= 512, "TMEM columns");
     static_assert(kAlloc <= 232448, "shared memory budget");
     static_assert(kStageBytes % 1024 == 0 && kGTileA % 1024 == 0, "swizzle atoms stay aligned");
 };
@@ -122,14 +113,13 @@ __device__ __forceinline__ float bf16_round(float x) { return __uint_as_float(bf
 // its other row pairs) while the X rows, far smaller, stay in L2.  Numbered
 // column fastest, a GEMM whose W exceeds L2 re-read it from HBM once per row
 // pair (1.94 GB of DRAM traffic for the 0.34 GB of the 8-stream gate/up).
-template <int BN>
 __device__ __forceinline__ GemmUnit gemm_unit(const GemmParams& p, int w)
 {
     GemmUnit x;
     x.tile = w / p.splits;
     x.split = w - x.tile * p.splits;
     const int m_pairs = (p.M + 2 * kGemmBM - 1) / (2 * kGemmBM);
-    x.n0 = (x.tile / m_pairs) * (p.paired_I ? BN / 2 : BN);  // paired: the output column base
+    x.n0 = (x.tile / m_pairs) * (p.paired_I ? kGemmBN / 2 : kGemmBN);  // paired: the output column base
     x.m0 = (x.tile % m_pairs) * 2 * kGemmBM;
     x.ks0 = x.split * p.kps;
     x.ks1 = min(p.k_steps, x.ks0 + p.kps);
@@ -216,12 +206,11 @@ __device__ __forceinline__ void store_rows_strided(const GemmParams& p, int m0, 
     store4_rows<NR>(p, m0, mstep, nrows, n, a);
 }
 
-template <int BN>
 __global__ void __launch_bounds__(kGThreads, 1)
     gemm_bf16_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                  const GemmParams p)
 {
-    using L = GLayout<BN>;
+    using L = GLayout;
     constexpr int kGStages = L::kStages, kGStageBytes = L::kStageBytes, kGTileB = L::kTileB;
     constexpr int NB = L::kAccSets;
     extern __shared__ uint8_t smem_raw[];
@@ -236,7 +225,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + L::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + L::kOffMisc + 4);
     volatile int* last_flag = reinterpret_cast<volatile int*>(sm + L::kOffMisc + 8);
-    const bool split = BN == 128 && p.splits > 1;  // the plan splits K only with 128-wide tiles
+    const bool split = p.splits > 1;
 
     const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -277,7 +266,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         bool ok = true;
         uint32_t n = 0, s = 0, ph = 0;  // steps loaded, the next one's stage and its turn's parity
         for (int w = blockIdx.x; ok && w < p.units; w += gridDim.x) {
-            const GemmUnit x = gemm_unit<BN>(p, w);
+            const GemmUnit x = gemm_unit(p, w);
             const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
 #pragma unroll 1
             for (int ks = x.ks0; ks < x.ks1; ++ks, ++n) {
@@ -291,7 +280,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                     const int kc = ks * kGemmBK;
                     tma_load_at(base, &tm_x, bar, kc, x.m0, 0, 0);
                     if (x.two) tma_load_at(base + kGTileA, &tm_x, bar, kc, x.m0 + kGemmBM, 0, 0);
-                    if (p.paired_I) {  // BN / 2 gate rows, then the same up rows
+                    if (p.paired_I) {  // 64 gate rows, then the same up rows
                         tma_load_at(base + 2 * kGTileA, &tm_w, bar, kc, x.n0, 0, 0);
                         tma_load_at(base + 2 * kGTileA + kGTileB / 2, &tm_w, bar, kc, x.n0, 1, 0);
                     } else {
@@ -313,7 +302,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        constexpr uint32_t kId = idesc_bf16_f32(kGemmBM, BN, false, false);
+        constexpr uint32_t kId = idesc_bf16_f32(kGemmBM, kGemmBN, false, false);
         const uint32_t s0 = uniform(smem_addr(sm)), t0 = uniform(tbase);
         const uint32_t bfull = smem_addr(full), bempty = smem_addr(empty), baf = smem_addr(acc_full),
                        bae = smem_addr(acc_empty);
@@ -321,7 +310,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         uint32_t s = 0, ph = 0, u = 0;
         int site = 3;
         for (int w = blockIdx.x; ok && w < p.units; w += gridDim.x, ++u) {
-            const GemmUnit x = gemm_unit<BN>(p, w);
+            const GemmUnit x = gemm_unit(p, w);
             const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
             const uint32_t buf = u % NB;
             site = 4;
@@ -362,7 +351,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         bool ok = true;
         int u = 0;
         for (int w = blockIdx.x; w < p.units; w += gridDim.x, ++u) {
-            const GemmUnit x = gemm_unit<BN>(p, w);
+            const GemmUnit x = gemm_unit(p, w);
             const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
             const int buf = u % NB;
             if (ok) ok = __all_sync(0xffffffffu, g_wait(&acc_full[buf], (u / NB) & 1, deadline));
@@ -376,16 +365,16 @@ __global__ void __launch_bounds__(kGThreads, 1)
                                       : nullptr;
                     const uint32_t tacc = tbase + lane_off + buf * L::kSetStride + mt * L::kMtStride;
 #pragma unroll 1
-                    for (int c = 0; c < (p.paired_I ? BN / 64 : BN / 32); ++c) {
+                    for (int c = 0; c < (p.paired_I ? kGemmBN / 64 : kGemmBN / 32); ++c) {
                         // thread = row in TMEM -> a row-major 32 x 32 block in shared
                         // memory -> 4 rows of 8 float4 per warp instruction
                         float v[32];
                         tmem_ld32(tacc + c * 32, v);
                         if (p.paired_I) {
-                            // gate column j and up column j + BN / 2: SiLU(gate) * up,
+                            // gate column j and up column j + 64: SiLU(gate) * up,
                             // each rounded to bf16 first as the unfused path stores them
                             float u[32];
-                            tmem_ld32(tacc + BN / 2 + c * 32, u);
+                            tmem_ld32(tacc + kGemmBN / 2 + c * 32, u);
                             tmem_ld_wait();
 #pragma unroll
                             for (int i = 0; i < 32; ++i) v[i] = silu_times(bf16_round(v[i]), bf16_round(u[i]));
@@ -494,6 +483,237 @@ __global__ void __launch_bounds__(kGThreads, 1)
     if (warp == 1) tmem_dealloc(tbase, 512);
 }
 
+
+// ---------------------------------------------------------------- paired GEMM
+// Two CTAs (a cluster) share a tile of 512 rows of W x BN rows of X.  A tile of
+// the kernel above is bound by shared memory: an MMA of 128 x 128 x 16 reads 8 KB
+// in the 64 cycles it takes and the copies that refill the ring write as much
+// again, 224 B per cycle where an SM moves 128 (872 cycles per 64-wide K step were
+// measured, 896 follow from that, 512 from the tensor core).  Here W is the A
+// operand, two blocks of 256 rows, each CTA holding 128 rows of both, and X the B
+// operand, each CTA holding half of its rows: per K step 8 MMAs of 256 x BN x 16
+// read 4 KB + 16 BN and the copies write 32 KB + 64 BN, max(4 BN, 512 + 1.5 BN)
+// cycles, bound by the tensor core from BN = 208 up.  The whole of TMEM holds one
+// set of accumulators (block b at column 256 b, lane = W row, column = X row), so
+// eight epilogue warps read it out as fast as they can while the ring refills.
+//   Rank 0's barriers `full` count the copies of both CTAs and its warp 1 issues
+// every MMA; a stage's and the accumulators' commits arrive in both CTAs, and
+// both CTAs' epilogue warps arrive on rank 0's acc_empty.
+//   Eight streams of the 7B widths (1568 rows; tiles of 192 or 256 x 256 on single
+// CTAs before -> pairs): gate/up 266 -> 240 us (BN = 224: 518 tiles, 6.8 rounds of
+// 76 pairs; 1780 TFLOP/s), down 172 -> 123 (BN = 160: 70 tiles, one round; 1730
+// TFLOP/s), QKV 44 -> 40, O 43 -> 36; two layers of the block 1312 -> 1189 us.
+constexpr int kPThreads = 320;  // producer, MMA issuer, eight epilogue warps
+constexpr int kPEpiWarps = 8;
+constexpr int kPTileW = 128 * kGemmBK * 2;  // 16 KB: this CTA's rows of one W block x 64 K
+constexpr int kPEpiBytes = kPEpiWarps * 32 * kGStageLd * 4;
+constexpr int kPBarBytes = 256;
+constexpr int kPSmemMax = 232448;
+
+__host__ __device__ constexpr int pair_stage_bytes(int bn) { return 2 * kPTileW + bn / 2 * kGemmBK * 2; }
+__host__ __device__ constexpr int pair_stages(int bn)
+{
+    return (kPSmemMax - 1024 - kPBarBytes - kPEpiBytes) / pair_stage_bytes(bn) >= 4 ? 4 : 3;
+}
+constexpr int pair_smem(int bn) { return pair_stages(bn) * pair_stage_bytes(bn) + kPEpiBytes + kPBarBytes + 1024; }
+static_assert(pair_smem(kPairMaxBN) <= kPSmemMax && pair_smem(224) <= kPSmemMax, "shared memory budget");
+static_assert(pair_smem(kPairMinBN) > 233472 / 2, "one CTA per SM");
+
+__global__ void __launch_bounds__(kPThreads, 1)
+    gemm_pair_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
+                 const GemmParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+    const int BN = p.pair_bn, S = pair_stages(BN), stage_bytes = pair_stage_bytes(BN);
+    uint8_t* epi = sm + S * stage_bytes;
+    uint64_t* full = reinterpret_cast<uint64_t*>(epi + kPEpiBytes);  // stage loaded (rank 0: in both CTAs)
+    uint64_t* empty = full + 4;                                      // stage read by its MMAs
+    uint64_t* acc_full = full + 8;
+    uint64_t* acc_empty = full + 9;
+    uint64_t* drain = full + 10;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 11);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int rank = uniform(cluster_ctarank());
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < S; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], 1);
+        }
+        mbar_init(acc_full, 1);
+        mbar_init(acc_empty, 2 * kPEpiWarps);
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) tmem_alloc_pair(tmem_slot, 512);
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = *tmem_slot;
+    cluster_sync();  // both CTAs' barriers stand
+    auto fail = [&](int site) {
+        if (atomicExch(const_cast<int*>(abort_flag), 1) == 0)
+            *reinterpret_cast<volatile int32_t*>(p.status) = DEV_TIMEOUT_GEMM | (site << 8);
+    };
+    // Tiles are numbered X rows fastest, as above: the pairs running at the same
+    // time share W tiles.
+    const int m_tiles = (p.M + BN - 1) / BN, step = gridDim.x / 2;
+    // blocks of W of unit w: rows n0 (+ 256), or the gate and up rows from n0
+    auto unit_n0 = [&](int w) { return w / m_tiles * (p.paired_I ? 256 : 512); };
+    auto two_blocks = [&](int n0) { return p.paired_I || n0 + 256 < p.N; };
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ TMA producer
+        if (elect_one()) {
+            tma_prefetch_desc(&tm_x);
+            tma_prefetch_desc(&tm_w);
+        }
+        __syncwarp();
+        const uint32_t s0 = uniform(smem_addr(sm)), bfull = smem_addr(full), bempty = smem_addr(empty);
+        const uint32_t rfull = uniform(dsmem_addr(bfull, 0));
+        bool ok = true;
+        int n = 0;
+        uint32_t s = 0, ph = 0;
+        for (int w = blockIdx.x / 2; ok && w < p.units; w += step) {
+            const int n0 = unit_n0(w) + rank * 128, m0 = w % m_tiles * BN + rank * (BN / 2);
+            const bool two = two_blocks(unit_n0(w));
+            const uint32_t bytes = 2u * ((two ? 2 : 1) * kPTileW + BN / 2 * kGemmBK * 2);  // of both CTAs
+            const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
+#pragma unroll 1
+            for (int ks = 0; ks < p.k_steps; ++ks, ++n) {
+                if (n >= S && !wait_warp(bempty + 8 * s, ph ^ 1u, deadline)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t base = s0 + s * stage_bytes, bar = rfull + 8 * s;
+                if (elect_one()) {
+                    const int kc = ks * kGemmBK;
+                    if (rank == 0) expect_at(bfull + 8 * s, bytes);
+                    tma_load_pair(base, &tm_w, bar, kc, n0, 0, 0);
+                    if (two) tma_load_pair(base + kPTileW, &tm_w, bar, kc, p.paired_I ? n0 : n0 + 256, p.paired_I ? 1 : 0, 0);
+                    tma_load_pair(base + 2 * kPTileW, &tm_x, bar, kc, m0, 0, 0);
+                }
+                if (++s == static_cast<uint32_t>(S)) s = 0, ph ^= 1;
+            }
+            if (!ok && lane == 0) fail(2);
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
+        }
+        // Every copy lands before the CTA's memory goes away: rank 0's last MMAs have
+        // waited for those of both CTAs.  After a failure the two may have stopped at
+        // different steps and some of the barriers stay open, so time passes instead,
+        // far more than a copy takes.
+        if (!ok) {
+            const unsigned long long until = g_globaltimer() + 2000000ull;
+            while (g_globaltimer() < until) __nanosleep(1000);
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer (rank 0)
+        if (rank == 0) {
+            const uint32_t id = uniform(idesc_bf16_f32(256, BN, false, false));
+            const uint32_t s0 = uniform(smem_addr(sm)), t0 = uniform(tbase);
+            const uint32_t bfull = smem_addr(full), bempty = smem_addr(empty), baf = smem_addr(acc_full),
+                           bae = smem_addr(acc_empty);
+            bool ok = true;
+            uint32_t s = 0, ph = 0, u = 0;
+            int site = 3;
+            for (int w = blockIdx.x / 2; ok && w < p.units; w += step, ++u) {
+                const bool two = two_blocks(unit_n0(w));
+                const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
+                site = 4;
+                if (u >= 1 && !(ok = wait_warp(bae, (u - 1) & 1, deadline))) break;
+                tc_fence_after();
+#pragma unroll 1
+                for (int ks = 0; ks < p.k_steps; ++ks) {
+                    site = 3;
+                    if (!(ok = wait_warp(bfull + 8 * s, ph, deadline))) break;
+                    tc_fence_after();
+                    const uint32_t sa = s0 + s * stage_bytes;
+                    const uint64_t da0 = sdesc_sw128(sa, 16, 1024);
+                    const uint64_t da1 = sdesc_sw128(sa + kPTileW, 16, 1024);
+                    const uint64_t dx = sdesc_sw128(sa + 2 * kPTileW, 16, 1024);
+#pragma unroll
+                    for (int kk = 0; kk < kGemmBK / 16; ++kk) {
+                        const bool acc = ks > 0 || kk > 0;
+                        umma_ss_pair(t0, da0 + 2 * kk, dx + 2 * kk, id, acc);
+                        if (two) umma_ss_pair(t0 + 256, da1 + 2 * kk, dx + 2 * kk, id, acc);
+                    }
+                    commit_elect_pair(bempty + 8 * s);
+                    if (++s == static_cast<uint32_t>(S)) s = 0, ph ^= 1;
+                }
+                if (!ok) break;
+                commit_elect_pair(baf);
+            }
+            if (!ok && lane == 0) fail(site);
+            // every MMA issued so far must finish before TMEM is released
+            commit_elect_pair(smem_addr(drain));
+        }
+        wait_warp(smem_addr(drain), 0, g_globaltimer() + p.watchdog_ns);
+    } else {
+        // ------------------------------------------------------------ epilogue (warps 2..9)
+        // thread = W row (TMEM lane); a 32-column TMEM load holds 32 rows of X, which
+        // go through shared memory to 4 rows of 8 float4 per warp instruction
+        const int quad = warp & 3, half = (warp - 2) >> 2;
+        const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
+        float* stg = reinterpret_cast<float*>(epi) + (warp - 2) * 32 * kGStageLd;
+        const int sub = lane >> 3, c4 = lane & 7;
+        const uint32_t bae = dsmem_addr(smem_addr(acc_empty), 0);
+        bool ok = true;
+        uint32_t u = 0;
+        for (int w = blockIdx.x / 2; ok && w < p.units; w += step, ++u) {
+            const int n0 = unit_n0(w), m0 = w % m_tiles * BN;
+            const int mend = min(BN, p.M - m0);               // rows of the tile below M
+            const int chunks = (mend + 31) / 32;
+            const int items = p.paired_I || !two_blocks(n0) ? chunks : 2 * chunks;
+            const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
+            ok = wait_warp(smem_addr(acc_full), u & 1, deadline);
+            if (!ok) break;
+            tc_fence_after();
+            bool released = false;
+#pragma unroll 1
+            for (int i = half; i < items; i += 2) {
+                const int b = i >= chunks ? 1 : 0, c = i - b * chunks;
+                float v[32];
+                tmem_ld32(tbase + lane_off + 256 * b + 32 * c, v);
+                if (p.paired_I) {
+                    // SiLU(gate) * up, each rounded to bf16 first as the unfused path
+                    // stores them
+                    float g[32];
+                    tmem_ld32(tbase + lane_off + 256 + 32 * c, g);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = silu_times(bf16_round(v[j]), bf16_round(g[j]));
+                }
+                tmem_ld_wait();
+                if (i + 2 >= items) {  // the warp's last read: the MMA may refill the accumulators
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) arrive_cluster(bae);
+                    released = true;
+                }
+#pragma unroll
+                for (int j = 0; j < 32; ++j) stg[j * kGStageLd + lane] = v[j];
+                __syncwarp();
+                float4 acc[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    acc[q] = *reinterpret_cast<const float4*>(stg + (4 * q + sub) * kGStageLd + 4 * c4);
+                store_rows4(p, m0 + 32 * c, sub, min(32, mend - 32 * c), n0 + 256 * b + rank * 128 + quad * 32 + 4 * c4,
+                            acc);
+                __syncwarp();
+            }
+            if (!released && lane == 0) arrive_cluster(bae);  // a warp without a chunk
+        }
+        if (!ok && lane == 0) fail(5);
+    }
+    tc_fence_before();
+    __syncthreads();
+    // neither CTA leaves, or frees TMEM, while the other's signals may still come
+    cluster_sync();
+    if (warp == 1) tmem_dealloc_pair(tbase, 512);
+}
 
 // ---------------------------------------------------------------- thin GEMM
 // M <= 256 rows.  The roles swap: W is the A operand (128 of its rows per
@@ -923,28 +1143,30 @@ GemmPlan gemm_plan(int M, int N, int K, int sms)
     GemmPlan g{};
     g.m_pairs = (M + 2 * kGemmBM - 1) / (2 * kGemmBM);
     g.k_steps = (K + kGemmBK - 1) / kGemmBK;
-    // Wider tiles (192 or 256 W rows) when the 128-wide ones take several
-    // rounds on the SMs and fewer rounds of wider ones cost less: a 256-wide
-    // unit measured 1.82x a 128-wide one (twice the work), a 192-wide one
-    // 1.41x.  Only with K long enough to hide the epilogue they cannot overlap
-    // (one accumulator set) and 128-byte aligned rows (at K = 200, or with
-    // K = 3592, they were slower).
-    g.bn = kGemmBN;
     const int narrow = (N + kGemmBN - 1) / kGemmBN * g.m_pairs;
+    // Pairs of CTAs, when the 128-wide tiles fill the SMs (with fewer, splitting
+    // their K is faster) and rounds x cycles per K step come out lower; the
+    // accumulators' read-out, which the pair does not overlap, counts as four K
+    // steps.  Only with K long enough to carry it and 128-byte aligned rows.
     if (narrow >= sms && g.k_steps >= 32 && (K % 64) == 0) {
-        double best = (narrow + sms - 1) / sms;
-        const int widths[2] = {192, 256};
-        const double unit_cost[2] = {1.41, 1.82};
-        for (int i = 0; i < 2; ++i) {
-            const int t = (N + widths[i] - 1) / widths[i] * g.m_pairs;
-            const double cost = ((t + sms - 1) / sms) * unit_cost[i];
-            if (cost < best - 0.05) {
+        double best = (narrow + sms - 1) / sms * static_cast<double>(g.k_steps) * kNarrowCycles;
+        for (int bn = kPairMinBN; bn <= kPairMaxBN; bn += 32) {
+            const int units = (N + 511) / 512 * ((M + bn - 1) / bn), pairs = sms / 2;
+            const double cost = (units + pairs - 1) / pairs * (g.k_steps + 4.0) * std::max(4.0 * bn, 512 + 1.5 * bn);
+            if (cost < best * 0.98) {
                 best = cost;
-                g.bn = widths[i];
+                g.pair_bn = bn;
             }
         }
     }
-    g.n_tiles = (N + g.bn - 1) / g.bn;
+    if (g.pair_bn) {
+        g.n_tiles = (N + 511) / 512;
+        g.kps = g.k_steps;
+        g.splits = 1;
+        g.units = g.n_tiles * ((M + g.pair_bn - 1) / g.pair_bn);
+        return g;
+    }
+    g.n_tiles = (N + kGemmBN - 1) / kGemmBN;
     const int tiles = g.n_tiles * g.m_pairs;
     // split K only while the tiles alone leave SMs idle, into as many ranges as
     // keep every unit in one wave
@@ -960,33 +1182,37 @@ GemmPlan gemm_plan(int M, int N, int K, int sms)
 
 cudaError_t gemm_prepare()
 {
-    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         GLayout<128>::kAlloc);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gemm_bf16_tc<192>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 GLayout<192>::kAlloc);
+    const cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               GLayout::kAlloc);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(gemm_bf16_tc<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                GLayout<256>::kAlloc);
+    return cudaFuncSetAttribute(gemm_pair_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmemMax);
 }
 
 cudaError_t launch_gemm(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const GemmParams& p,
                         int sms, cudaStream_t st)
 {
     if (p.units <= 0) return cudaSuccess;
-    if (p.bn != 128 && p.bn != 192 && p.bn != 256) return cudaErrorInvalidValue;
     if (p.paired_I && (p.splits != 1 || p.paired_I != p.N || p.bias || p.add)) return cudaErrorInvalidValue;
-    const int grid = p.units < sms ? p.units : sms;
-    if (p.bn != 128) {
-        if (p.splits != 1) return cudaErrorInvalidValue;
-        if (p.bn == 192)
-            gemm_bf16_tc<192><<<grid, kGThreads, GLayout<192>::kAlloc, st>>>(tm_x, tm_w, p);
-        else
-            gemm_bf16_tc<256><<<grid, kGThreads, GLayout<256>::kAlloc, st>>>(tm_x, tm_w, p);
-        return cudaGetLastError();
+    if (p.pair_bn) {
+        if (p.splits != 1 || p.pair_bn < kPairMinBN || p.pair_bn > kPairMaxBN || p.pair_bn % 32)
+            return cudaErrorInvalidValue;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(2 * std::max(1, std::min(p.units, sms / 2)));
+        cfg.blockDim = dim3(kPThreads);
+        cfg.dynamicSmemBytes = pair_smem(p.pair_bn);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, gemm_pair_tc, tm_x, tm_w, p);
     }
+    const int grid = p.units < sms ? p.units : sms;
     if (p.splits == 1) {
-        gemm_bf16_tc<128><<<grid, kGThreads, GLayout<128>::kAlloc, st>>>(tm_x, tm_w, p);
+        gemm_bf16_tc<<<grid, kGThreads, GLayout::kAlloc, st>>>(tm_x, tm_w, p);
         return cudaGetLastError();
     }
     // split K: the splits of a tile wait for one another, so every unit's CTA
@@ -995,8 +1221,8 @@ cudaError_t launch_gemm(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const 
     CUtensorMap a = tm_x, b = tm_w;
     GemmParams q = p;
     void* args[] = {&a, &b, &q};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(gemm_bf16_tc<128>), dim3(grid),
-                                       dim3(kGThreads), args, GLayout<128>::kAlloc, st);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(gemm_bf16_tc), dim3(grid),
+                                       dim3(kGThreads), args, GLayout::kAlloc, st);
 }
 
 namespace {

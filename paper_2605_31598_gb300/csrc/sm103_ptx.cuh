@@ -295,10 +295,11 @@ __device__ __forceinline__ bool elect_one()
 }
 
 // D[d] (+)= A B (bf16 in, fp32 accumulator; umma_ts: A in TMEM, umma_ss: both operands
-// in shared memory), issued by one lane of a converged warp whose lanes all hold the same operands.  tcgen05.mma takes them
-// from uniform registers: where the compiler sees one lane in a branch of its
-// own it moves each into place for every MMA, and eight of them take 380 to 950
-// cycles to issue (more when the neighbouring warps do arithmetic) instead of 85.
+// in shared memory), issued by one lane of a converged warp whose lanes all hold
+// the same operands.  tcgen05.mma takes them from uniform registers: where the
+// compiler sees one lane in a branch of its own it moves each into place for
+// every MMA, and eight of them take 380 to 950 cycles to issue (more when the
+// neighbouring warps do arithmetic) instead of 85.
 __device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, bool accumulate)
 {
     if (elect_one())
@@ -318,6 +319,57 @@ __device__ __forceinline__ void commit_elect(uint32_t bar)
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                      : "memory");
 }
+
+// ---------------------------------------------------------------- CTA pairs
+// The cta_group::2 forms: the two CTAs of a cluster work on one tile.  An MMA,
+// issued by rank 0 alone, has M = 256 (each CTA's shared memory holds 128 rows of
+// A and half the rows of B at the same offsets, each CTA's TMEM takes its own 128
+// rows of D); alloc and dealloc are executed by one warp of both CTAs.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols)
+{
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(dst_smem)),
+                 "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols)
+{
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void umma_ss_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate)
+{
+    if (elect_one())
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+            "l"(a), "l"(b), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
+            : "memory");
+}
+// arrives on the barrier at this offset of both CTAs
+__device__ __forceinline__ void commit_elect_pair(uint32_t bar)
+{
+    if (elect_one())
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+            "h"(static_cast<uint16_t>(3))
+            : "memory");
+}
+// into this CTA's shared memory, counted on `bar`, a barrier of either CTA of the
+// pair (a shared::cluster address)
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
+                                              int c3)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
+__device__ __forceinline__ void arrive_cluster(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 // Bounded wait of a converged warp: the polls stay inside one asm statement, so
 // the code around it remains uniform; the deadline is looked at between them.
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, unsigned long long deadline)

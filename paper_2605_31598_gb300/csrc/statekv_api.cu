@@ -983,21 +983,21 @@ statekv_status statekv_block_frame(statekv_handle* h, const statekv_block_config
         const cuuint64_t sw[3] = {static_cast<cuuint64_t>(K) * 2,
                                   static_cast<cuuint64_t>(K) * (paired ? pair_I : N) * 2,
                                   static_cast<cuuint64_t>(K) * N * 2};
-        const cuuint32_t box[4] = {static_cast<cuuint32_t>(kGemmBK), static_cast<cuuint32_t>(kGemmBM), 1, 1};
-        const cuuint32_t wbox[4] = {static_cast<cuuint32_t>(kGemmBK),
-                                    static_cast<cuuint32_t>(paired ? g.bn / 2 : g.bn), 1, 1};
+        const GemmBox gb = gemm_box(g, paired);
+        const cuuint32_t box[4] = {static_cast<cuuint32_t>(kGemmBK), static_cast<cuuint32_t>(gb.x), 1, 1};
+        const cuuint32_t wbox[4] = {static_cast<cuuint32_t>(kGemmBK), static_cast<cuuint32_t>(gb.w), 1, 1};
         if (!encode_4d(&tx, X, dx, sx, box) || !encode_4d(&tw, Wt, dw, sw, wbox)) return false;
         GemmParams gp{};
         gp.M = rows;
         gp.N = paired ? pair_I : N;
         gp.K = K;
-        gp.bn = g.bn;
+        gp.pair_bn = g.pair_bn;
         gp.paired_I = paired ? pair_I : 0;
-        gp.n_tiles = paired ? (pair_I + g.bn / 2 - 1) / (g.bn / 2) : g.n_tiles;
+        gp.n_tiles = paired ? (pair_I + gb.cols - 1) / gb.cols : g.n_tiles;
         gp.k_steps = g.k_steps;
         gp.kps = g.kps;
         gp.splits = g.splits;
-        gp.units = paired ? gp.n_tiles * g.m_pairs : g.units;
+        gp.units = paired ? gp.n_tiles * (g.units / g.n_tiles) : g.units;
         gp.bias = static_cast<const __nv_bfloat16*>(bias);
         gp.D = paired ? D_pair : D;
         gp.add = add ? 1 : 0;

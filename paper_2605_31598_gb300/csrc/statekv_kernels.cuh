@@ -185,18 +185,30 @@ cudaError_t launch_silu_mul(const __nv_bfloat16* gu, __nv_bfloat16* a, long long
 // tile's rows over all splits in split order.
 constexpr int kGemmBM = 128, kGemmBN = 128, kGemmBK = 64;
 struct GemmPlan {
-    int bn;                     // W rows per tile: 128, or 192 / 256 for GEMMs with many tiles (no K split)
+    int pair_bn;                // X rows per tile of the CTA-pair kernel (no K split); 0: 128-wide tiles
     int n_tiles, m_pairs, k_steps, kps, splits, units, counters;
     size_t partial_bytes;
 };
 GemmPlan gemm_plan(int M, int N, int K, int sms);
+// X rows per tile of the CTA-pair kernel: multiples of 32 in this range
+constexpr int kPairMinBN = 96, kPairMaxBN = 256;
+// rows of the X and W tensor maps' boxes (64 K-columns, 128-byte swizzle) and
+// output columns per tile
+struct GemmBox {
+    int x, w, cols;
+};
+inline GemmBox gemm_box(const GemmPlan& g, bool paired)
+{
+    if (g.pair_bn) return {g.pair_bn / 2, 128, paired ? 256 : 512};
+    return {kGemmBM, paired ? kGemmBN / 2 : kGemmBN, paired ? kGemmBN / 2 : kGemmBN};
+}
 struct GemmParams {
     int M, N, K;
-    int bn;                     // the plan's tile width; the W tensor map's box has bn rows
+    int pair_bn;                // the plan's
     int n_tiles, k_steps, kps, splits, units;
     int paired_I;               // > 0: W = gate rows [0, I) then up rows [I, 2 I), D = SiLU(gate) * up
-                                // [M][I] (N = I); the W map is [2][I][K] with boxes of bn / 2 rows,
-                                // tile t covers output columns [t bn / 2, (t + 1) bn / 2); splits = 1
+                                // [M][I] (N = I); the W map is [2][I][K]; tile t covers output columns
+                                // [gemm_box(..).cols t, .. (t + 1)); splits = 1
     const __nv_bfloat16* bias;  // nullable [N]
     __nv_bfloat16* D;           // [M][N]
     int add;                    // 1: D += X W^T

@@ -246,3 +246,19 @@ def test_block_multi_layer_call_equals_layer_calls(streams, tokens):
                 assert torch.equal(ca[0][:, :n * tokens], cb[0][:, :n * tokens])
                 assert torch.equal(ca[1][:, :n * tokens], cb[1][:, :n * tokens])
     assert engs[0].sync() == 0 and engs[1].sync() == 0
+
+
+@pytest.mark.gpu
+def test_block_paired_ctas_ragged_tiles():
+    """11 streams of 196 tokens (2156 rows) and widths that leave ragged tiles of
+    the CTA-pair GEMM (512 W rows x 160 rows of X): hidden 2112 and 36 heads of 64
+    (QKV with bias and down with the residual: 4.1 and 4.5 tiles of W, the last one
+    of a single 256-row block), MLP 2112 (8.25 gate/up tiles of 256), 13.5 tiles of
+    X (no row of the last tile's second half exists)."""
+    from paper_2605_31598_gb300.inputs import BlockShape
+
+    _need_gpu()
+    shape = Shape(28, 4, 64, 196, 208, 2, num_layers=1, num_streams=11)
+    stats = {}
+    worst = run_block_parity(shape, BlockShape(2112, 2112), 2, check_frames=[2], stats=stats)
+    print("paired ragged block worst |dx|", worst, stats)
