@@ -50,7 +50,7 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8])
 // order), scale 1/sqrt(mean + eps), y = v * scale * g rounded once to bf16.
 // Every norm of the block goes through here, so a norm fused into another
 // kernel and the standalone one agree bit for bit.
-__device__ __forceinline__ void norm_write(const float (&v)[kNormChunks][8], int nc, const uint4* gr,
+__device__ __forceinline__ void norm_write(const float (&v)[kNormChunks][8], int nc, const uint4 (&gr)[kNormChunks],
                                            float eps, int H, uint4* yr, float* red)
 {
     float ss = 0.f;
@@ -74,7 +74,7 @@ __device__ __forceinline__ void norm_write(const float (&v)[kNormChunks][8], int
         const int i = threadIdx.x + c * kNormThreads;
         if (i < nc) {
             float gw[8], o[8];
-            unpack8(gr[i], gw);
+            unpack8(gr[c], gw);
 #pragma unroll
             for (int e = 0; e < 8; ++e) o[e] = v[c][e] * r * gw[e];
             yr[i] = pack8(o);
@@ -106,53 +106,81 @@ __global__ void __launch_bounds__(kNormThreads)
                    int H, const RopeParams rp, float2* rope)
 {
     ptx::pdl_launch_dependents();
+    const int nc = H / 8;
+    // The norm's weights are fetched before the wait: no kernel of the block call
+    // writes them, and what ran before the call lies behind the memset it starts with.
+    uint4 gr[kNormChunks];
+#pragma unroll
+    for (int c = 0; c < kNormChunks; ++c) {
+        const int i = threadIdx.x + c * kNormThreads;
+        if (i < nc) gr[c] = reinterpret_cast<const uint4*>(g)[i];
+    }
     ptx::pdl_wait();
     if (rope && threadIdx.x < rp.d / 2)
         rope[static_cast<size_t>(blockIdx.x) * (rp.d / 2) + threadIdx.x] = rope_angle(rp, blockIdx.x, threadIdx.x);
     __shared__ float red[kNormThreads / 32];
     const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<size_t>(blockIdx.x) * H);
-    const int nc = H / 8;
     float v[kNormChunks][8];
 #pragma unroll
     for (int c = 0; c < kNormChunks; ++c) {
         const int i = threadIdx.x + c * kNormThreads;
         if (i < nc) unpack8(xr[i], v[c]);
     }
-    norm_write(v, nc, reinterpret_cast<const uint4*>(g), eps, H,
+    norm_write(v, nc, gr, eps, H,
                reinterpret_cast<uint4*>(y + static_cast<size_t>(blockIdx.x) * H), red);
 }
 
 // One CTA per token: the d/2 angles of its position are formed once (fp64
 // product and reduction modulo 2 pi, fp32 sin/cos) into shared memory, then
-// every q and k head's pairs are rotated from that table and v is copied.
+// every q and k head's pairs are rotated from that table and v is copied.  A
+// thread takes eight pairs, two 16-byte loads that are in flight while the
+// angles are formed (with a pair and its four 2-byte accesses at a time the
+// kernel was bound by their number: 1568 rows of 36 heads of 128 took 17 us, now
+// 11).
 __global__ void __launch_bounds__(256) qkv_rope_kernel(const RopeParams p)
 {
     ptx::pdl_launch_dependents();
     ptx::pdl_wait();
-    __shared__ float cs_tab[64], sn_tab[64];
-    const int half = p.d / 2;
+    __shared__ __align__(16) float cs_tab[64], sn_tab[64];
+    const int half = p.d / 2, gph = half / 8;  // 8-pair groups per head
     const int row = blockIdx.x;  // s * T + t
     const __nv_bfloat16* src = p.qkv + static_cast<size_t>(row) * (p.Hq + 2 * p.Hkv) * p.d;
+    const int groups = (p.Hq + p.Hkv) * gph;
+    int e = threadIdx.x;
+    uint4 r1{}, r2{};
+    auto load = [&] {  // (d is 64 or 128 and the buffers' rows are whole heads: 16-byte aligned)
+        const __nv_bfloat16* at = src + e / gph * p.d + 8 * (e % gph);
+        r1 = *reinterpret_cast<const uint4*>(at);
+        r2 = *reinterpret_cast<const uint4*>(at + half);
+    };
+    if (e < groups) load();
     if (threadIdx.x < half) {
         const float2 a = rope_angle(p, row, threadIdx.x);
         cs_tab[threadIdx.x] = a.x;
         sn_tab[threadIdx.x] = a.y;
     }
     __syncthreads();
-    const int qk_pairs = (p.Hq + p.Hkv) * half;
-    for (int e = threadIdx.x; e < qk_pairs; e += blockDim.x) {
-        const int hh = e / half, k = e - hh * half;
-        const float x1 = __bfloat162float(src[hh * p.d + k]);
-        const float x2 = __bfloat162float(src[hh * p.d + k + half]);
-        const float c = cs_tab[k], sn = sn_tab[k];
+    while (e < groups) {
+        const int hh = e / gph, k = 8 * (e % gph);
+        float x1[8], x2[8], o1[8], o2[8];
+        unpack8(r1, x1);
+        unpack8(r2, x2);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float c = cs_tab[k + i], sn = sn_tab[k + i];
+            o1[i] = x1[i] * c - x2[i] * sn;
+            o2[i] = x2[i] * c + x1[i] * sn;
+        }
         __nv_bfloat16* dst = hh < p.Hq ? p.q + (static_cast<size_t>(row) * p.Hq + hh) * p.d
                                        : p.k + (static_cast<size_t>(row) * p.Hkv + (hh - p.Hq)) * p.d;
-        dst[k] = __float2bfloat16(x1 * c - x2 * sn);
-        dst[k + half] = __float2bfloat16(x2 * c + x1 * sn);
+        e += blockDim.x;
+        if (e < groups) load();
+        *reinterpret_cast<uint4*>(dst + k) = pack8(o1);
+        *reinterpret_cast<uint4*>(dst + k + half) = pack8(o2);
     }
     const uint4* vs = reinterpret_cast<const uint4*>(src + (p.Hq + p.Hkv) * p.d);
     uint4* vd = reinterpret_cast<uint4*>(p.v + static_cast<size_t>(row) * p.Hkv * p.d);
-    for (int e = threadIdx.x; e < p.Hkv * p.d / 8; e += blockDim.x) vd[e] = vs[e];
+    for (int i = threadIdx.x; i < p.Hkv * p.d / 8; i += blockDim.x) vd[i] = vs[i];
 }
 
 // 8 outputs per thread: a = SiLU(gate) * up, gate in columns [0, I), up in [I, 2I).
@@ -175,8 +203,8 @@ __global__ void silu_mul_kernel(const __nv_bfloat16* gu, __nv_bfloat16* a, int r
 
 // Every kernel of the block is launched with programmatic stream
 // serialization: it starts launching while the previous kernel finishes and
-// waits (pdl_wait, first thing) for that kernel's completion before it reads
-// or writes anything.
+// waits (pdl_wait) for that kernel's completion before it reads or writes
+// anything but weights.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args)
 {
