@@ -502,7 +502,9 @@ __global__ void __launch_bounds__(kGThreads, 1)
 //   Eight streams of the 7B widths (1568 rows; tiles of 192 or 256 x 256 on single
 // CTAs before -> pairs): gate/up 266 -> 240 us (BN = 224: 518 tiles, 6.8 rounds of
 // 76 pairs; 1780 TFLOP/s), down 172 -> 123 (BN = 160: 70 tiles, one round; 1730
-// TFLOP/s), QKV 44 -> 40, O 43 -> 36; two layers of the block 1312 -> 1189 us.
+// TFLOP/s), QKV 44 -> 39, O 43 -> 37; two layers of the block 1312 -> 1189 us, and
+// 1131 with programmatic launches (a GEMM's first ring of weights is requested while
+// the kernel before it ends; 1157 before that) and a leaner rotation kernel.
 constexpr int kPThreads = 320;  // producer, MMA issuer, eight epilogue warps
 constexpr int kPEpiWarps = 8;
 constexpr int kPTileW = 128 * kGemmBK * 2;  // 16 KB: this CTA's rows of one W block x 64 K
@@ -554,6 +556,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
     cluster_sync();  // both CTAs' barriers stand
+    pdl_launch_dependents();
     auto fail = [&](int site) {
         if (atomicExch(const_cast<int*>(abort_flag), 1) == 0)
             *reinterpret_cast<volatile int32_t*>(p.status) = DEV_TIMEOUT_GEMM | (site << 8);
@@ -577,6 +580,25 @@ __global__ void __launch_bounds__(kPThreads, 1)
         bool ok = true;
         int n = 0;
         uint32_t s = 0, ph = 0;
+        auto load_w = [&](uint32_t base, uint32_t bar, int ks, int n0, bool two) {
+            const int kc = ks * kGemmBK;
+            tma_load_pair(base, &tm_w, bar, kc, n0, 0, 0);
+            if (two) tma_load_pair(base + kPTileW, &tm_w, bar, kc, p.paired_I ? n0 : n0 + 256, p.paired_I ? 1 : 0, 0);
+        };
+        // The weights do not depend on the previous kernel of the stream: the first
+        // ring's tiles of W (and the phases' byte counts) are requested before waiting
+        // for it, X after.
+        {
+            const int w = blockIdx.x / 2;
+            const bool two = two_blocks(unit_n0(w));
+            const uint32_t bytes = 2u * ((two ? 2 : 1) * kPTileW + BN / 2 * kGemmBK * 2);
+            for (int i = 0; i < min(S, p.k_steps); ++i)
+                if (elect_one()) {
+                    if (rank == 0) expect_at(bfull + 8 * i, bytes);
+                    load_w(s0 + i * stage_bytes, rfull + 8 * i, i, unit_n0(w) + rank * 128, two);
+                }
+        }
+        pdl_wait();
         for (int w = blockIdx.x / 2; ok && w < p.units; w += step) {
             const int n0 = unit_n0(w) + rank * 128, m0 = w % m_tiles * BN + rank * (BN / 2);
             const bool two = two_blocks(unit_n0(w));
@@ -590,11 +612,11 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 }
                 const uint32_t base = s0 + s * stage_bytes, bar = rfull + 8 * s;
                 if (elect_one()) {
-                    const int kc = ks * kGemmBK;
-                    if (rank == 0) expect_at(bfull + 8 * s, bytes);
-                    tma_load_pair(base, &tm_w, bar, kc, n0, 0, 0);
-                    if (two) tma_load_pair(base + kPTileW, &tm_w, bar, kc, p.paired_I ? n0 : n0 + 256, p.paired_I ? 1 : 0, 0);
-                    tma_load_pair(base + 2 * kPTileW, &tm_x, bar, kc, m0, 0, 0);
+                    if (n >= S) {  // (the first ring's W is on its way)
+                        if (rank == 0) expect_at(bfull + 8 * s, bytes);
+                        load_w(base, bar, ks, n0, two);
+                    }
+                    tma_load_pair(base + 2 * kPTileW, &tm_x, bar, ks * kGemmBK, m0, 0, 0);
                 }
                 if (++s == static_cast<uint32_t>(S)) s = 0, ph ^= 1;
             }
@@ -660,6 +682,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
         float* stg = reinterpret_cast<float*>(epi) + (warp - 2) * 32 * kGStageLd;
         const int sub = lane >> 3, c4 = lane & 7;
         const uint32_t bae = dsmem_addr(smem_addr(acc_empty), 0);
+        const bool vec = (p.N & 3) == 0;  // whole groups of four columns, 8-byte aligned
+        pdl_wait();
         bool ok = true;
         uint32_t u = 0;
         for (int w = blockIdx.x / 2; ok && w < p.units; w += step, ++u) {
@@ -668,6 +692,28 @@ __global__ void __launch_bounds__(kPThreads, 1)
             const int chunks = (mend + 31) / 32;
             const int items = p.paired_I || !two_blocks(n0) ? chunks : 2 * chunks;
             const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
+            // What the output adds to is fetched ahead: the bias of both blocks now,
+            // an item's residual while the one before it is written.
+            const int ncol = n0 + rank * 128 + quad * 32 + 4 * c4;
+            float bias[2][4];
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int n = ncol + 256 * b + e;
+                    bias[b][e] = p.bias && n < p.N ? __bfloat162float(p.bias[n]) : 0.f;
+                }
+            uint2 old[8];
+            auto load_old = [&](int i) {
+                const int b = i >= chunks ? 1 : 0, c = i - b * chunks, n = ncol + 256 * b;
+                if (!p.add || !vec || i >= items || n >= p.N) return;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int r = 32 * c + 4 * q + sub;
+                    if (r < mend) old[q] = *reinterpret_cast<const uint2*>(p.D + static_cast<size_t>(m0 + r) * p.N + n);
+                }
+            };
+            load_old(half);
             ok = wait_warp(smem_addr(acc_full), u & 1, deadline);
             if (!ok) break;
             tc_fence_after();
@@ -700,8 +746,33 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
                     acc[q] = *reinterpret_cast<const float4*>(stg + (4 * q + sub) * kGStageLd + 4 * c4);
-                store_rows4(p, m0 + 32 * c, sub, min(32, mend - 32 * c), n0 + 256 * b + rank * 128 + quad * 32 + 4 * c4,
-                            acc);
+                const int n = ncol + 256 * b;
+                if (!vec) {
+                    store_rows4(p, m0 + 32 * c, sub, min(32, mend - 32 * c), n, acc);
+                } else if (n < p.N) {
+                    uint2 o[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        float f[4] = {acc[q].x, acc[q].y, acc[q].z, acc[q].w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) f[e] += b ? bias[1][e] : bias[0][e];
+                        if (p.add) {
+                            const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&old[q].x));
+                            const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&old[q].y));
+                            f[0] += lo.x;
+                            f[1] += lo.y;
+                            f[2] += hi.x;
+                            f[3] += hi.y;
+                        }
+                        o[q] = make_uint2(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]));
+                    }
+                    load_old(i + 2);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int r = 32 * c + 4 * q + sub;
+                        if (r < mend) *reinterpret_cast<uint2*>(p.D + static_cast<size_t>(m0 + r) * p.N + n) = o[q];
+                    }
+                }
                 __syncwarp();
             }
             if (!released && lane == 0) arrive_cluster(bae);  // a warp without a chunk
@@ -1201,13 +1272,15 @@ cudaError_t launch_gemm(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const 
         cfg.blockDim = dim3(kPThreads);
         cfg.dynamicSmemBytes = pair_smem(p.pair_bn);
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         return cudaLaunchKernelEx(&cfg, gemm_pair_tc, tm_x, tm_w, p);
     }
     const int grid = p.units < sms ? p.units : sms;
