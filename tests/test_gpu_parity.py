@@ -359,3 +359,65 @@ def test_split_attention_with_streams_at_different_frames():
     assert torch.isfinite(out).all() and torch.isfinite(imp).all()
     assert (out[1:].float() - out1.float()).abs().max().item() <= OUT_ATOL
     torch.testing.assert_close(imp[1:], imp1, rtol=IMP_RTOL, atol=IMP_ATOL)
+
+
+SELECT = {
+    # (shape, zero queries: importance ties by the hundred, frames)
+    "one_pass": (Shape(4, 2, 64, 16, 64, 8, num_layers=3, num_streams=2), False, 8),
+    "ties": (Shape(2, 2, 64, 48, 1500, 36), True, 36),
+    "ties_member_wise": (Shape(2, 1, 64, 33, 700, 25, num_layers=2), True, 25),
+    "large_member_wise": (Shape(2, 1, 128, 50, 3001, 62), False, 62),
+    "large_ties": (Shape(2, 2, 64, 100, 6000, 62), True, 62),
+    "large": (Shape(2, 2, 64, 200, 11000, 57, num_layers=2), False, 57),
+    "many_heads": (Shape(16, 16, 64, 100, 6000, 62), False, 62),
+}
+
+
+@pytest.mark.parametrize("selection", [0, 2])
+@pytest.mark.parametrize("name", sorted(SELECT))
+def test_selection_is_exact_for_the_exported_importance(name, selection):
+    """The kept positions, slot by slot: the B pool members largest in (importance,
+    earlier position), freed slots in ascending order taken by the admitted tokens
+    in ascending order.  The ranking is redone from the importance the step exports
+    (layer mode: summed over the heads in order, in fp32), so nothing is rounded."""
+    shape, zero_q, frames = SELECT[name]
+    S, L, H, T, B = (shape.num_streams, shape.num_layers, shape.num_kv_heads, shape.tokens_per_frame,
+                     shape.state_capacity)
+    eng = StateKV(make_config(shape, selection=selection))
+    for n in range(1, frames + 1):
+        q, k, v = batch_qkv(shape, n, streams=list(range(S)), layers=list(range(L)), device="cuda")
+        if zero_q:
+            q = torch.zeros_like(q)
+        imp = torch.full((S, L, H, B + T), float("nan"), device="cuda")
+        if n > frames - 3:
+            torch.cuda.synchronize()
+            before = [[eng.state(s, l)[2].cpu().numpy().copy() for l in range(L)] for s in range(S)]
+        assert eng.prefill_frame(q, k, v, torch.empty_like(q), imp) == 0
+        if n <= frames - 3:
+            continue
+        torch.cuda.synchronize()
+        count = min(B, (n - 1) * T)
+        imps = imp.cpu().numpy()
+        for s in range(S):
+            for l in range(L):
+                after = eng.state(s, l)[2].cpu().numpy()
+                for h in range(H):
+                    x = imps[s, l, h]
+                    if selection == 2:
+                        x = np.zeros(B + T, np.float32)
+                        for h2 in range(H):
+                            x = x + imps[s, l, h2]
+                    pos = np.concatenate([before[s][l][h][:count], (n - 1) * T + np.arange(T)]).astype(np.int64)
+                    sc = np.concatenate([x[:count], x[B:]])
+                    kept = np.zeros(count + T, bool)
+                    kept[np.lexsort((pos, -sc))[:B]] = True
+                    want = np.full(B, -1, np.int64)
+                    want[:count] = pos[:count]
+                    free = [i for i in range(B) if i >= count or not kept[i]]
+                    adm = [t for t in range(T) if kept[count + t]]
+                    for i, t in zip(free, adm):
+                        want[i] = (n - 1) * T + t
+                    live = min(B, count + T)
+                    got = after[h].astype(np.int64)
+                    assert (got[:live] == want[:live]).all(), (name, n, s, l, h)
+    assert eng.sync() == 0
