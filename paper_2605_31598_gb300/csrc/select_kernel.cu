@@ -70,6 +70,9 @@ __device__ __forceinline__ int block_exclusive_scan(int x, int* warp_sums, int& 
 // For each of kMem pool members (columns col[e], active act[e]): the sum of
 // x[mt * stride + col] over mt < MT, added in mt order.  Twelve tiles' loads of
 // all members (24 independent loads) are in flight before any addition.
+// (Plain loads: the kernel is resident while the attention kernel still writes
+// the partials, so the read-only path, which may move a load ahead of the wait, is
+// not for them.)
 constexpr int kMem = 2;
 __device__ __forceinline__ void tiles_sum(const float* x, int MT, int stride, const int (&col)[kMem],
                                           const bool (&act)[kMem], float (&s)[kMem])
@@ -83,7 +86,7 @@ __device__ __forceinline__ void tiles_sum(const float* x, int MT, int stride, co
         for (int m = 0; m < 12; ++m)
 #pragma unroll
             for (int e = 0; e < kMem; ++e)
-                v[m][e] = (act[e] && mt + m < MT) ? __ldg(x + static_cast<size_t>(mt + m) * stride + col[e]) : 0.f;
+                v[m][e] = (act[e] && mt + m < MT) ? x[static_cast<size_t>(mt + m) * stride + col[e]] : 0.f;
 #pragma unroll
         for (int m = 0; m < 12; ++m)
 #pragma unroll
@@ -104,7 +107,7 @@ __device__ __forceinline__ float4 rows_sum4(const float* x, int MT, int stride, 
         float4 v[12];
 #pragma unroll
         for (int m = 0; m < 12; ++m)
-            v[m] = mt + m < MT ? __ldg(reinterpret_cast<const float4*>(x + static_cast<size_t>(mt + m) * stride + c0))
+            v[m] = mt + m < MT ? *reinterpret_cast<const float4*>(x + static_cast<size_t>(mt + m) * stride + c0)
                                : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int m = 0; m < 12; ++m)
