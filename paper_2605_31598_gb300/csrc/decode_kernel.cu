@@ -27,8 +27,9 @@
 // four KV heads and 12.5k rows, 3.8 us of HBM time -- so what bounds it is the
 // chain of latencies.  As four launches (append, partial, a combine of one
 // thread per output element and chunk-serial loads, counter) it took 51 us per
-// layer, 38 of them in the combine; this one takes 13.5 (5.3 of them the copies,
-// 4 the merge across CTAs).
+// layer, 38 of them in the combine; this one takes 12.7 (13.5 before the keys were
+// requested into L2 ahead of the previous layer's end; 5.3 of these were the
+// copies, 4 the merge across CTAs).
 // Every wait is bounded by the watchdog.
 #include "sm103_ptx.cuh"
 #include "statekv_kernels.cuh"
@@ -148,8 +149,22 @@ __global__ void __launch_bounds__(kDecThreads)
         }
     }
     __syncwarp();
+    // The CTA's keys are requested into L2 while the stream's previous kernel ends
+    // (a decoder's layers follow one another: most SMs idle while the last CTAs of the
+    // previous layer merge their chunks).  The counters may be about to change, and
+    // rows about to be written: this is a hint within the cache, and L2 is where
+    // later writes land and the copies below read.  A lane takes 32 keys of K and V.
+    if (p.prefetch) {
+        const int hint = min(static_cast<long long>(__ldcg(p.frames + head)) * p.T + __ldcg(p.text + head), p.cap);
+        for (int k = chunk * p.ck + 32 * static_cast<int>(threadIdx.x); k < min(hint, (chunk + 1) * p.ck);
+             k += 32 * kDecThreads) {
+            const uint32_t bytes = min(32, min(hint, (chunk + 1) * p.ck) - k) * D * 2;
+            bulk_prefetch_l2(p.cache_k + (head * p.cap + k) * D, bytes);
+            bulk_prefetch_l2(p.cache_v + (head * p.cap + k) * D, bytes);
+        }
+    }
     // everything above overlaps the end of the stream's previous kernel
-    // (programmatic launch); nothing it wrote is read before this wait
+    // (programmatic launch); nothing it wrote is used before this wait
     pdl_wait();
     pdl_launch_dependents();
     const int len0 = p.frames[head] * p.T + p.text[head];  // rows before the new tokens

@@ -148,6 +148,12 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
                  :: "r"(smem_addr(sdst)), "l"(gsrc), "r"(bytes), "r"(smem_addr(bar)) : "memory");
 }
 
+// global -> L2 prefetch of `bytes` (a multiple of 16, 16-byte aligned); nothing waits for it
+__device__ __forceinline__ void bulk_prefetch_l2(const void* gsrc, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gsrc), "r"(bytes) : "memory");
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap)
 {

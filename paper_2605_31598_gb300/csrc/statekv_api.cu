@@ -492,6 +492,7 @@ statekv_status run_decode(statekv_handle* h, const statekv_decode_args& a, cudaS
                     dp.nchunk = static_cast<int>(used);
                 }
             }
+            dp.prefetch = units * dp.nchunk <= sms;  // (further waves stream from HBM as it is)
         }
         dp.q = static_cast<const __nv_bfloat16*>(a.q);
         dp.out = static_cast<__nv_bfloat16*>(a.out);

@@ -288,6 +288,7 @@ struct DecodeParams {
     int n, G, Hq, Hkv, T;
     long long cap;
     int ck, nchunk;             // keys per chunk (a multiple of 128), chunks
+    int prefetch;               // 1: request the chunk's rows into L2 ahead of the previous kernel's end
     float scale_log2;
     int32_t* status;
     unsigned long long watchdog_ns;
