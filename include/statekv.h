@@ -205,6 +205,21 @@ statekv_status statekv_state_metrics(const uint8_t* mask_n, const uint8_t* mask_
                                      int32_t T, int64_t row_stride, double* out,
                                      statekv_stream stream);
 
+/* The same statistics from scores, the top-B sets included, in one and two
+ * kernels.  Results equal those of the calls above, bit for bit.
+ * topb_concentration: out fp64 [count][rows][2] (device), for each of `count`
+ *   budgets (host array, read before the call returns; each >= 0) the sums of
+ *   statekv_concentration_sums over that budget's top-B of scores[r][0 .. n).
+ * topb_metrics: S_n from scores_n[r][0 .. n_seen), S_n1 from
+ *   scores_n1[r][0 .. n_seen + T), both fp32 [rows][row_stride]; masks uint8
+ *   [2][rows][row_stride] (device) receives both, out is as above. */
+statekv_status statekv_topb_concentration(const float* scores, int32_t rows, int64_t n, int64_t row_stride,
+                                          const int64_t* budgets, int32_t count, double* out,
+                                          statekv_stream stream);
+statekv_status statekv_topb_metrics(const float* scores_n, const float* scores_n1, int32_t rows, int64_t n_seen,
+                                    int32_t T, int64_t row_stride, int64_t B, uint8_t* masks, double* out,
+                                    statekv_stream stream);
+
 /* ---- Full per-frame transformer block ----------------------------------
  * One frame of every layer of a Qwen2-style decoder around the StateKV step,
  * layers in order (layer l + 1 reads layer l's output), per layer:

@@ -119,14 +119,47 @@ __device__ __forceinline__ void red_dsmem_add(uint32_t addr, unsigned v)
     asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
+// The cluster's partial sums, one set per CTA, added in rank order by the first.
+template <int K>
+__device__ void cluster_total(const double (&v)[K], double* sh, int r, int C, double* out)
+{
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int i = 0; i < K; ++i) sh[i] = v[i];
+    ptx::cluster_sync();
+    if (r == 0 && threadIdx.x < K) {
+        double t = 0.0;
+        for (int q = 0; q < C; ++q)
+            t += ld_dsmem_f64(ptx::dsmem_addr(ptx::smem_addr(sh + threadIdx.x), q));
+        out[threadIdx.x] = t;
+    }
+    ptx::cluster_sync();
+}
+
 constexpr int kTopbBins = 2048;
+
+// The calls of one launch, blockIdx.y each.
+constexpr int kTopbJobs = 16;
+struct TopbJobs {
+    struct {
+        const float* scores;
+        uint8_t* mask;
+        long long n, B;
+    } job[kTopbJobs];
+};
 
 // One cluster of C CTAs per row.  Every pass, each CTA counts its share's digits,
 // adds the non-empty bins to the first CTA's counts of that pass, and finds the
-// bin of the k-th largest key in the merged counts.
-__global__ void __launch_bounds__(kDiagThreads) topb_mask_kernel(const float* scores, long long n,
-                                                                 long long stride, long long B,
-                                                                 uint8_t* mask, int C)
+// bin of the k-th largest key in the merged counts.  The result is the mask, or
+// (kSums) the two sums of concentration_kernel over it, taken from the registers
+// that hold the row: same order, same bits, no mask written or read.  Several
+// budgets, or the two frames of the state metrics, go in one launch: 28 rows on
+// eight CTAs each leave half of the thread slots idle.  Mask, concentration at two
+// budgets and state metrics of 28 rows of 25k: nine launches 248 us, four 204 (what
+// is left is mostly the host's: two copies of results and the calls).
+template <bool kSums>
+__global__ void __launch_bounds__(kDiagThreads) topb_kernel(const __grid_constant__ TopbJobs jobs,
+                                                            long long stride, double* out, int C)
 {
     __shared__ __align__(16) unsigned hist[kTopbBins], merged[3][kTopbBins];
     __shared__ unsigned wsum[kDiagWarps];
@@ -134,17 +167,20 @@ __global__ void __launch_bounds__(kDiagThreads) topb_mask_kernel(const float* sc
     __shared__ unsigned long long sh_k;
     const int r = blockIdx.x % C, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long rowi = blockIdx.x / C;
-    const float* row = scores + static_cast<size_t>(rowi) * stride;
-    uint8_t* mrow = mask + static_cast<size_t>(rowi) * stride;
+    const long long n = jobs.job[blockIdx.y].n, B = jobs.job[blockIdx.y].B;
+    const float* row = jobs.job[blockIdx.y].scores + static_cast<size_t>(rowi) * stride;
+    uint8_t* mrow = kSums ? nullptr : jobs.job[blockIdx.y].mask + static_cast<size_t>(rowi) * stride;
     long long lo, hi;
     row_share(n, r, C, lo, hi);
     // this thread's entries base + tid + e kDiagThreads of a batch, as score bits
+    // (kSums: as they are, for the sums)
     unsigned x[kDiagBatch] = {};
+    auto bits = [](unsigned v) { return kSums ? score_bits(__uint_as_float(v)) : v; };
     auto load = [&](long long base) {
 #pragma unroll
         for (int e = 0; e < kDiagBatch; ++e) {
             const long long i = base + tid + e * kDiagThreads;
-            x[e] = i < hi ? score_bits(row[i]) : 0u;
+            x[e] = i >= hi ? 0u : kSums ? __float_as_uint(row[i]) : score_bits(row[i]);
         }
     };
     constexpr long long kStep = kDiagBatch * kDiagThreads;
@@ -167,8 +203,8 @@ __global__ void __launch_bounds__(kDiagThreads) topb_mask_kernel(const float* sc
                 if (!cached) load(base);
 #pragma unroll
                 for (int e = 0; e < kDiagBatch; ++e)
-                    if (base + tid + e * kDiagThreads < hi && (x[e] & tmask) == thr)
-                        atomicAdd(&hist[(x[e] >> shift) & dmask], 1u);
+                    if (base + tid + e * kDiagThreads < hi && (bits(x[e]) & tmask) == thr)
+                        atomicAdd(&hist[(bits(x[e]) >> shift) & dmask], 1u);
             }
             __syncthreads();
             const uint32_t m0 = ptx::dsmem_addr(ptx::smem_addr(merged[pass]), 0);
@@ -223,12 +259,13 @@ __global__ void __launch_bounds__(kDiagThreads) topb_mask_kernel(const float* sc
     }
     // kept(j) <=> j < n and key(j) above the threshold, or equal and in time
     unsigned long long seen = 0;  // equal entries of this CTA's earlier batches
+    double top = 0.0, rest = 0.0;
     for (long long base = lo; base < hi; base += kStep) {
-        if (!none && !all && !cached) load(base);
+        if (none || all ? kSums : !cached) load(base);
 #pragma unroll
         for (int e = 0; e < kDiagBatch; ++e) {
             const long long i = base + tid + e * kDiagThreads;
-            const unsigned d = x[e] & tmask;
+            const unsigned d = bits(x[e]) & tmask;
             bool keep = all || d > thr || (d == thr && ties == ~0ull);
             if (ties != ~0ull) {  // rank of the equal entries, in position order (uniform branch)
                 const bool eq = i < hi && d == thr;
@@ -245,29 +282,27 @@ __global__ void __launch_bounds__(kDiagThreads) topb_mask_kernel(const float* sc
                 __syncthreads();
                 if (eq) keep = rank < ties;
             }
-            if (i < hi) mrow[i] = !none && keep ? 1 : 0;
+            if constexpr (kSums) {
+                const bool in = i < hi && !none && keep;
+                const double t = (in ? top : rest) + __uint_as_float(x[e]);
+                top = in ? t : top;
+                rest = in ? rest : t;
+            } else if (i < hi) {
+                mrow[i] = !none && keep ? 1 : 0;
+            }
         }
+    }
+    if constexpr (kSums) {
+        __shared__ double sh[2 * kDiagWarps], part[2];
+        double v[2] = {};
+        block_sum2(top, rest, sh, v);
+        v[1] += v[0];
+        cluster_total(v, part, r, C, out + 2 * (blockIdx.y * static_cast<size_t>(gridDim.x / C) + rowi));
+        return;
     }
     long long t0, t1;  // entries past n
     row_share(stride - n, r, C, t0, t1);
     for (long long j = n + t0 + tid; j < n + t1; j += kDiagThreads) mrow[j] = 0;
-}
-
-// The cluster's partial sums, one set per CTA, added in rank order by the first.
-template <int K>
-__device__ void cluster_total(const double (&v)[K], double* sh, int r, int C, double* out)
-{
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int i = 0; i < K; ++i) sh[i] = v[i];
-    ptx::cluster_sync();
-    if (r == 0 && threadIdx.x < K) {
-        double t = 0.0;
-        for (int q = 0; q < C; ++q)
-            t += ld_dsmem_f64(ptx::dsmem_addr(ptx::smem_addr(sh + threadIdx.x), q));
-        out[threadIdx.x] = t;
-    }
-    ptx::cluster_sync();
 }
 
 __global__ void __launch_bounds__(kDiagThreads) concentration_kernel(const float* scores,
@@ -355,7 +390,8 @@ __global__ void __launch_bounds__(kDiagThreads) state_metrics_kernel(
 // CTAs per row, a power of two up to 8 (the portable cluster size): no more than
 // give each about 2048 entries, and none added once the rows alone fill the SMs
 // twice.  28 rows of 25k scores: 50 us on one CTA
-// per row, 16 on eight (top-B).
+// per row, 16 on eight (top-B).  (Several jobs a launch keep the C of one, so the
+// sums do too.)
 int row_cluster(int rows, long long n)
 {
     int C = 1;
@@ -364,10 +400,10 @@ int row_cluster(int rows, long long n)
 }
 
 template <class... KArgs, class... Args>
-cudaError_t launch_rows(void (*kernel)(KArgs...), int rows, int C, cudaStream_t st, Args... args)
+cudaError_t launch_rows(void (*kernel)(KArgs...), int rows, int jobs, int C, cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(rows) * C);
+    cfg.gridDim = dim3(static_cast<unsigned>(rows) * C, static_cast<unsigned>(jobs));
     cfg.blockDim = dim3(kDiagThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -394,14 +430,46 @@ cudaError_t launch_topb_mask(const float* scores, int rows, long long n, long lo
                              long long B, uint8_t* mask, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    return launch_rows(topb_mask_kernel, rows, row_cluster(rows, n), st, scores, n, stride, B, mask);
+    TopbJobs jobs{};
+    jobs.job[0] = {scores, mask, n, B};
+    return launch_rows(topb_kernel<false>, rows, 1, row_cluster(rows, n), st, jobs, stride,
+                       static_cast<double*>(nullptr));
+}
+
+cudaError_t launch_topb_concentration(const float* scores, int rows, long long n, long long stride,
+                                      const int64_t* budgets, int count, double* out, cudaStream_t st)
+{
+    if (rows <= 0) return cudaSuccess;
+    for (int b0 = 0; b0 < count; b0 += kTopbJobs) {
+        const int nb = count - b0 < kTopbJobs ? count - b0 : kTopbJobs;
+        TopbJobs jobs{};
+        for (int i = 0; i < nb; ++i) jobs.job[i] = {scores, nullptr, n, budgets[b0 + i]};
+        const cudaError_t e = launch_rows(topb_kernel<true>, rows, nb, row_cluster(rows, n), st, jobs, stride,
+                                          out + static_cast<size_t>(b0) * rows * 2);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_topb_metrics(const float* scores_n, const float* scores_n1, int rows, long long n_seen, int T,
+                                long long stride, long long B, uint8_t* mask_n, uint8_t* mask_n1, double* out,
+                                cudaStream_t st)
+{
+    if (rows <= 0) return cudaSuccess;
+    TopbJobs jobs{};
+    jobs.job[0] = {scores_n, mask_n, n_seen, B};
+    jobs.job[1] = {scores_n1, mask_n1, n_seen + T, B};
+    const cudaError_t e = launch_rows(topb_kernel<false>, rows, 2, row_cluster(rows, n_seen + T), st, jobs, stride,
+                                      static_cast<double*>(nullptr));
+    return e != cudaSuccess ? e
+                            : launch_state_metrics(mask_n, mask_n1, scores_n1, rows, n_seen, T, stride, out, st);
 }
 
 cudaError_t launch_concentration(const float* scores, const uint8_t* mask, int rows, long long n,
                                  long long stride, double* out, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    return launch_rows(concentration_kernel, rows, row_cluster(rows, n), st, scores, mask, n, stride, out);
+    return launch_rows(concentration_kernel, rows, 1, row_cluster(rows, n), st, scores, mask, n, stride, out);
 }
 
 cudaError_t launch_state_metrics(const uint8_t* mask_n, const uint8_t* mask_n1, const float* w,
@@ -409,7 +477,7 @@ cudaError_t launch_state_metrics(const uint8_t* mask_n, const uint8_t* mask_n1, 
                                  cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    return launch_rows(state_metrics_kernel, rows, row_cluster(rows, n_seen + T), st, mask_n, mask_n1, w,
+    return launch_rows(state_metrics_kernel, rows, 1, row_cluster(rows, n_seen + T), st, mask_n, mask_n1, w,
                        n_seen, T, stride, out);
 }
 

@@ -798,6 +798,36 @@ statekv_status statekv_state_metrics(const uint8_t* mask_n, const uint8_t* mask_
     return STATEKV_OK;
 }
 
+statekv_status statekv_topb_concentration(const float* scores, int32_t rows, int64_t n, int64_t row_stride,
+                                          const int64_t* budgets, int32_t count, double* out,
+                                          statekv_stream stream)
+{
+    if (!scores || !out || !budgets || !aligned(scores, 4) || !aligned(out, 8) || rows < 0 || n < 0 ||
+        row_stride < n || row_stride > (1ll << 31) || count < 0)
+        return STATEKV_ERR_INVALID_ARG;
+    for (int32_t i = 0; i < count; ++i)
+        if (budgets[i] < 0) return STATEKV_ERR_INVALID_ARG;
+    if (launch_topb_concentration(scores, rows, n, row_stride, budgets, count, out,
+                                  reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
+        return STATEKV_ERR_CUDA;
+    return STATEKV_OK;
+}
+
+statekv_status statekv_topb_metrics(const float* scores_n, const float* scores_n1, int32_t rows, int64_t n_seen,
+                                    int32_t T, int64_t row_stride, int64_t B, uint8_t* masks, double* out,
+                                    statekv_stream stream)
+{
+    if (!scores_n || !scores_n1 || !masks || !out || !aligned(scores_n, 4) || !aligned(scores_n1, 4) ||
+        !aligned(out, 8) || rows < 0 || n_seen < 0 || T < 0 || n_seen > row_stride || T > row_stride - n_seen ||
+        row_stride > (1ll << 31) || B < 0)
+        return STATEKV_ERR_INVALID_ARG;
+    if (launch_topb_metrics(scores_n, scores_n1, rows, n_seen, T, row_stride, B, masks,
+                            masks + static_cast<size_t>(rows) * row_stride, out,
+                            reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
+        return STATEKV_ERR_CUDA;
+    return STATEKV_OK;
+}
+
 namespace {
 
 // Workspace carve-up of one block call (all offsets 256-byte aligned).

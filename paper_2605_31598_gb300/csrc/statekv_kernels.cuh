@@ -151,6 +151,11 @@ struct ScoresParams {
 
 // App. A diagnostics (diag_kernel.cu).
 cudaError_t launch_scores_reduce(const ScoresParams& p, int U, cudaStream_t st);
+cudaError_t launch_topb_concentration(const float* scores, int rows, long long n, long long stride,
+                                      const int64_t* budgets, int count, double* out, cudaStream_t st);
+cudaError_t launch_topb_metrics(const float* scores_n, const float* scores_n1, int rows, long long n_seen, int T,
+                                long long stride, long long B, uint8_t* mask_n, uint8_t* mask_n1, double* out,
+                                cudaStream_t st);
 cudaError_t launch_topb_mask(const float* scores, int rows, long long n, long long stride,
                              long long B, uint8_t* mask, cudaStream_t st);
 cudaError_t launch_concentration(const float* scores, const uint8_t* mask, int rows, long long n,

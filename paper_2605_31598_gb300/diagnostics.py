@@ -6,14 +6,14 @@ the heads), the concentration C_{n,B} of historical attention in the top-B
 historical tokens (App. A.1), and the candidate-pool recall, weighted recall,
 retention and churn of consecutive top-B oracle states (App. A.2).  The sums
 and the top-B sets are computed by the library's kernels
-(``statekv_topb_mask``, ``statekv_concentration_sums``,
-``statekv_state_metrics``); this module passes device pointers and divides the
+(``statekv_topb_mask``, ``statekv_topb_concentration``,
+``statekv_topb_metrics``); this module passes device pointers and divides the
 returned sums.
 """
 from __future__ import annotations
 
-from .statekv import (check, statekv_concentration_sums, statekv_state_metrics,
-                      statekv_topb_mask)
+from .statekv import (check, statekv_state_metrics, statekv_topb_concentration,
+                      statekv_topb_mask, statekv_topb_metrics)
 
 
 def _stream(stream):
@@ -43,11 +43,10 @@ def concentration(scores, n_hist: int, budgets, *, stream=None):
 
     rows, stride = scores.shape
     out = torch.empty((len(budgets), rows, 2), dtype=torch.float64, device=scores.device)
-    for i, B in enumerate(budgets):
-        mask = topb_mask(scores, n_hist, B, stream=stream)
-        check(statekv_concentration_sums(scores.data_ptr(), mask.data_ptr(), rows, n_hist, stride,
-                                         out[i].data_ptr(), _stream(stream)),
-              "statekv_concentration_sums")
+    if len(budgets):
+        check(statekv_topb_concentration(scores.data_ptr(), rows, n_hist, stride, budgets,
+                                         out.data_ptr(), _stream(stream)),
+              "statekv_topb_concentration")
     o = out.cpu().numpy()
     return (o[:, :, 0] / o[:, :, 1]).T.copy()
 
@@ -60,12 +59,18 @@ def state_metrics(scores_n, scores_next, n_seen: int, T: int, B: int, *, stream=
     import torch
 
     rows, stride = scores_next.shape
-    s_n = topb_mask(scores_n, n_seen, B, stream=stream)
-    s_next = topb_mask(scores_next, n_seen + T, B, stream=stream)
     out = torch.empty((rows, 6), dtype=torch.float64, device=scores_next.device)
-    check(statekv_state_metrics(s_n.data_ptr(), s_next.data_ptr(), scores_next.data_ptr(), rows,
-                                n_seen, T, stride, out.data_ptr(), _stream(stream)),
-          "statekv_state_metrics")
+    if scores_n.shape == scores_next.shape:
+        masks = torch.empty((2, rows, stride), dtype=torch.uint8, device=scores_next.device)
+        check(statekv_topb_metrics(scores_n.data_ptr(), scores_next.data_ptr(), rows, n_seen, T,
+                                   stride, B, masks.data_ptr(), out.data_ptr(), _stream(stream)),
+              "statekv_topb_metrics")
+    else:
+        s_n = topb_mask(scores_n, n_seen, B, stream=stream)
+        s_next = topb_mask(scores_next, n_seen + T, B, stream=stream)
+        check(statekv_state_metrics(s_n.data_ptr(), s_next.data_ptr(), scores_next.data_ptr(), rows,
+                                    n_seen, T, stride, out.data_ptr(), _stream(stream)),
+              "statekv_state_metrics")
     o = out.cpu().numpy()
     return {
         "recall": o[:, 0] / o[:, 1],

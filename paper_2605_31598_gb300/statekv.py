@@ -33,6 +33,7 @@ EXPORTED = ("statekv_arena_bytes", "statekv_init", "statekv_prefill_frame",
             "statekv_debug_check",
             "statekv_scores_workspace_bytes", "statekv_full_attention_scores",
             "statekv_topb_mask", "statekv_concentration_sums", "statekv_state_metrics",
+            "statekv_topb_concentration", "statekv_topb_metrics",
             "statekv_block_workspace_bytes", "statekv_block_frame",
             "statekv_destroy", "statekv_status_string")
 
@@ -165,6 +166,14 @@ def lib() -> ctypes.CDLL:
                                                 ctypes.c_int32, ctypes.c_int64, ctypes.c_int32,
                                                 ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p]
             L.statekv_state_metrics.restype = st
+            L.statekv_topb_concentration.argtypes = [
+                ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_int64,
+                P(ctypes.c_int64), ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p]
+            L.statekv_topb_concentration.restype = st
+            L.statekv_topb_metrics.argtypes = [
+                ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_int32,
+                ctypes.c_int64, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
+            L.statekv_topb_metrics.restype = st
             L.statekv_block_workspace_bytes.argtypes = [ctypes.c_void_p, P(statekv_block_config),
                                                         ctypes.c_int32, P(ctypes.c_size_t)]
             L.statekv_block_workspace_bytes.restype = st
@@ -305,6 +314,20 @@ def statekv_state_metrics(mask_n: int, mask_n1: int, scores_n1: int, rows: int, 
     return lib().statekv_state_metrics(ctypes.c_void_p(mask_n), ctypes.c_void_p(mask_n1),
                                        ctypes.c_void_p(scores_n1), rows, n_seen, T, row_stride,
                                        ctypes.c_void_p(out), ctypes.c_void_p(stream))
+
+
+def statekv_topb_concentration(scores: int, rows: int, n: int, row_stride: int, budgets, out: int,
+                               stream: int) -> int:
+    b = (ctypes.c_int64 * len(budgets))(*budgets)
+    return lib().statekv_topb_concentration(ctypes.c_void_p(scores), rows, n, row_stride, b, len(b),
+                                            ctypes.c_void_p(out), ctypes.c_void_p(stream))
+
+
+def statekv_topb_metrics(scores_n: int, scores_n1: int, rows: int, n_seen: int, T: int,
+                         row_stride: int, B: int, masks: int, out: int, stream: int) -> int:
+    return lib().statekv_topb_metrics(ctypes.c_void_p(scores_n), ctypes.c_void_p(scores_n1), rows,
+                                      n_seen, T, row_stride, B, ctypes.c_void_p(masks),
+                                      ctypes.c_void_p(out), ctypes.c_void_p(stream))
 
 
 def statekv_block_workspace_bytes(handle: int, bc: statekv_block_config, stream_count: int) -> int:

@@ -121,3 +121,17 @@ def test_diagnostics_arguments_rejected_on_host(lib):
     assert lib.statekv_full_attention_scores(None, None, None, None, 0, None) == 1
     n = ctypes.c_size_t(0)
     assert lib.statekv_scores_workspace_bytes(None, 1, 1, ctypes.byref(n)) == 1
+
+
+def test_fused_diagnostics_arguments_rejected_on_host(lib):
+    """As above, for the calls that make their own top-B sets."""
+    fake = 1 << 20  # 16-byte aligned, never touched
+    conc, metrics = statekv.statekv_topb_concentration, statekv.statekv_topb_metrics
+    assert conc(0, 1, 10, 16, [4], fake, 0) == 1            # null scores
+    assert conc(fake, 1, 10, 16, [4], 0, 0) == 1            # null out
+    assert conc(fake, 1, 20, 16, [4], fake, 0) == 1         # n > row_stride
+    assert conc(fake, 1, 10, 16, [4, -1], fake, 0) == 1     # a budget < 0
+    assert conc(fake, 1, 10, 16, [4], fake + 4, 0) == 1     # misaligned
+    assert metrics(fake, fake, 1, 10, 7, 16, 4, fake, fake, 0) == 1   # n_seen + T > row_stride
+    assert metrics(fake, fake, 1, 10, 6, 16, -1, fake, fake, 0) == 1  # B < 0
+    assert metrics(fake, fake, 1, 10, 6, 16, 4, 0, fake, 0) == 1      # null masks

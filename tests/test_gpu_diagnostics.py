@@ -16,7 +16,7 @@ import torch
 
 import oracle
 from paper_2605_31598_gb300 import StateKV, make_config
-from paper_2605_31598_gb300 import diagnostics
+from paper_2605_31598_gb300 import diagnostics, statekv
 from paper_2605_31598_gb300.inputs import WORKLOADS, batch_qkv
 
 from .parity import IMP_ATOL, IMP_RTOL, OUT_ATOL
@@ -183,3 +183,40 @@ def test_row_kernels_over_cluster_sizes(rows, n, stride):
                                     plain[r, ::-1][:n].astype(np.float64), n // 9)
         for key in want:
             assert m[key][r] == pytest.approx(want[key], rel=1e-12), (key, r)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,n,stride", [(1, 0, 3), (3, 1000, 1100), (2, 16390, 16391), (1, 70001, 70500)])
+def test_fused_statistics_equal_the_separate_kernels(rows, n, stride):
+    """Sums of top-B sets that were never written out, and two masks of one
+    launch: the same bits as mask and sum kernels one after the other, with
+    ties, negative entries (rank 0, summed as they are) and more budgets than
+    one launch takes."""
+    _need_gpu()
+    rng = np.random.default_rng(rows + n)
+    vals = (rng.integers(0, 9, size=(rows, stride)) / 3.0).astype(np.float32)
+    vals[:, ::2] = np.exp(rng.standard_normal(vals[:, ::2].shape))
+    vals[0, ::5] = -1.0
+    g = torch.as_tensor(vals, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    budgets = [0, 1, n // 9, n, n + 5] + [7 * i + 2 for i in range(13)]
+    got = torch.empty((len(budgets), rows, 2), dtype=torch.float64, device="cuda")
+    assert statekv.statekv_topb_concentration(g.data_ptr(), rows, n, stride, budgets, got.data_ptr(), stream) == 0
+    want = torch.empty_like(got)
+    for i, B in enumerate(budgets):
+        mask = diagnostics.topb_mask(g, n, B)
+        assert statekv.statekv_concentration_sums(g.data_ptr(), mask.data_ptr(), rows, n, stride,
+                                                  want[i].data_ptr(), stream) == 0
+    assert torch.equal(got, want)
+    seen, T = n - n // 9, n // 9
+    other = g.flip(1).contiguous()
+    for B in [0, max(1, n // 7)]:
+        masks = torch.empty((2, rows, stride), dtype=torch.uint8, device="cuda")
+        out, ref = (torch.empty((rows, 6), dtype=torch.float64, device="cuda") for _ in range(2))
+        assert statekv.statekv_topb_metrics(g.data_ptr(), other.data_ptr(), rows, seen, T, stride, B,
+                                            masks.data_ptr(), out.data_ptr(), stream) == 0
+        a, b = diagnostics.topb_mask(g, seen, B), diagnostics.topb_mask(other, seen + T, B)
+        assert torch.equal(masks[0], a) and torch.equal(masks[1], b)
+        assert statekv.statekv_state_metrics(a.data_ptr(), b.data_ptr(), other.data_ptr(), rows, seen, T,
+                                             stride, ref.data_ptr(), stream) == 0
+        assert torch.equal(out, ref)
