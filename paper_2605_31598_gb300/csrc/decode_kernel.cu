@@ -159,8 +159,8 @@ __global__ void __launch_bounds__(kDecThreads)
         for (int k = chunk * p.ck + 32 * static_cast<int>(threadIdx.x); k < min(hint, (chunk + 1) * p.ck);
              k += 32 * kDecThreads) {
             const uint32_t bytes = min(32, min(hint, (chunk + 1) * p.ck) - k) * D * 2;
-            bulk_prefetch_l2(p.cache_k + (head * p.cap + k) * D, bytes);
-            bulk_prefetch_l2(p.cache_v + (head * p.cap + k) * D, bytes);
+            prefetch_l2(p.cache_k + (head * p.cap + k) * D, bytes);
+            prefetch_l2(p.cache_v + (head * p.cap + k) * D, bytes);
         }
     }
     // everything above overlaps the end of the stream's previous kernel

@@ -2,7 +2,8 @@
 //     (Sec. 3.3, Eq. 6; per layer and KV head as in App. A).
 // K4: decode-cache append (Sec. 3.2 detailed state; Sec. 3.3 "append").
 //
-// K3 runs one CTA per (unit, KV head), and in the same launch a few CTAs per unit
+// K3 runs one CTA per (unit, KV head) (a cluster for the sums of large pools, see
+// select_split), and in the same launch a few CTAs per unit
 // that append the frame's K and V to the decode cache (K4's work).  It is launched
 // programmatically behind the attention kernel: it is in place when that ends, and
 // the append, which needs nothing of the attention kernel's, takes the SMs that
@@ -167,10 +168,14 @@ __device__ __forceinline__ void finish_unit(const SelectParams& p, int u, int nf
         for (int h = threadIdx.x; h < p.Hkv; h += kSelThreads) p.frames[base + h] = nf + 1;
 }
 
+constexpr int kMaxSelSplit = 8;
 constexpr int kBins = 2048;   // radix digits of 11 bits
 constexpr int kDirect = 256;  // candidates ranked by counting instead of another pass
 static_assert(kBins / 4 <= kSelThreads && kBins % 128 == 0, "four bins per thread, whole warps");
 
+// kSplit: a cluster of p.split CTAs makes the keys of a head, each from its share of
+// the pool's columns; they meet in the first CTA's shared memory, which goes on alone.
+template <bool kSplit>
 __global__ void __launch_bounds__(kSelThreads)
     state_select_gather(const SelectParams p)
 {
@@ -189,6 +194,8 @@ __global__ void __launch_bounds__(kSelThreads)
         finish_unit(p, u, nf0);
         return;
     }
+    const int C = kSplit ? p.split : 1, rank = kSplit ? static_cast<int>(ptx::cluster_ctarank()) : 0;
+    if (kSplit) ptx::cluster_sync();  // the cluster's CTAs run: their shared memory can be written
     ptx::pdl_wait();  // the attention kernel's partials; it has read the state
     const int T = p.T, B = p.B, P = p.P, D = p.D;
     uint64_t* key = reinterpret_cast<uint64_t*>(smem_raw);            // [P]
@@ -201,9 +208,10 @@ __global__ void __launch_bounds__(kSelThreads)
     __shared__ int warp_sums[kSelWarps + 1];
     __shared__ unsigned long long sh_prefix, sh_mask;
     __shared__ int sh_k, sh_in, sh_shift, sh_ncand;
-    __shared__ unsigned long long warp_and[kSelWarps], warp_or[kSelWarps];
+    constexpr int kMaxC = kSplit ? kMaxSelSplit : 1;
+    __shared__ unsigned long long warp_and[kMaxC * kSelWarps], warp_or[kMaxC * kSelWarps];
 
-    const int unit_head = blockIdx.x - p.U * p.appenders, u = unit_head / p.Hkv, hkv = unit_head - u * p.Hkv;
+    const int unit_head = (blockIdx.x - p.U * p.appenders) / C, u = unit_head / p.Hkv, hkv = unit_head - u * p.Hkv;
     const int ua = p.units.unit_abs(u);
     const int tid = threadIdx.x, lane = tid & 31;
     const size_t head = static_cast<size_t>(ua) * p.Hkv + hkv;
@@ -218,9 +226,17 @@ __global__ void __launch_bounds__(kSelThreads)
     // the counters come from the arena: a state larger than B or a negative frame
     // count would index past the pool (uniform across the CTA)
     if (!SKV_CHECK(count >= 0 && count <= B && nf >= 0, p.status, 1)) {
-        finish_unit(p, u, nf);
+        if (rank == 0) finish_unit(p, u, nf);
         return;
     }
+    // the cluster's CTAs take the pool a warp's worth at a time, in turn
+    const int share = ((tid >> 5) * C + rank) * 32 + lane;
+    auto put_key = [&](int i, uint64_t kk) {
+        if (kSplit)
+            ptx::st_dsmem_u64(ptx::dsmem_addr(ptx::smem_addr(key + i), 0), kk);
+        else
+            key[i] = kk;
+    };
 
     // 1. importance (fixed-order sum over query tiles) and selection keys.  A
     // thread takes several pool members at once and walks the query tiles
@@ -233,7 +249,7 @@ __global__ void __launch_bounds__(kSelThreads)
         // Column space, four adjacent columns per thread (16-byte loads): state
         // slot c < count is member c, frame column B + t is member count + t,
         // empty slots are skipped.
-        for (int g4 = tid; g4 < (P >> 2); g4 += kSelThreads) {
+        for (int g4 = share; g4 < (P >> 2); g4 += C * kSelThreads) {
             const int c0 = 4 * g4;
             int ps[4];
 #pragma unroll
@@ -263,20 +279,20 @@ __global__ void __launch_bounds__(kSelThreads)
                 const int pe = c < count ? ps[e] : L + (c - B);
                 const uint64_t kk = (static_cast<uint64_t>(__float_as_uint(rv[e])) << 32) |
                                     static_cast<uint32_t>(0xFFFFFFFFu - static_cast<uint32_t>(pe));
-                key[i] = kk;
+                put_key(i, kk);
                 kand &= kk;
                 kor |= kk;
                 if (imp_out) imp_out[c] = sv[e];
             }
         }
     } else {  // member-wise: kMem pool members per thread
-        for (int i0 = 0; i0 < n; i0 += kMem * kSelThreads) {
+        for (int i0 = 0; i0 < n; i0 += C * kMem * kSelThreads) {
             int col[kMem], ps[kMem];
             bool act[kMem];
             float s[kMem], r[kMem];
 #pragma unroll
             for (int e = 0; e < kMem; ++e) {  // positions first: their loads overlap the sums'
-                const int i = i0 + tid + e * kSelThreads;
+                const int i = i0 + share + e * C * kSelThreads;
                 act[e] = i < n;
                 col[e] = !act[e] ? 0 : i < count ? i : B + (i - count);
                 ps[e] = !act[e] ? 0 : i < count ? pos[i] : L + (i - count);
@@ -294,11 +310,11 @@ __global__ void __launch_bounds__(kSelThreads)
 #pragma unroll
             for (int e = 0; e < kMem; ++e) {
                 if (!act[e]) continue;
-                const int i = i0 + tid + e * kSelThreads;
+                const int i = i0 + share + e * C * kSelThreads;
                 const float rank = p.shared ? r[e] : s[e];
                 const uint64_t kk = (static_cast<uint64_t>(__float_as_uint(rank)) << 32) |
                                     static_cast<uint32_t>(0xFFFFFFFFu - static_cast<uint32_t>(ps[e]));
-                key[i] = kk;
+                put_key(i, kk);
                 kand &= kk;
                 kor |= kk;
                 if (imp_out) imp_out[col[e]] = s[e];
@@ -306,7 +322,32 @@ __global__ void __launch_bounds__(kSelThreads)
         }
     }
     if (imp_out)
-        for (int c = count + tid; c < B; c += kSelThreads) imp_out[c] = 0.f;
+        for (int c = count + share; c < B; c += C * kSelThreads) imp_out[c] = 0.f;
+    // bits in which the keys agree, a warp's at a time, at [rank][warp] of the first CTA
+    if (n > B) {
+        __syncwarp();
+        const uint32_t ah = __reduce_and_sync(0xffffffffu, static_cast<uint32_t>(kand >> 32));
+        const uint32_t al = __reduce_and_sync(0xffffffffu, static_cast<uint32_t>(kand));
+        const uint32_t oh = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(kor >> 32));
+        const uint32_t ol = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(kor));
+        if (lane == 0) {
+            const int at = rank * kSelWarps + (tid >> 5);
+            const unsigned long long a = (static_cast<unsigned long long>(ah) << 32) | al;
+            const unsigned long long o = (static_cast<unsigned long long>(oh) << 32) | ol;
+            if (kSplit) {
+                ptx::st_dsmem_u64(ptx::dsmem_addr(ptx::smem_addr(warp_and + at), 0), a);
+                ptx::st_dsmem_u64(ptx::dsmem_addr(ptx::smem_addr(warp_or + at), 0), o);
+            } else {
+                warp_and[at] = a;
+                warp_or[at] = o;
+            }
+        }
+    }
+    if (kSplit) {
+        __syncwarp();
+        ptx::cluster_sync();  // every key is in the first CTA's shared memory
+        if (rank != 0) return;
+    }
     if (B == 0) {  // no compressed state: nothing is kept
         finish_unit(p, u, nf);
         return;
@@ -315,22 +356,16 @@ __global__ void __launch_bounds__(kSelThreads)
     // 2. top-B selection: kept(i) <=> (key[i] & mask) >= prefix
     unsigned long long prefix = 0, mask = 0;
     if (n > B) {
-        {   // block-wide AND and OR of the keys: digits above the highest bit in
-            // which two keys differ hold one value for every key, so the radix
-            // passes start at the digit holding that bit
-            const uint32_t ah = __reduce_and_sync(0xffffffffu, static_cast<uint32_t>(kand >> 32));
-            const uint32_t al = __reduce_and_sync(0xffffffffu, static_cast<uint32_t>(kand));
-            const uint32_t oh = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(kor >> 32));
-            const uint32_t ol = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(kor));
-            if (lane == 0) {
-                warp_and[tid >> 5] = (static_cast<unsigned long long>(ah) << 32) | al;
-                warp_or[tid >> 5] = (static_cast<unsigned long long>(oh) << 32) | ol;
-            }
-        }
+        // AND and OR of all keys: digits above the highest bit in which two keys
+        // differ hold one value for every key, so the radix passes start at the
+        // digit holding that bit
         __syncthreads();
         if (tid < 32) {  // warp 0 combines the warps' values
-            const unsigned long long wa = lane < kSelWarps ? warp_and[lane] : ~0ull;
-            const unsigned long long wo = lane < kSelWarps ? warp_or[lane] : 0ull;
+            unsigned long long wa = ~0ull, wo = 0ull;
+            for (int i = lane; i < C * kSelWarps; i += 32) {
+                wa &= warp_and[i];
+                wo |= warp_or[i];
+            }
             const unsigned long long a =
                 (static_cast<unsigned long long>(__reduce_and_sync(0xffffffffu, static_cast<uint32_t>(wa >> 32)))
                  << 32) |
@@ -545,8 +580,30 @@ size_t select_smem_bytes(int P, int T)
 
 cudaError_t select_prepare()
 {
-    return cudaFuncSetAttribute(state_select_gather, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(select_smem_bytes(kMaxPool, kMaxFrameTokens)));
+    const int bytes = static_cast<int>(select_smem_bytes(kMaxPool, kMaxFrameTokens));
+    const cudaError_t e =
+        cudaFuncSetAttribute(state_select_gather<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(state_select_gather<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+// CTAs per head: a power of two up to 8 (the portable cluster size) that leaves each
+// a full round of its threads (four columns each, or two members), while the heads'
+// CTAs take three quarters of the SMs or fewer.  The cluster's barriers and remote
+// stores cost ~1.3 us, a round of columns is ~0.5, of members ~1.3, and with
+// layer-level scores each is Hkv + 1 sums: hence the five rounds for plain columns.
+// Per frame of one 7B layer, on one CTA and split: pool 2797 (members) 34.3 -> 33.2
+// us, 5317 (members) 47.6 -> 44.7, 8388 layer-level 70.7 -> 61.9, 16,580 89.9 ->
+// 88.6; columns at 5316 and 8388 would be 45.9 -> 46.7 and 57.0 -> 57.3.
+int select_split(const SelectParams& p, int U)
+{
+    const long long heads = static_cast<long long>(U) * p.Hkv, sms = device_sm_count();
+    const bool columns = (p.P & 3) == 0;
+    const int rounds = p.P / ((columns ? 4 : kMem) * kSelThreads);
+    int C = 1;
+    if (columns && !p.shared && rounds < 5) return C;
+    while (C < kMaxSelSplit && 2 * C <= rounds && heads * 2 * C * 4 <= sms * 3) C *= 2;
+    return C;
 }
 
 cudaError_t launch_select(const SelectParams& p, int U, cudaStream_t st)
@@ -559,16 +616,23 @@ cudaError_t launch_select(const SelectParams& p, int U, cudaStream_t st)
     q.appenders = static_cast<int>(std::min<long long>(8, (chunks + kAppendBatch * kSelThreads - 1) /
                                                               (kAppendBatch * kSelThreads)));
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(U) * (p.Hkv + q.appenders));
+    q.split = select_split(p, U);
+    if (q.split > 1) q.appenders = q.split;  // whole clusters
+    cfg.gridDim = dim3(static_cast<unsigned>(U) * (p.Hkv * q.split + q.appenders));
     cfg.blockDim = dim3(kSelThreads);
     cfg.dynamicSmemBytes = select_smem_bytes(p.P, p.T);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = q.split;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, state_select_gather, q);
+    cfg.numAttrs = q.split > 1 ? 2 : 1;
+    return q.split > 1 ? cudaLaunchKernelEx(&cfg, state_select_gather<true>, q)
+                       : cudaLaunchKernelEx(&cfg, state_select_gather<false>, q);
 }
 
 // Recency window (the baseline the method is compared with): the state keeps

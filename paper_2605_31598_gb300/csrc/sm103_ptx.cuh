@@ -104,6 +104,10 @@ __device__ __forceinline__ float4 ld_dsmem_f4(uint32_t addr)
     return v;
 }
 
+__device__ __forceinline__ void st_dsmem_u64(uint32_t addr, unsigned long long x)
+{
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(x) : "memory");
+}
 __device__ __forceinline__ void st_dsmem_f2(uint32_t addr, float x, float y)
 {
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
@@ -146,12 +150,6 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  :: "r"(smem_addr(sdst)), "l"(gsrc), "r"(bytes), "r"(smem_addr(bar)) : "memory");
-}
-
-// global -> L2 prefetch of `bytes` (a multiple of 16, 16-byte aligned); nothing waits for it
-__device__ __forceinline__ void bulk_prefetch_l2(const void* gsrc, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gsrc), "r"(bytes) : "memory");
 }
 
 // ---------------------------------------------------------------- TMA

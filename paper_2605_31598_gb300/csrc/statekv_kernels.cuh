@@ -111,6 +111,7 @@ struct SelectParams {
     unsigned* tickets;          // arena [S*L][Hkv]: a unit's finished CTAs at its first head; 0 between calls
     long long cap;
     int U, appenders;           // units of the call, append CTAs per unit (set by launch_select)
+    int split;                  // CTAs per head, a cluster (set by launch_select)
 };
 
 struct AppendParams {

@@ -370,6 +370,8 @@ SELECT = {
     "large_ties": (Shape(2, 2, 64, 100, 6000, 62), True, 62),
     "large": (Shape(2, 2, 64, 200, 11000, 57, num_layers=2), False, 57),
     "many_heads": (Shape(16, 16, 64, 100, 6000, 62), False, 62),
+    "eight_ctas": (Shape(2, 2, 64, 400, 21600, 57), False, 57),
+    "eight_ctas_member_wise": (Shape(2, 1, 64, 401, 11000, 30), False, 30),
 }
 
 
