@@ -236,7 +236,8 @@ statekv_status statekv_topb_metrics(const float* scores_n, const float* scores_n
  * library's own tensor-core GEMMs: for up to 256 rows (one stream's frame) a
  * split-K kernel whose clusters add their partial sums in distributed shared
  * memory, with bias + RoPE, the residual add and SiLU * up in its epilogues;
- * above that a cooperative split-K kernel.  Weight matrices are row-major
+ * above that tiles shared by pairs of CTAs, or a cooperative split-K kernel where
+ * the tiles are too few to fill the GPU.  Weight matrices are row-major
  * [out features][in features] (torch.nn.Linear layout). */
 typedef struct {
     int32_t hidden;            /* model width (multiple of 8, at most 8192) */
