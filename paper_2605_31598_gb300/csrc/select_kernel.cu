@@ -28,6 +28,7 @@
 //      4.5 us at a pool of 16.6k: a frame with that state 107 -> 89 us);
 //   3. evicted / empty slots (ascending) receive the admitted frame tokens
 //      (ascending) as 128-bit row copies, and their positions are updated.
+#include "append_plan.h"
 #include "sm103_ptx.cuh"
 #include "statekv_kernels.cuh"
 
@@ -36,7 +37,6 @@
 namespace statekv {
 namespace {
 
-constexpr int kSelThreads = 640;
 constexpr int kSelWarps = kSelThreads / 32;
 static_assert(kSelWarps <= 32, "one warp combines the warps' values");
 
@@ -122,34 +122,34 @@ __device__ __forceinline__ float4 rows_sum4(const float* x, int MT, int stride, 
     return s;
 }
 
-// One append CTA: its share of the unit's K, then V rows, 16 bytes per copy and
-// kAppendBatch copies per thread in flight.
-constexpr int kAppendBatch = 8;
+// One append CTA: its share of the unit's K, then V rows, kAppendBatch copies per
+// thread in flight.
+template <class I>
 __device__ __forceinline__ void append_share(const SelectParams& p, int u, int part)
 {
     const int chunks = p.D / 8;
-    const int per = p.T * p.Hkv * chunks;  // 16-byte chunks of one matrix, source order [t][hkv][chunk]
+    const long long copies = append_copies(p.T, p.Hkv, p.D);
+    const I per = static_cast<I>(copies);
     const size_t base = static_cast<size_t>(p.units.unit_abs(u)) * p.Hkv;
     const long long row0 = static_cast<long long>(p.frames[base]) * p.T;
-    const uint4* k = reinterpret_cast<const uint4*>(p.k) + static_cast<size_t>(u) * per;
-    const uint4* v = reinterpret_cast<const uint4*>(p.v) + static_cast<size_t>(u) * per;
-    for (int i0 = part * kAppendBatch * kSelThreads + threadIdx.x; i0 < 2 * per;
+    const uint4* k = reinterpret_cast<const uint4*>(p.k) + u * copies;
+    const uint4* v = reinterpret_cast<const uint4*>(p.v) + u * copies;
+    for (I i0 = part * kAppendBatch * kSelThreads + threadIdx.x; i0 < 2 * per;
          i0 += p.appenders * kAppendBatch * kSelThreads) {
         uint4 x[kAppendBatch];
 #pragma unroll
         for (int e = 0; e < kAppendBatch; ++e) {
-            const int i = i0 + e * kSelThreads;
+            const I i = i0 + e * kSelThreads;
             if (i < 2 * per) x[e] = i < per ? k[i] : v[i - per];
         }
 #pragma unroll
         for (int e = 0; e < kAppendBatch; ++e) {
-            const int i = i0 + e * kSelThreads;
+            const I i = i0 + e * kSelThreads;
             if (i >= 2 * per) break;
-            const int r = i < per ? i : i - per, t = r / (p.Hkv * chunks), hc = r - t * (p.Hkv * chunks);
-            const int hkv = hc / chunks, ch = hc - hkv * chunks;
-            const long long row = row0 + t;
+            const AppendAt at = append_at(i, per, p.Hkv, chunks);
+            const long long row = row0 + at.t;
             if (!SKV_CHECK(row >= 0 && row < p.cap, p.status, 4)) continue;
-            reinterpret_cast<uint4*>(i < per ? p.cache_k : p.cache_v)[((base + hkv) * p.cap + row) * chunks + ch] = x[e];
+            reinterpret_cast<uint4*>(i < per ? p.cache_k : p.cache_v)[((base + at.hkv) * p.cap + row) * chunks + at.ch] = x[e];
         }
     }
 }
@@ -190,7 +190,10 @@ __global__ void __launch_bounds__(kSelThreads)
         // the inputs and counters are there; it reads neither cache nor writes these
         const int u = blockIdx.x / p.appenders;
         const int nf0 = p.frames[static_cast<size_t>(p.units.unit_abs(u)) * p.Hkv];
-        append_share(p, u, blockIdx.x - u * p.appenders);
+        if (append_narrow(p.T, p.Hkv, p.D))
+            append_share<int>(p, u, blockIdx.x - u * p.appenders);
+        else
+            append_share<long long>(p, u, blockIdx.x - u * p.appenders);
         finish_unit(p, u, nf0);
         return;
     }
@@ -612,7 +615,7 @@ cudaError_t launch_select(const SelectParams& p, int U, cudaStream_t st)
     SelectParams q = p;
     q.U = U;
     // append CTAs per unit: one batch of copies each, up to eight
-    const long long chunks = 2ll * p.T * p.Hkv * (p.D / 8);
+    const long long chunks = 2 * append_copies(p.T, p.Hkv, p.D);
     q.appenders = static_cast<int>(std::min<long long>(8, (chunks + kAppendBatch * kSelThreads - 1) /
                                                               (kAppendBatch * kSelThreads)));
     cudaLaunchConfig_t cfg{};
