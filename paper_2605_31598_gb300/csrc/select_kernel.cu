@@ -3,14 +3,16 @@
 // K4: decode-cache append (Sec. 3.2 detailed state; Sec. 3.3 "append").
 //
 // K3 runs one CTA per (unit, KV head) (a cluster for the sums of large pools, see
-// select_split), and in the same launch a few CTAs per unit
+// select_split), and in the same launch, after these, a few CTAs per unit
 // that append the frame's K and V to the decode cache (K4's work).  It is launched
-// programmatically behind the attention kernel: it is in place when that ends, and
-// the append, which needs nothing of the attention kernel's, takes the SMs that
-// kernel's last round leaves idle.  (As a launch of its own on a side stream the
-// append needed two events per frame and kept the other two kernels from
-// overlapping.  Per frame, before and after: toy 17.2 and 11.5 us, one 7B layer
-// 32.5 and 29.0, four small-backbone layers 34.6 and 26.7.)
+// programmatically behind the attention kernel, so it is in place when that ends.
+// The append CTAs wait for that too, although they need nothing of the attention
+// kernel's: what was written before it (K, V, the frame counters) is visible to this
+// grid only after the wait.  Last in the grid they take no SM from a head's CTA
+// (first in it, the wait cost 4 us of 227 at 28 layers; last, none).  (As a launch of
+// its own on a side stream the append needed two events per frame and kept the other
+// two kernels from overlapping.  Per frame, before and after: toy 17.2 and 12.1 us,
+// one 7B layer 32.5 and 28.5, four small-backbone layers 34.6 and 25.5.)
 //   1. importance of every pool member = the fixed-order sum of the attention
 //      kernel's per-query-tile partials (deterministic); with layer-level
 //      selection (App. A) the ranking score is the same sum taken over every
@@ -185,19 +187,20 @@ __global__ void __launch_bounds__(kSelThreads)
     // tiles, which nothing here writes, and waits for this grid's completion
     // before it reads anything else.
     ptx::pdl_launch_dependents();
-    if (static_cast<int>(blockIdx.x) < p.U * p.appenders) {
-        // the attention kernel started after everything before it had completed, so
-        // the inputs and counters are there; it reads neither cache nor writes these
-        const int u = blockIdx.x / p.appenders;
+    const int C = kSplit ? p.split : 1;
+    const int app = static_cast<int>(blockIdx.x) - p.U * p.Hkv * C;  // append CTA, after the heads'
+    if (app >= 0) {
+        ptx::pdl_wait();  // K, V and the counters, written before the attention kernel
+        const int u = app / p.appenders;
         const int nf0 = p.frames[static_cast<size_t>(p.units.unit_abs(u)) * p.Hkv];
         if (append_narrow(p.T, p.Hkv, p.D))
-            append_share<int>(p, u, blockIdx.x - u * p.appenders);
+            append_share<int>(p, u, app - u * p.appenders);
         else
-            append_share<long long>(p, u, blockIdx.x - u * p.appenders);
+            append_share<long long>(p, u, app - u * p.appenders);
         finish_unit(p, u, nf0);
         return;
     }
-    const int C = kSplit ? p.split : 1, rank = kSplit ? static_cast<int>(ptx::cluster_ctarank()) : 0;
+    const int rank = kSplit ? static_cast<int>(ptx::cluster_ctarank()) : 0;
     if (kSplit) ptx::cluster_sync();  // the cluster's CTAs run: their shared memory can be written
     ptx::pdl_wait();  // the attention kernel's partials; it has read the state
     const int T = p.T, B = p.B, P = p.P, D = p.D;
@@ -214,7 +217,7 @@ __global__ void __launch_bounds__(kSelThreads)
     constexpr int kMaxC = kSplit ? kMaxSelSplit : 1;
     __shared__ unsigned long long warp_and[kMaxC * kSelWarps], warp_or[kMaxC * kSelWarps];
 
-    const int unit_head = (blockIdx.x - p.U * p.appenders) / C, u = unit_head / p.Hkv, hkv = unit_head - u * p.Hkv;
+    const int unit_head = blockIdx.x / C, u = unit_head / p.Hkv, hkv = unit_head - u * p.Hkv;
     const int ua = p.units.unit_abs(u);
     const int tid = threadIdx.x, lane = tid & 31;
     const size_t head = static_cast<size_t>(ua) * p.Hkv + hkv;
