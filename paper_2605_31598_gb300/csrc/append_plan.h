@@ -22,6 +22,15 @@ SKV_HOST_DEVICE long long append_copies(int T, int Hkv, int D) { return static_c
 // 128 are 2^31, and the configuration allows 65,535 heads.
 SKV_HOST_DEVICE bool append_narrow(int T, int Hkv, int D) { return 2 * append_copies(T, Hkv, D) <= 1ll << 30; }
 
+// Append CTAs per unit: one batch of copies for each thread, up to eight CTAs, and
+// whole clusters where the heads' CTAs come in clusters of `split` (1, 2, 4 or 8).
+inline int append_ctas(int T, int Hkv, int D, int split)
+{
+    const long long per_cta = kAppendBatch * kSelThreads;
+    const long long n = (2 * append_copies(T, Hkv, D) + per_cta - 1) / per_cta;
+    return (static_cast<int>(n < 8 ? n : 8) + split - 1) / split * split;
+}
+
 struct AppendAt {
     int t, hkv, ch;
 };

@@ -617,13 +617,9 @@ cudaError_t launch_select(const SelectParams& p, int U, cudaStream_t st)
     if (U <= 0) return cudaSuccess;
     SelectParams q = p;
     q.U = U;
-    // append CTAs per unit: one batch of copies each, up to eight
-    const long long chunks = 2 * append_copies(p.T, p.Hkv, p.D);
-    q.appenders = static_cast<int>(std::min<long long>(8, (chunks + kAppendBatch * kSelThreads - 1) /
-                                                              (kAppendBatch * kSelThreads)));
-    cudaLaunchConfig_t cfg{};
     q.split = select_split(p, U);
-    if (q.split > 1) q.appenders = q.split;  // whole clusters
+    q.appenders = append_ctas(p.T, p.Hkv, p.D, q.split);
+    cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(U) * (p.Hkv * q.split + q.appenders));
     cfg.blockDim = dim3(kSelThreads);
     cfg.dynamicSmemBytes = select_smem_bytes(p.P, p.T);
