@@ -35,6 +35,7 @@
 #include "statekv_kernels.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace statekv {
 namespace {
@@ -70,32 +71,44 @@ __device__ __forceinline__ int block_exclusive_scan(int x, int* warp_sums, int& 
     return warp_sums[kSelWarps];  // warp_sums is not written again before the caller's next barrier
 }
 
-// For each of kMem pool members (columns col[e], active act[e]): the sum of
-// x[mt * stride + col] over mt < MT, added in mt order.  Twelve tiles' loads of
-// all members (24 independent loads) are in flight before any addition.
+// For each of M pool members (columns col[e], active act[e]): the sum of
+// x[mt * stride + col] over mt < MT, added in mt order.  K tiles' loads of all
+// members (24 or 32 independent loads) are in flight before any addition.
 // (Plain loads: the kernel is resident while the attention kernel still writes
 // the partials, so the read-only path, which may move a load ahead of the wait, is
 // not for them.)
-constexpr int kMem = 2;
-__device__ __forceinline__ void tiles_sum(const float* x, int MT, int stride, const int (&col)[kMem],
-                                          const bool (&act)[kMem], float (&s)[kMem])
+template <int M, int K>
+__device__ __forceinline__ void tiles_sum(const float* x, int MT, int stride, const int (&col)[M],
+                                          const bool (&act)[M], float (&s)[M])
 {
 #pragma unroll
-    for (int e = 0; e < kMem; ++e) s[e] = 0.f;
+    for (int e = 0; e < M; ++e) s[e] = 0.f;
 #pragma unroll 1
-    for (int mt = 0; mt < MT; mt += 12) {
-        float v[12][kMem];
+    for (int mt = 0; mt < MT; mt += K) {
+        float v[K][M];
 #pragma unroll
-        for (int m = 0; m < 12; ++m)
+        for (int m = 0; m < K; ++m)
 #pragma unroll
-            for (int e = 0; e < kMem; ++e)
+            for (int e = 0; e < M; ++e)
                 v[m][e] = (act[e] && mt + m < MT) ? x[static_cast<size_t>(mt + m) * stride + col[e]] : 0.f;
 #pragma unroll
-        for (int m = 0; m < 12; ++m)
+        for (int m = 0; m < K; ++m)
 #pragma unroll
-            for (int e = 0; e < kMem; ++e)
+            for (int e = 0; e < M; ++e)
                 if (mt + m < MT) s[e] += v[m][e];
     }
+}
+
+// Members per thread and round where one CTA takes the pool member by member: two
+// with twelve query tiles' loads in flight; or eight with four, if there are no more
+// tiles than that, layer-level scores (heads to add up, a round of latencies each)
+// and three or more rounds by twos.  Two layers of 32 heads, two tiles, layer-level:
+// pool 4355 168 us a frame by twos, 110 by eights (133 was eights for every pool on
+// the 8-bit selection); 12 layers of 12 heads, pool 1257 56 and 66 us.
+constexpr int kMem = 2, kMemFewTiles = 8;
+__host__ __device__ constexpr int select_members(int MT, int shared, int P)
+{
+    return MT <= 4 && shared && P > 2 * kMem * kSelThreads ? kMemFewTiles : kMem;
 }
 
 // For 4 adjacent columns c0..c0+3 (16-byte aligned): the sums of
@@ -291,41 +304,48 @@ __global__ void __launch_bounds__(kSelThreads)
                 if (imp_out) imp_out[c] = sv[e];
             }
         }
-    } else {  // member-wise: kMem pool members per thread
-        for (int i0 = 0; i0 < n; i0 += C * kMem * kSelThreads) {
-            int col[kMem], ps[kMem];
-            bool act[kMem];
-            float s[kMem], r[kMem];
+    } else {  // member-wise: M pool members per thread
+        auto members = [&](auto per_thread, auto tiles) {
+            constexpr int M = decltype(per_thread)::value, K = decltype(tiles)::value;
+            for (int i0 = 0; i0 < n; i0 += C * M * kSelThreads) {
+                int col[M], ps[M];
+                bool act[M];
+                float s[M], r[M];
 #pragma unroll
-            for (int e = 0; e < kMem; ++e) {  // positions first: their loads overlap the sums'
-                const int i = i0 + share + e * C * kSelThreads;
-                act[e] = i < n;
-                col[e] = !act[e] ? 0 : i < count ? i : B + (i - count);
-                ps[e] = !act[e] ? 0 : i < count ? pos[i] : L + (i - count);
-                r[e] = 0.f;
-            }
-            tiles_sum(part, p.MT, P, col, act, s);
-            if (p.shared) {  // the ranking score: the same sums for every KV head, heads in order
-                for (int h2 = 0; h2 < p.Hkv; ++h2) {
-                    float sh[kMem];
-                    tiles_sum(part0 + static_cast<size_t>(h2) * p.MT * P, p.MT, P, col, act, sh);
+                for (int e = 0; e < M; ++e) {  // positions first: their loads overlap the sums'
+                    const int i = i0 + share + e * C * kSelThreads;
+                    act[e] = i < n;
+                    col[e] = !act[e] ? 0 : i < count ? i : B + (i - count);
+                    ps[e] = !act[e] ? 0 : i < count ? pos[i] : L + (i - count);
+                    r[e] = 0.f;
+                }
+                tiles_sum<M, K>(part, p.MT, P, col, act, s);
+                if (p.shared) {  // the ranking score: the same sums for every KV head, heads in order
+                    for (int h2 = 0; h2 < p.Hkv; ++h2) {
+                        float sh[M];
+                        tiles_sum<M, K>(part0 + static_cast<size_t>(h2) * p.MT * P, p.MT, P, col, act, sh);
 #pragma unroll
-                    for (int e = 0; e < kMem; ++e) r[e] += sh[e];
+                        for (int e = 0; e < M; ++e) r[e] += sh[e];
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < M; ++e) {
+                    if (!act[e]) continue;
+                    const int i = i0 + share + e * C * kSelThreads;
+                    const float rank = p.shared ? r[e] : s[e];
+                    const uint64_t kk = (static_cast<uint64_t>(__float_as_uint(rank)) << 32) |
+                                        static_cast<uint32_t>(0xFFFFFFFFu - static_cast<uint32_t>(ps[e]));
+                    put_key(i, kk);
+                    kand &= kk;
+                    kor |= kk;
+                    if (imp_out) imp_out[col[e]] = s[e];
                 }
             }
-#pragma unroll
-            for (int e = 0; e < kMem; ++e) {
-                if (!act[e]) continue;
-                const int i = i0 + share + e * C * kSelThreads;
-                const float rank = p.shared ? r[e] : s[e];
-                const uint64_t kk = (static_cast<uint64_t>(__float_as_uint(rank)) << 32) |
-                                    static_cast<uint32_t>(0xFFFFFFFFu - static_cast<uint32_t>(ps[e]));
-                put_key(i, kk);
-                kand &= kk;
-                kor |= kk;
-                if (imp_out) imp_out[col[e]] = s[e];
-            }
-        }
+        };
+        if (!kSplit && select_members(p.MT, p.shared, P) == kMemFewTiles)
+            members(std::integral_constant<int, kMemFewTiles>{}, std::integral_constant<int, 4>{});
+        else
+            members(std::integral_constant<int, kMem>{}, std::integral_constant<int, 12>{});
     }
     if (imp_out)
         for (int c = count + share; c < B; c += C * kSelThreads) imp_out[c] = 0.f;

@@ -423,3 +423,23 @@ def test_selection_is_exact_for_the_exported_importance(name, selection):
                     got = after[h].astype(np.int64)
                     assert (got[:live] == want[:live]).all(), (name, n, s, l, h)
     assert eng.sync() == 0
+
+
+FEW_TILES = {
+    # (shape, frames): 64 heads (a CTA each) whose pools are taken member by member.  With
+    # at most four query tiles and a pool above 2560 the sums are formed eight members at a
+    # time, else two at a time.
+    "one_tile_two_rounds": (Shape(32, 32, 64, 100, 5201, 55, num_layers=2), 55),
+    "four_tiles": (Shape(32, 8, 64, 128, 2501, 22, num_layers=8), 22),
+    "five_tiles": (Shape(32, 8, 64, 129, 2502, 22, num_layers=8), 22),
+    "pool_2557": (Shape(32, 32, 64, 100, 2457, 27, num_layers=2), 27),
+    "pool_2561": (Shape(32, 32, 64, 100, 2461, 27, num_layers=2), 27),
+}
+
+
+@pytest.mark.parametrize("name", sorted(FEW_TILES))
+def test_layer_selection_is_exact_with_few_query_tiles(name, monkeypatch):
+    """As above, for layer-level scores over few query tiles."""
+    shape, frames = FEW_TILES[name]
+    monkeypatch.setitem(SELECT, name, (shape, False, frames))
+    test_selection_is_exact_for_the_exported_importance(name, 2)
