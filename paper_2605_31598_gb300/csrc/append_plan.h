@@ -22,17 +22,13 @@ SKV_HOST_DEVICE long long append_copies(int T, int Hkv, int D) { return static_c
 // 128 are 2^31, and the configuration allows 65,535 heads.
 SKV_HOST_DEVICE bool append_narrow(int T, int Hkv, int D) { return 2 * append_copies(T, Hkv, D) <= 1ll << 30; }
 
-// Append CTAs per unit: one batch of copies for each thread, up to 24 CTAs, and
+// Append CTAs per unit: one batch of copies for each thread, up to eight CTAs, and
 // whole clusters where the heads' CTAs come in clusters of `split` (1, 2, 4 or 8).
-// The append runs beside the selection, so many copies on few CTAs outlast it: one
-// layer of 28 heads of 128 with 399 tokens (70 batches) 57.8 us a frame on eight,
-// 49.0 on 24; 16 heads, 167 tokens (17) 28.6 and 26.9; five batches or fewer (four
-// heads, 196 tokens) are the same.
 inline int append_ctas(int T, int Hkv, int D, int split)
 {
     const long long per_cta = kAppendBatch * kSelThreads;
     const long long n = (2 * append_copies(T, Hkv, D) + per_cta - 1) / per_cta;
-    return (static_cast<int>(n < 24 ? n : 24) + split - 1) / split * split;
+    return (static_cast<int>(n < 8 ? n : 8) + split - 1) / split * split;
 }
 
 struct AppendAt {

@@ -61,8 +61,8 @@ def test_every_copy_has_its_place(program, T, hkv, d):
                          capture_output=True, text=True).stdout.split("\n")
     copies, narrow, *ctas = map(int, out[0].split())
     assert copies == per
-    # the kernel's loop goes past the last copy by at most 24 CTAs' batches of 8 x 640
-    assert not narrow or 2 * per + 25 * 8 * 640 < 2 ** 31
+    # the kernel's loop goes past the last copy by at most 8 CTAs' batches of 8 x 640
+    assert not narrow or 2 * per + 9 * 8 * 640 < 2 ** 31
     for i, line in zip(at, out[1:]):
         r = i % per
         assert tuple(map(int, line.split())) == (r // (hkv * ch), r // ch % hkv, r % ch), i
@@ -70,9 +70,9 @@ def test_every_copy_has_its_place(program, T, hkv, d):
 
 @pytest.mark.parametrize("T,hkv,d", [(16, 1, 64), (196, 4, 128), (399, 28, 128), (401, 1, 64), (4096, 65535, 128)])
 def test_append_ctas_cover_the_copies_in_whole_clusters(program, T, hkv, d):
-    """As many CTAs as batches of copies, 24 at most; a cluster size rounds that up
+    """As many CTAs as batches of copies, eight at most; a cluster size rounds that up
     and never takes CTAs away."""
     out = subprocess.run([program, str(T), str(hkv), str(d)], check=True, capture_output=True, text=True).stdout
-    want = min(24, -(-2 * T * hkv * (d // 8) // (8 * 640)))
+    want = min(8, -(-2 * T * hkv * (d // 8) // (8 * 640)))
     for split, n in zip((1, 2, 4, 8), map(int, out.split()[2:])):
         assert n % split == 0 and want <= n < want + split, (split, n)
