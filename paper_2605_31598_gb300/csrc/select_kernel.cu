@@ -35,7 +35,6 @@
 #include "statekv_kernels.cuh"
 
 #include <algorithm>
-#include <type_traits>
 
 namespace statekv {
 namespace {
@@ -106,9 +105,9 @@ __device__ __forceinline__ void tiles_sum(const float* x, int MT, int stride, co
 // pool 4355 168 us a frame by twos, 110 by eights (133 was eights for every pool on
 // the 8-bit selection); 12 layers of 12 heads, pool 1257 56 and 66 us.
 constexpr int kMem = 2, kMemFewTiles = 8;
-__host__ __device__ constexpr int select_members(int MT, int shared, int P)
+int select_members(const SelectParams& p, int split)
 {
-    return MT <= 4 && shared && P > 2 * kMem * kSelThreads ? kMemFewTiles : kMem;
+    return split == 1 && (p.P & 3) != 0 && p.MT <= 4 && p.shared && p.P > 2 * kMem * kSelThreads ? kMemFewTiles : kMem;
 }
 
 // For 4 adjacent columns c0..c0+3 (16-byte aligned): the sums of
@@ -190,10 +189,13 @@ static_assert(kBins / 4 <= kSelThreads && kBins % 128 == 0, "four bins per threa
 
 // kSplit: a cluster of p.split CTAs makes the keys of a head, each from its share of
 // the pool's columns; they meet in the first CTA's shared memory, which goes on alone.
-template <bool kSplit>
+// kMembers: see select_members (an instantiation of its own: as a branch of one kernel
+// the second form cost the first 2 to 5%).
+template <bool kSplit, int kMembers>
 __global__ void __launch_bounds__(kSelThreads)
     state_select_gather(const SelectParams p)
 {
+    constexpr int kTiles = kMembers == kMem ? 12 : 4;  // query tiles whose loads are in flight
     extern __shared__ __align__(16) uint8_t smem_raw[];
     // A kernel launched programmatically behind this one (the transformer
     // block's output projection) may start now: it requests its first weight
@@ -264,7 +266,7 @@ __global__ void __launch_bounds__(kSelThreads)
     const float* part0 = p.partials + static_cast<size_t>(u) * p.Hkv * p.MT * P;
     // bits every selection key shares: the radix select starts below them
     unsigned long long kand = ~0ull, kor = 0ull;
-    if ((P & 3) == 0) {
+    if (kMembers == kMem && (P & 3) == 0) {
         // Column space, four adjacent columns per thread (16-byte loads): state
         // slot c < count is member c, frame column B + t is member count + t,
         // empty slots are skipped.
@@ -304,48 +306,41 @@ __global__ void __launch_bounds__(kSelThreads)
                 if (imp_out) imp_out[c] = sv[e];
             }
         }
-    } else {  // member-wise: M pool members per thread
-        auto members = [&](auto per_thread, auto tiles) {
-            constexpr int M = decltype(per_thread)::value, K = decltype(tiles)::value;
-            for (int i0 = 0; i0 < n; i0 += C * M * kSelThreads) {
-                int col[M], ps[M];
-                bool act[M];
-                float s[M], r[M];
+    } else {  // member-wise: kMembers pool members per thread
+        for (int i0 = 0; i0 < n; i0 += C * kMembers * kSelThreads) {
+            int col[kMembers], ps[kMembers];
+            bool act[kMembers];
+            float s[kMembers], r[kMembers];
 #pragma unroll
-                for (int e = 0; e < M; ++e) {  // positions first: their loads overlap the sums'
-                    const int i = i0 + share + e * C * kSelThreads;
-                    act[e] = i < n;
-                    col[e] = !act[e] ? 0 : i < count ? i : B + (i - count);
-                    ps[e] = !act[e] ? 0 : i < count ? pos[i] : L + (i - count);
-                    r[e] = 0.f;
-                }
-                tiles_sum<M, K>(part, p.MT, P, col, act, s);
-                if (p.shared) {  // the ranking score: the same sums for every KV head, heads in order
-                    for (int h2 = 0; h2 < p.Hkv; ++h2) {
-                        float sh[M];
-                        tiles_sum<M, K>(part0 + static_cast<size_t>(h2) * p.MT * P, p.MT, P, col, act, sh);
+            for (int e = 0; e < kMembers; ++e) {  // positions first: their loads overlap the sums'
+                const int i = i0 + share + e * C * kSelThreads;
+                act[e] = i < n;
+                col[e] = !act[e] ? 0 : i < count ? i : B + (i - count);
+                ps[e] = !act[e] ? 0 : i < count ? pos[i] : L + (i - count);
+                r[e] = 0.f;
+            }
+            tiles_sum<kMembers, kTiles>(part, p.MT, P, col, act, s);
+            if (p.shared) {  // the ranking score: the same sums for every KV head, heads in order
+                for (int h2 = 0; h2 < p.Hkv; ++h2) {
+                    float sh[kMembers];
+                    tiles_sum<kMembers, kTiles>(part0 + static_cast<size_t>(h2) * p.MT * P, p.MT, P, col, act, sh);
 #pragma unroll
-                        for (int e = 0; e < M; ++e) r[e] += sh[e];
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < M; ++e) {
-                    if (!act[e]) continue;
-                    const int i = i0 + share + e * C * kSelThreads;
-                    const float rank = p.shared ? r[e] : s[e];
-                    const uint64_t kk = (static_cast<uint64_t>(__float_as_uint(rank)) << 32) |
-                                        static_cast<uint32_t>(0xFFFFFFFFu - static_cast<uint32_t>(ps[e]));
-                    put_key(i, kk);
-                    kand &= kk;
-                    kor |= kk;
-                    if (imp_out) imp_out[col[e]] = s[e];
+                    for (int e = 0; e < kMembers; ++e) r[e] += sh[e];
                 }
             }
-        };
-        if (!kSplit && select_members(p.MT, p.shared, P) == kMemFewTiles)
-            members(std::integral_constant<int, kMemFewTiles>{}, std::integral_constant<int, 4>{});
-        else
-            members(std::integral_constant<int, kMem>{}, std::integral_constant<int, 12>{});
+#pragma unroll
+            for (int e = 0; e < kMembers; ++e) {
+                if (!act[e]) continue;
+                const int i = i0 + share + e * C * kSelThreads;
+                const float rank = p.shared ? r[e] : s[e];
+                const uint64_t kk = (static_cast<uint64_t>(__float_as_uint(rank)) << 32) |
+                                    static_cast<uint32_t>(0xFFFFFFFFu - static_cast<uint32_t>(ps[e]));
+                put_key(i, kk);
+                kand &= kk;
+                kor |= kk;
+                if (imp_out) imp_out[col[e]] = s[e];
+            }
+        }
     }
     if (imp_out)
         for (int c = count + share; c < B; c += C * kSelThreads) imp_out[c] = 0.f;
@@ -607,10 +602,12 @@ size_t select_smem_bytes(int P, int T)
 cudaError_t select_prepare()
 {
     const int bytes = static_cast<int>(select_smem_bytes(kMaxPool, kMaxFrameTokens));
-    const cudaError_t e =
-        cudaFuncSetAttribute(state_select_gather<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(state_select_gather<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    for (auto kernel : {state_select_gather<true, kMem>, state_select_gather<false, kMem>,
+                        state_select_gather<false, kMemFewTiles>}) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // CTAs per head: a power of two up to 8 (the portable cluster size) that leaves each
@@ -653,8 +650,10 @@ cudaError_t launch_select(const SelectParams& p, int U, cudaStream_t st)
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = q.split > 1 ? 2 : 1;
-    return q.split > 1 ? cudaLaunchKernelEx(&cfg, state_select_gather<true>, q)
-                       : cudaLaunchKernelEx(&cfg, state_select_gather<false>, q);
+    const auto kernel = q.split > 1                                     ? state_select_gather<true, kMem>
+                        : select_members(p, q.split) == kMemFewTiles ? state_select_gather<false, kMemFewTiles>
+                                                                     : state_select_gather<false, kMem>;
+    return cudaLaunchKernelEx(&cfg, kernel, q);
 }
 
 // Recency window (the baseline the method is compared with): the state keeps
