@@ -633,6 +633,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (rank 0)
+        pdl_wait();  // the deadlines start when the previous kernel has ended
         if (rank == 0) {
             const uint32_t id = uniform(idesc_bf16_f32(256, BN, false, false));
             const uint32_t s0 = uniform(smem_addr(sm)), t0 = uniform(tbase);
@@ -1047,7 +1048,6 @@ __global__ void __launch_bounds__(kGThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
-    const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
     auto fail = [&](int site) {
         if (atomicExch(const_cast<int*>(abort_flag), 1) == 0)
             *reinterpret_cast<volatile int32_t*>(p.status) = DEV_TIMEOUT_GEMM | (site << 8);
@@ -1080,6 +1080,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         for (uint32_t n = 0; n < pre; ++n)
             if (elect_one()) load_w(n, n);
         pdl_wait();
+        const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
         for (uint32_t n = 0; n < pre; ++n)
             if (elect_one())
                 tma_load_at(s0 + n * stage_bytes + x_off, &tm_x, bfull + 8 * n, (ks0 + n) * kGemmBK, 0, 0, 0);
@@ -1107,6 +1108,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
         const uint32_t s0 = uniform(smem_addr(sm)), t0 = uniform(tbase), bfull = smem_addr(full),
                        bempty = smem_addr(empty);
         uint32_t s = 0, ph = 0;
+        pdl_wait();  // the deadline starts when the previous kernel has ended
+        const unsigned long long deadline = g_globaltimer() + p.watchdog_ns;
 #pragma unroll 1
         for (int ks = ks0; ks < ks1; ++ks) {
             if (!(ok = wait_warp(bfull + 8 * s, ph, deadline))) break;
@@ -1135,7 +1138,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
         const int r = quad * 32 + lane;
         const int chunks = (p.M + 31) / 32;
-        ok = __all_sync(0xffffffffu, g_wait(acc_full, 0, deadline));
+        pdl_wait();
+        ok = __all_sync(0xffffffffu, g_wait(acc_full, 0, g_globaltimer() + p.watchdog_ns));
         if (!ok) fail(8);
         if (ok) tc_fence_after();
         if (ok && p.op == kThinSilu && p.splits == 1) {

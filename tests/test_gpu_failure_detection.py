@@ -13,7 +13,8 @@ import pytest
 import torch
 
 from paper_2605_31598_gb300 import StateKV, make_config
-from paper_2605_31598_gb300.inputs import WORKLOADS, batch_qkv
+from paper_2605_31598_gb300.inputs import WORKLOADS, BlockShape, Shape, batch_qkv, block_weights
+from paper_2605_31598_gb300.statekv import SELECTION_LAYER, block_weights_array, statekv_block_config
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +50,34 @@ def test_expired_wait_is_reported_and_the_context_survives():
     assert fresh.prefill_frame(q, k, v, out) == 0
     assert fresh.sync() == 0
     assert torch.isfinite(out.float()).all()
+
+
+@pytest.mark.parametrize("shape,hidden", [
+    # one stream: the output projection is the GEMM for few rows
+    (Shape(1024, 64, 64, 256, 16384, 3), 128),
+    # three streams: it is the one on CTA pairs (51 x 3 tiles of 128 columns fill the SMs)
+    (Shape(768, 32, 64, 256, 24320, 3, num_streams=3), 6528),
+])
+def test_waiting_for_the_previous_kernel_is_not_a_timeout(shape, hidden):
+    """The block's output projection is launched programmatically and is in place while
+    the selection runs.  Here that takes longer than the watchdog (layer-level scores
+    over many heads and a large pool: 1.3 and 1.5 ms against 1 ms, alone), and every kernel
+    by itself less than half of it, so a wait may only be timed from the end of the
+    selection on.  The results are those of a handle with the default watchdog."""
+    block = BlockShape(hidden, 256)
+    warr = block_weights_array(weights := block_weights(shape, block, device="cuda"))
+    bc = statekv_block_config(block.hidden, block.intermediate, block.rms_eps, block.rope_theta, 1.0, 0)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(0)
+    x = torch.randn((shape.num_streams, shape.tokens_per_frame, hidden), generator=g, device="cuda").bfloat16()
+    outs = []
+    for ms in (0, 1):
+        eng = StateKV(make_config(shape, selection=SELECTION_LAYER, watchdog_ms=ms))
+        ws = torch.empty(eng.block_workspace_bytes(bc), dtype=torch.uint8, device="cuda")
+        outs.append(torch.full_like(x, float("nan")))
+        for _ in range(2):
+            assert eng.block_frame(bc, warr, x, outs[-1], ws) == 0
+        assert eng.sync() == 0, hex(eng.device_error())
+        eng.close()
+    assert weights and torch.isfinite(outs[0].float()).all()
+    assert torch.equal(outs[0], outs[1])
