@@ -14,11 +14,13 @@
 //   state_metrics       App. A.2: the counts and weights behind candidate-pool
 //                       recall, weighted recall, retention and churn
 // A few dozen rows of tens of thousands of scores are too few CTAs at one per
-// row, and each CTA then walks its row alone: 28 rows of 25k scores took 50 us
-// (top-B: up to eight passes), 27 us (concentration: two fp64 adds per score on
-// 28 SMs) and 65 us (metrics).  A row is therefore shared by the CTAs of one
+// row, and each CTA then walks its row alone: 28 rows of 25k scores took 42 us
+// (top-B: up to eight passes), 25 us (concentration: two fp64 adds per score on
+// 28 SMs) and 38 us (metrics).  A long row is therefore shared by the CTAs of one
 // thread-block cluster (row_cluster), which merge their histograms and sums in
-// distributed shared memory: 16, 11 and 12 us.  Sums are
+// distributed shared memory: 15, 8 and 9 us.  A row that one CTA takes alone has a
+// kernel without the merging: 28 rows of 2048 in 5.2, 4.3 and 5.3 us, where a
+// cluster of one took 7.9, 5.8 and 6.5.  Sums are
 // added in one fixed order for a given cluster size, so they are deterministic.
 #include "sm103_ptx.cuh"
 #include "statekv_kernels.cuh"
@@ -33,15 +35,20 @@ constexpr int kDiagBatch = 8;  // scores per thread in flight (and kept between 
 
 // Sums of two doubles per thread over the block; thread 0 gets them.  An fp64
 // add of a warp takes 16 cycles of the SM, so the warps reduce both values at
-// once, one in each half (5 adds where two full trees take 10).
-__device__ void block_sum2(double a, double b, double* sh, double (&out)[2])
+// once, one in each half (5 adds where two full trees take 10).  `some`: the warp has
+// entries at all (a short row leaves most without: concentration of 2000 rows of 64
+// 28.7 -> 20.9 us).
+__device__ void block_sum2(double a, double b, bool some, double* sh, double (&out)[2])
 {
     static_assert(kDiagWarps == 16, "one warp adds the warps' two sums");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool up = lane >= 16;
-    double x = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+    double x = 0.0;
+    if (some) {
+        x = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    }
     if ((lane & 15) == 0) sh[(up ? kDiagWarps : 0) + warp] = x;
     __syncthreads();
     if (warp == 0) {
@@ -119,10 +126,17 @@ __device__ __forceinline__ void red_dsmem_add(uint32_t addr, unsigned v)
     asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// The cluster's partial sums, one set per CTA, added in rank order by the first.
-template <int K>
-__device__ void cluster_total(const double (&v)[K], double* sh, int r, int C, double* out)
+// The cluster's partial sums, one set per CTA, added in rank order by the first (a
+// CTA alone writes its own).
+template <bool kCluster, int K>
+__device__ void row_total(const double (&v)[K], double* sh, int r, int C, double* out)
 {
+    if constexpr (!kCluster) {
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int i = 0; i < K; ++i) out[i] = v[i];
+        return;
+    }
     if (threadIdx.x == 0)
 #pragma unroll
         for (int i = 0; i < K; ++i) sh[i] = v[i];
@@ -157,16 +171,18 @@ struct TopbJobs {
 // eight CTAs each leave half of the thread slots idle.  Mask, concentration at two
 // budgets and state metrics of 28 rows of 25k: nine launches 248 us, four 204 (what
 // is left is mostly the host's: two copies of results and the calls).
-template <bool kSums>
+template <bool kSums, bool kCluster>
 __global__ void __launch_bounds__(kDiagThreads) topb_kernel(const __grid_constant__ TopbJobs jobs,
                                                             long long stride, double* out, int C)
 {
-    __shared__ __align__(16) unsigned hist[kTopbBins], merged[3][kTopbBins];
+    __shared__ __align__(16) unsigned hist[kTopbBins];
+    __shared__ __align__(16) unsigned merged[kCluster ? 3 : 1][kCluster ? kTopbBins : 1];
+    __shared__ __align__(16) unsigned eq_before[kDiagBatch * kDiagWarps];
     __shared__ unsigned wsum[kDiagWarps];
     __shared__ unsigned sh_bin, sh_count, sh_equal;
     __shared__ unsigned long long sh_k;
-    const int r = blockIdx.x % C, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long rowi = blockIdx.x / C;
+    const int r = kCluster ? blockIdx.x % C : 0, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long rowi = kCluster ? blockIdx.x / C : blockIdx.x;
     const long long n = jobs.job[blockIdx.y].n, B = jobs.job[blockIdx.y].B;
     const float* row = jobs.job[blockIdx.y].scores + static_cast<size_t>(rowi) * stride;
     uint8_t* mrow = kSums ? nullptr : jobs.job[blockIdx.y].mask + static_cast<size_t>(rowi) * stride;
@@ -190,14 +206,17 @@ __global__ void __launch_bounds__(kDiagThreads) topb_kernel(const __grid_constan
     unsigned long long ties = ~0ull;       // equal entries to keep, in position order (~0: all)
     if (!none && !all) {
         if (cached) load(lo);
-        for (int i = tid; i < 3 * kTopbBins; i += kDiagThreads) (&merged[0][0])[i] = 0;
-        ptx::cluster_sync();
+        if constexpr (kCluster) {
+            for (int i = tid; i < 3 * kTopbBins; i += kDiagThreads) (&merged[0][0])[i] = 0;
+            ptx::cluster_sync();
+        }
         unsigned long long k = static_cast<unsigned long long>(B);
 #pragma unroll 1
         for (int pass = 0; pass < 3; ++pass) {
             const int shift = pass == 0 ? 20 : pass == 1 ? 9 : 0;
             const unsigned dmask = pass == 2 ? 0x1FFu : 0x7FFu;
-            for (int i = tid; i < kTopbBins; i += kDiagThreads) hist[i] = 0;
+            static_assert(kTopbBins == 4 * kDiagThreads, "four bins per thread");
+            *reinterpret_cast<uint4*>(hist + 4 * tid) = make_uint4(0u, 0u, 0u, 0u);
             __syncthreads();
             for (long long base = lo; base < hi; base += kStep) {
                 if (!cached) load(base);
@@ -207,14 +226,19 @@ __global__ void __launch_bounds__(kDiagThreads) topb_kernel(const __grid_constan
                         atomicAdd(&hist[(bits(x[e]) >> shift) & dmask], 1u);
             }
             __syncthreads();
-            const uint32_t m0 = ptx::dsmem_addr(ptx::smem_addr(merged[pass]), 0);
-            for (int i = tid; i < kTopbBins; i += kDiagThreads)
-                if (hist[i]) red_dsmem_add(m0 + 4 * i, hist[i]);
-            ptx::cluster_sync();
             // the bin, from the largest digit down: thread t owns the four digits
-            // 2047 - 4 t - j (one 16-byte remote load: as four words, the eight
-            // CTAs' reads of one SM took 6 us a pass)
-            const float4 c4 = ptx::ld_dsmem_f4(m0 + 4 * (kTopbBins - 4 - 4 * tid));
+            // 2047 - 4 t - j (one 16-byte load: as four words, the eight CTAs'
+            // remote reads of one SM took 6 us a pass)
+            float4 c4;
+            if constexpr (kCluster) {
+                const uint32_t m0 = ptx::dsmem_addr(ptx::smem_addr(merged[pass]), 0);
+                for (int i = tid; i < kTopbBins; i += kDiagThreads)
+                    if (hist[i]) red_dsmem_add(m0 + 4 * i, hist[i]);
+                ptx::cluster_sync();
+                c4 = ptx::ld_dsmem_f4(m0 + 4 * (kTopbBins - 4 - 4 * tid));
+            } else {
+                c4 = *reinterpret_cast<const float4*>(hist + kTopbBins - 4 - 4 * tid);
+            }
             const unsigned c[4] = {__float_as_uint(c4.w), __float_as_uint(c4.z), __float_as_uint(c4.y),
                                    __float_as_uint(c4.x)};
             const unsigned local = c[0] + c[1] + c[2] + c[3];
@@ -246,42 +270,61 @@ __global__ void __launch_bounds__(kDiagThreads) topb_kernel(const __grid_constan
             if (sh_count == k) break;  // every entry of the bin is kept
             if (pass == 2) ties = k;
         }
-        if (ties != ~0ull) {
-            // the k lowest positions among the entries equal to the threshold: the
-            // CTAs' counts of them, in rank order, are in their last histograms
-            if (tid == 0) sh_equal = hist[thr & 0x1FFu];
-            ptx::cluster_sync();
-            unsigned long long before = 0;
-            for (int q = 0; q < r; ++q) before += ld_dsmem_u32(ptx::dsmem_addr(ptx::smem_addr(&sh_equal), q));
-            ties = before < ties ? ties - before : 0;
+        if constexpr (kCluster) {
+            if (ties != ~0ull) {
+                // the k lowest positions among the entries equal to the threshold: the
+                // CTAs' counts of them, in rank order, are in their last histograms
+                if (tid == 0) sh_equal = hist[thr & 0x1FFu];
+                ptx::cluster_sync();
+                unsigned long long before = 0;
+                for (int q = 0; q < r; ++q) before += ld_dsmem_u32(ptx::dsmem_addr(ptx::smem_addr(&sh_equal), q));
+                ties = before < ties ? ties - before : 0;
+            }
+            ptx::cluster_sync();  // no CTA leaves while others read its shared memory
         }
-        ptx::cluster_sync();  // no CTA leaves while others read its shared memory
     }
     // kept(j) <=> j < n and key(j) above the threshold, or equal and in time
     unsigned long long seen = 0;  // equal entries of this CTA's earlier batches
     double top = 0.0, rest = 0.0;
     for (long long base = lo; base < hi; base += kStep) {
         if (none || all ? kSums : !cached) load(base);
+        unsigned eq[kDiagBatch];  // lanes of the warp whose entry equals the threshold
+        if (ties != ~0ull) {
+            // how many come before, in position order: the warps' counts of the batch,
+            // entry e of every warp before entry e + 1, added up by the first warp (three
+            // barriers a batch; two for each e, 2000 rows of 64 equal scores took 83 us)
+            if (base > lo) __syncthreads();  // the previous batch's have been read
+#pragma unroll
+            for (int e = 0; e < kDiagBatch; ++e) {
+                eq[e] = __ballot_sync(0xffffffffu, base + tid + e * kDiagThreads < hi && (bits(x[e]) & tmask) == thr);
+                if (lane == 0) eq_before[e * kDiagWarps + warp] = __popc(eq[e]);
+            }
+            __syncthreads();
+            if (warp == 0) {
+                static_assert(kDiagBatch * kDiagWarps == 128, "four counts per lane");
+                uint4 q = *reinterpret_cast<const uint4*>(eq_before + 4 * lane);
+                const unsigned own = q.x + q.y + q.z + q.w;
+                unsigned incl = own;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                const unsigned b0 = incl - own;
+                q = make_uint4(b0, b0 + q.x, b0 + q.x + q.y, b0 + q.x + q.y + q.z);
+                *reinterpret_cast<uint4*>(eq_before + 4 * lane) = q;
+                if (lane == 31) sh_count = incl;
+            }
+            __syncthreads();
+        }
 #pragma unroll
         for (int e = 0; e < kDiagBatch; ++e) {
+            if (base + warp * 32 + e * kDiagThreads >= hi) break;  // nothing of the warp's
             const long long i = base + tid + e * kDiagThreads;
             const unsigned d = bits(x[e]) & tmask;
             bool keep = all || d > thr || (d == thr && ties == ~0ull);
-            if (ties != ~0ull) {  // rank of the equal entries, in position order (uniform branch)
-                const bool eq = i < hi && d == thr;
-                const unsigned bal = __ballot_sync(0xffffffffu, eq);
-                if (lane == 0) wsum[warp] = __popc(bal);
-                __syncthreads();
-                unsigned long long rank = seen + __popc(bal & ((1u << lane) - 1));
-                unsigned total = 0;
-                for (int w = 0; w < kDiagWarps; ++w) {
-                    if (w < warp) rank += wsum[w];
-                    total += wsum[w];
-                }
-                seen += total;
-                __syncthreads();
-                if (eq) keep = rank < ties;
-            }
+            if (ties != ~0ull && d == thr)
+                keep = seen + eq_before[e * kDiagWarps + warp] + __popc(eq[e] & ((1u << lane) - 1)) < ties;
             if constexpr (kSums) {
                 const bool in = i < hi && !none && keep;
                 const double t = (in ? top : rest) + __uint_as_float(x[e]);
@@ -291,13 +334,14 @@ __global__ void __launch_bounds__(kDiagThreads) topb_kernel(const __grid_constan
                 mrow[i] = !none && keep ? 1 : 0;
             }
         }
+        if (ties != ~0ull) seen += sh_count;
     }
     if constexpr (kSums) {
         __shared__ double sh[2 * kDiagWarps], part[2];
         double v[2] = {};
-        block_sum2(top, rest, sh, v);
+        block_sum2(top, rest, lo + warp * 32 < hi, sh, v);
         v[1] += v[0];
-        cluster_total(v, part, r, C, out + 2 * (blockIdx.y * static_cast<size_t>(gridDim.x / C) + rowi));
+        row_total<kCluster>(v, part, r, C, out + 2 * (blockIdx.y * static_cast<size_t>(gridDim.x / C) + rowi));
         return;
     }
     long long t0, t1;  // entries past n
@@ -305,14 +349,15 @@ __global__ void __launch_bounds__(kDiagThreads) topb_kernel(const __grid_constan
     for (long long j = n + t0 + tid; j < n + t1; j += kDiagThreads) mrow[j] = 0;
 }
 
+template <bool kCluster>
 __global__ void __launch_bounds__(kDiagThreads) concentration_kernel(const float* scores,
                                                                      const uint8_t* mask,
                                                                      long long n, long long stride,
                                                                      double* out, int C)
 {
     __shared__ double sh[2 * kDiagWarps], part[2];
-    const int r = blockIdx.x % C;
-    const long long rowi = blockIdx.x / C;
+    const int r = kCluster ? blockIdx.x % C : 0;
+    const long long rowi = kCluster ? blockIdx.x / C : blockIdx.x;
     const float* row = scores + static_cast<size_t>(rowi) * stride;
     const uint8_t* mrow = mask + static_cast<size_t>(rowi) * stride;
     long long lo, hi;
@@ -329,25 +374,27 @@ __global__ void __launch_bounds__(kDiagThreads) concentration_kernel(const float
         }
 #pragma unroll
         for (int e = 0; e < kDiagBatch; ++e) {
+            if (base + (threadIdx.x & ~31u) + e * kDiagThreads >= hi) break;  // nothing of the warp's
             const double t = (in[e] ? top : rest) + x[e];
             top = in[e] ? t : top;
             rest = in[e] ? rest : t;
         }
     }
     double v[2] = {};
-    block_sum2(top, rest, sh, v);
+    block_sum2(top, rest, lo + (threadIdx.x & ~31u) < hi, sh, v);
     v[1] += v[0];
-    cluster_total(v, part, r, C, out + 2 * rowi);
+    row_total<kCluster>(v, part, r, C, out + 2 * rowi);
 }
 
+template <bool kCluster>
 __global__ void __launch_bounds__(kDiagThreads) state_metrics_kernel(
     const uint8_t* mask_n, const uint8_t* mask_n1, const float* w, long long n_seen, int T,
     long long stride, double* out, int C)
 {
     __shared__ double sh[2 * kDiagWarps], part[6];
     __shared__ unsigned shi[kDiagWarps];
-    const int r = blockIdx.x % C;
-    const long long rowi = blockIdx.x / C;
+    const int r = kCluster ? blockIdx.x % C : 0;
+    const long long rowi = kCluster ? blockIdx.x / C : blockIdx.x;
     const size_t base0 = static_cast<size_t>(rowi) * stride;
     long long lo, hi;
     row_share(n_seen + T, r, C, lo, hi);
@@ -366,6 +413,7 @@ __global__ void __launch_bounds__(kDiagThreads) state_metrics_kernel(
         }
 #pragma unroll
         for (int e = 0; e < kDiagBatch; ++e) {
+            if (base + (threadIdx.x & ~31u) + e * kDiagThreads >= hi) break;  // nothing of the warp's
             cnt[0] += b[e] && pool[e];
             cnt[1] += b[e];
             cnt[2] += a[e] && b[e];
@@ -376,7 +424,7 @@ __global__ void __launch_bounds__(kDiagThreads) state_metrics_kernel(
         }
     }
     double wt[2] = {};
-    block_sum2(in_p, out_p, sh, wt);
+    block_sum2(in_p, out_p, lo + (threadIdx.x & ~31u) < hi, sh, wt);
     double v[6];
     v[0] = block_count(cnt[0], shi);
     v[1] = block_count(cnt[1], shi);
@@ -384,23 +432,29 @@ __global__ void __launch_bounds__(kDiagThreads) state_metrics_kernel(
     v[3] = wt[0] + wt[1];
     v[4] = block_count(cnt[2], shi);
     v[5] = block_count(cnt[3], shi);
-    cluster_total(v, part, r, C, out + 6 * rowi);
+    row_total<kCluster>(v, part, r, C, out + 6 * rowi);
 }
 
 // CTAs per row, a power of two up to 8 (the portable cluster size): no more than
-// give each about 2048 entries, and none added once the rows alone fill the SMs
-// twice.  28 rows of 25k scores: 50 us on one CTA
-// per row, 16 on eight (top-B).  (Several jobs a launch keep the C of one, so the
-// sums do too.)
+// give each 4096 entries (a batch, what its registers hold), and none added once the
+// rows alone fill the SMs twice.  Top-B of 28 rows, equal scores in brackets: 4096
+// entries 5.8 (6.5) us alone, 8.6 (9.6) on two; 8192 9.1 (10.2) on two, 9.8 (11.0) on
+// four, 8.9 (10.3) alone; 25k 42 us on one CTA per row with 8-bit digits, 19.4 (22.2)
+// on two, 15.0 (16.8) on four, 16.9 (18.0) on eight; 120 rows of 8192 11.7 (12.9) on
+// two, 17.6 (24.1) on four.  (Several jobs a launch keep the C of one, so the sums do
+// too.  The 152 SMs are written in: a call may come before any handle has read the
+// device's count, and the order of the sums should not follow it.)
 int row_cluster(int rows, long long n)
 {
     int C = 1;
-    while (C < 8 && n / (2 * C) >= 2048 && static_cast<long long>(rows) * C < 304) C *= 2;
+    while (C < 8 && n / (2 * C) >= kDiagBatch * kDiagThreads && static_cast<long long>(rows) * C < 2 * 152) C *= 2;
     return C;
 }
 
+// `clustered` on C CTAs per row, `alone` (no cluster, nothing to merge) where C is 1.
 template <class... KArgs, class... Args>
-cudaError_t launch_rows(void (*kernel)(KArgs...), int rows, int jobs, int C, cudaStream_t st, Args... args)
+cudaError_t launch_rows(void (*clustered)(KArgs...), void (*alone)(KArgs...), int rows, int jobs, int C,
+                        cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(rows) * C, static_cast<unsigned>(jobs));
@@ -412,8 +466,8 @@ cudaError_t launch_rows(void (*kernel)(KArgs...), int rows, int jobs, int C, cud
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args..., C);
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, C > 1 ? clustered : alone, args..., C);
 }
 
 }  // namespace
@@ -432,8 +486,8 @@ cudaError_t launch_topb_mask(const float* scores, int rows, long long n, long lo
     if (rows <= 0) return cudaSuccess;
     TopbJobs jobs{};
     jobs.job[0] = {scores, mask, n, B};
-    return launch_rows(topb_kernel<false>, rows, 1, row_cluster(rows, n), st, jobs, stride,
-                       static_cast<double*>(nullptr));
+    return launch_rows(topb_kernel<false, true>, topb_kernel<false, false>, rows, 1, row_cluster(rows, n), st, jobs,
+                       stride, static_cast<double*>(nullptr));
 }
 
 cudaError_t launch_topb_concentration(const float* scores, int rows, long long n, long long stride,
@@ -444,7 +498,8 @@ cudaError_t launch_topb_concentration(const float* scores, int rows, long long n
         const int nb = count - b0 < kTopbJobs ? count - b0 : kTopbJobs;
         TopbJobs jobs{};
         for (int i = 0; i < nb; ++i) jobs.job[i] = {scores, nullptr, n, budgets[b0 + i]};
-        const cudaError_t e = launch_rows(topb_kernel<true>, rows, nb, row_cluster(rows, n), st, jobs, stride,
+        const cudaError_t e = launch_rows(topb_kernel<true, true>, topb_kernel<true, false>, rows, nb,
+                                          row_cluster(rows, n), st, jobs, stride,
                                           out + static_cast<size_t>(b0) * rows * 2);
         if (e != cudaSuccess) return e;
     }
@@ -459,8 +514,8 @@ cudaError_t launch_topb_metrics(const float* scores_n, const float* scores_n1, i
     TopbJobs jobs{};
     jobs.job[0] = {scores_n, mask_n, n_seen, B};
     jobs.job[1] = {scores_n1, mask_n1, n_seen + T, B};
-    const cudaError_t e = launch_rows(topb_kernel<false>, rows, 2, row_cluster(rows, n_seen + T), st, jobs, stride,
-                                      static_cast<double*>(nullptr));
+    const cudaError_t e = launch_rows(topb_kernel<false, true>, topb_kernel<false, false>, rows, 2,
+                                      row_cluster(rows, n_seen + T), st, jobs, stride, static_cast<double*>(nullptr));
     return e != cudaSuccess ? e
                             : launch_state_metrics(mask_n, mask_n1, scores_n1, rows, n_seen, T, stride, out, st);
 }
@@ -469,7 +524,8 @@ cudaError_t launch_concentration(const float* scores, const uint8_t* mask, int r
                                  long long stride, double* out, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    return launch_rows(concentration_kernel, rows, 1, row_cluster(rows, n), st, scores, mask, n, stride, out);
+    return launch_rows(concentration_kernel<true>, concentration_kernel<false>, rows, 1, row_cluster(rows, n), st,
+                       scores, mask, n, stride, out);
 }
 
 cudaError_t launch_state_metrics(const uint8_t* mask_n, const uint8_t* mask_n1, const float* w,
@@ -477,8 +533,8 @@ cudaError_t launch_state_metrics(const uint8_t* mask_n, const uint8_t* mask_n1, 
                                  cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
-    return launch_rows(state_metrics_kernel, rows, 1, row_cluster(rows, n_seen + T), st, mask_n, mask_n1, w,
-                       n_seen, T, stride, out);
+    return launch_rows(state_metrics_kernel<true>, state_metrics_kernel<false>, rows, 1,
+                       row_cluster(rows, n_seen + T), st, mask_n, mask_n1, w, n_seen, T, stride, out);
 }
 
 }  // namespace statekv

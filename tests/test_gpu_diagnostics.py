@@ -220,3 +220,33 @@ def test_fused_statistics_equal_the_separate_kernels(rows, n, stride):
         assert statekv.statekv_state_metrics(a.data_ptr(), b.data_ptr(), other.data_ptr(), rows, seen, T,
                                              stride, ref.data_ptr(), stream) == 0
         assert torch.equal(out, ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,n,stride", [
+    (7, 64, 70), (400, 100, 101), (3, 511, 512), (3, 513, 513),  # warps without entries
+    (2, 4096, 4097), (5, 4097, 4100),   # one CTA: a whole batch, and one entry more
+    (5, 8191, 8200), (5, 8193, 8300),   # the last length of one CTA, then two
+    (1, 32768, 32768), (2, 32769, 32770),  # eight CTAs, a batch each, and one entry more
+])
+def test_rows_around_the_cluster_rule(rows, n, stride):
+    """The same checks at the lengths where the form or the cluster size changes."""
+    test_row_kernels_over_cluster_sizes(rows, n, stride)
+    test_fused_statistics_equal_the_separate_kernels(rows, n, stride)
+
+
+@pytest.mark.gpu
+def test_topb_of_a_few_entries():
+    """Rows of one to nine entries with zeros, negative entries, infinities and NaN, every budget."""
+    _need_gpu()
+    for n in range(1, 10):
+        vals = np.array([[0.0, 2.0, -1.0, np.inf, 2.0, np.nan, 0.0, np.inf, 1.0][:n]] * 2, np.float32)
+        vals[1] = vals[1, ::-1]
+        g = torch.as_tensor(vals, device="cuda")
+        for B in range(n + 2):
+            mask = diagnostics.topb_mask(g, n, B).cpu().numpy()
+            rank = np.where(vals > 0, vals, 0).astype(np.float64)  # negative entries and NaN rank as 0
+            for r in range(2):
+                want = np.zeros(n, np.uint8)
+                want[np.lexsort((np.arange(n), -rank[r]))[:B]] = 1
+                assert np.array_equal(mask[r], want), (n, B, r)
