@@ -340,10 +340,12 @@ statekv_status run_step(statekv_handle* h, const statekv_frame_args& a, cudaStre
     pa.watchdog_ns = 1000000ull * (c.watchdog_ms ? c.watchdog_ms : 2000u);
     const cudaError_t ek =
         timed(h, 1, st, [&] { return launch_attn(D, h->tm_sk, h->tm_sv, tm_fk, tm_fv, pa, U, st); });
-    if (ek != cudaSuccess) return STATEKV_ERR_CUDA;
+    // the append is done; joined also where the attention kernel could not be launched:
+    // later work on the stream must not pass it, and a capture must not end with it open
+    const cudaError_t ej = c.selection == 1 ? cudaStreamWaitEvent(st, h->ev_join, 0) : cudaSuccess;
+    if (ek != cudaSuccess || ej != cudaSuccess) return STATEKV_ERR_CUDA;
 
     if (c.selection == 1) {
-        if (cudaStreamWaitEvent(st, h->ev_join, 0) != cudaSuccess) return STATEKV_ERR_CUDA;  // the append is done
         RecencyParams pr{};
         pr.k = ap.k;
         pr.v = ap.v;

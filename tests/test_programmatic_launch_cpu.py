@@ -24,3 +24,12 @@ def test_the_selection_and_its_append_wait_before_they_read():
         for r in reads:
             assert r in part, r
             assert wait in part[: part.index(r)], f"{r} before the wait"
+
+
+def test_the_side_stream_is_joined_before_a_failed_launch_returns():
+    """Recency window: once the append is on the side stream, nothing returns before the
+    call's stream waits for it (no launch fails on demand, so the source is read)."""
+    body = kernel_body("statekv_api.cu", "statekv_status run_step")
+    forked = body[body.index("cudaEventRecord(h->ev_join"):]
+    between = forked[forked.index("return STATEKV_ERR_CUDA;") + 1: forked.index("cudaStreamWaitEvent(st, h->ev_join")]
+    assert "launch_attn(" in between and "return STATEKV_ERR" not in between
