@@ -58,6 +58,9 @@ struct DecLayout {
     static_assert(kDecWarps * kDecodeRows * (D + 8) * 4 + 2 * kDecWarps * kDecodeRows * 4 <= kOffBar &&
                       kDecodeRows * (kDecodeMaxChunks + 1) * 4 + kDecodeRows * D * 4 <= kOffBar,
                   "merge areas fit");
+    // chunks whose partials of 16 rows fit the staging memory at once (23 at D = 128)
+    static_assert((kOffBar - kDecodeRows * (kDecodeMaxChunks + 1) * 4) / (kDecodeRows * D * 4) >= 22,
+                  "merge of every chunk in three rounds at most");
     static_assert(kBlock % 1024 == 0, "swizzle atoms stay aligned");
 };
 
@@ -420,7 +423,7 @@ __global__ void __launch_bounds__(kDecThreads)
     float* rows = den + kDecodeRows;                            // [chunks of a round][R][D]
     uint64_t* landed = reinterpret_cast<uint64_t*>(dsm + L::kOffBar) + kDecWarps * kDecStages;
     const int nc = p.nchunk, items = R * (D / 4);
-    const int round = (L::kOffBar - kDecodeRows * (kDecodeMaxChunks + 1) * 4) / (R * D * 4);  // >= 5 chunks
+    const int round = (L::kOffBar - kDecodeRows * (kDecodeMaxChunks + 1) * 4) / (R * D * 4);  // >= 22 chunks
     const size_t hbase = (static_cast<size_t>(u) * p.Hkv + hkv) * nc;
     auto fetch = [&](int c0) {  // warp 0: chunks [c0, c0 + round) into `rows`
         const int cnt = min(round, nc - c0);

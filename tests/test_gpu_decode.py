@@ -163,3 +163,15 @@ def test_decode_token_edges(hq, hkv, d, T, frames, layers, steps):
             assert np.array_equal(oracle.as_bf16_bits(cv[:, :done + nt].transpose(0, 1)), vs)
         done += nt
     assert eng.sync() == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hq,d,T,frames,steps", [
+    (16, 128, 1020, 8, (1, 1)),  # 16 rows over 64 chunks: merged 23 at a time, in three rounds
+    (16, 64, 1020, 8, (1,)),     # 22 at a time
+    (8, 128, 1020, 8, (2,)),     # two tokens of eight heads
+    (16, 128, 700, 8, (1,)),     # 44 chunks, two rounds
+])
+def test_decode_merges_in_several_rounds(hq, d, T, frames, steps):
+    """One head of 16 query rows over more chunks than the staging memory holds at once."""
+    test_decode_token_edges(hq, 1, d, T, frames, 1, steps)
