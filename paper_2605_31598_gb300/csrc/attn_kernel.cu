@@ -1039,7 +1039,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             __syncwarp();
             cluster_sync();  // phase 2
-            if (ok) {
+            if (ok && p.out != nullptr) {  // (the watchdog self-test has no output)
                 const int rank = static_cast<int>(cluster_ctarank());
                 const int r0 = kBM * rank / p.split, r1 = kBM * (rank + 1) / p.split;
                 const uint32_t a0 = smem_addr(ost);
@@ -1180,7 +1180,7 @@ cudaError_t launch_one(const CUtensorMap& tm_sk, const CUtensorMap& tm_sv, const
     const long long W = static_cast<long long>(p.MT) * p.Hkv * U;
     if (W <= 0) return cudaSuccess;
     if (W > 0x7FFFFFFFll) return cudaErrorInvalidValue;
-    p.split = p.selftest_stall ? 1 : split_for<D>(W, (p.keys_hint + kBN - 1) / kBN + (p.T + kBN - 1) / kBN);
+    p.split = split_for<D>(W, (p.keys_hint + kBN - 1) / kBN + (p.T + kBN - 1) / kBN);
     const int sms = current_device_sms();
     const int grid = p.split > 1 ? static_cast<int>(W) * p.split : static_cast<int>(W < sms ? W : sms);
     cudaLaunchAttribute attr[2];

@@ -1283,7 +1283,8 @@ statekv_status statekv_watchdog_selftest(statekv_handle* h, statekv_stream strea
     const statekv_config& c = h->cfg;
     // One work unit (stream 0, layer 0) whose producer first waits on a barrier
     // that nothing completes: no input is read, no copy or MMA is issued, and
-    // every role of the CTA leaves through its bounded waits.
+    // every role of the CTA (of each CTA of a cluster, where a frame step of the
+    // unit would take one) leaves through its bounded waits.
     AttnParams pa{};
     pa.counts = h->at<int32_t>(h->lay.counts);
     pa.status = h->status_dev;
@@ -1297,6 +1298,7 @@ statekv_status statekv_watchdog_selftest(statekv_handle* h, statekv_stream strea
     pa.MT = h->d.MT;
     pa.causal = c.causal_in_frame;
     pa.count_mul = 1;
+    pa.keys_hint = static_cast<int>(std::min<long long>(c.state_capacity, most_rows(h, 0, 1, 0, 1)));
     pa.scale_log2 = h->d.scale * 1.4426950408889634f;
     pa.watchdog_ns = 1000000ull * (c.watchdog_ms ? c.watchdog_ms : 2000u);
     pa.selftest_stall = 1;

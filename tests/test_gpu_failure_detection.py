@@ -81,3 +81,28 @@ def test_waiting_for_the_previous_kernel_is_not_a_timeout(shape, hidden):
         eng.close()
     assert weights and torch.isfinite(outs[0].float()).all()
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("shape,frames", [
+    (Shape(2, 1, 128, 64, 1100, 22), 18),   # one unit of ten key tiles: eight CTAs
+    (Shape(6, 3, 64, 37, 1900, 60), 52),    # three units
+])
+def test_expired_wait_of_a_cluster_is_reported(shape, frames):
+    """The self-test on the attention kernel's form for few units over many keys, a
+    cluster of CTAs each: every CTA's waits run out, all of them pass the cluster's
+    barriers, and the launch ends with the self-test's site."""
+    eng = StateKV(make_config(shape, watchdog_ms=100))
+    for n in range(1, frames + 1):
+        q, k, v = batch_qkv(shape, n, streams=[0], layers=[0], device="cuda")
+        assert eng.prefill_frame(q, k, v, torch.empty_like(q)) == 0
+    assert eng.sync() == 0
+    t0 = time.monotonic()
+    assert eng.watchdog_selftest() == 0
+    assert eng.sync() == DEVICE_TIMEOUT
+    assert time.monotonic() - t0 < 10.0
+    code = eng.device_error()
+    assert code & 0xFF == 1 and (code >> 8) & 0xFF == 1, hex(code)
+    fresh = StateKV(make_config(shape))
+    out = torch.full_like(q, float("nan"))
+    assert fresh.prefill_frame(q, k, v, out) == 0 and fresh.sync() == 0
+    assert torch.isfinite(out.float()).all()
