@@ -199,13 +199,6 @@ __device__ __forceinline__ void store_rows4(const GemmParams& p, int mrow0, int 
     store4_rows<8>(p, mrow0 + sub, 4, nrows < 8 ? nrows : 8, n, acc);
 }
 
-template <int NR>
-__device__ __forceinline__ void store_rows_strided(const GemmParams& p, int m0, int mstep, int nrows,
-                                                   int n, float4 (&a)[NR])
-{
-    store4_rows<NR>(p, m0, mstep, nrows, n, a);
-}
-
 __global__ void __launch_bounds__(kGThreads, 1)
     gemm_bf16_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                  const GemmParams p)
@@ -471,7 +464,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                             a[i].w += bias[3];
                         }
                         // pair row r = tile row (r >= 128: second tile) -> global row m0 + r
-                        store_rows_strided(p, x.m0 + rb, 4, min(kRG, (r1 - rb + 3) / 4), n, a);
+                        store4_rows<kRG>(p, x.m0 + rb, 4, min(kRG, (r1 - rb + 3) / 4), n, a);
                     }
                 }
             }
@@ -683,7 +676,6 @@ __global__ void __launch_bounds__(kPThreads, 1)
         float* stg = reinterpret_cast<float*>(epi) + (warp - 2) * 32 * kGStageLd;
         const int sub = lane >> 3, c4 = lane & 7;
         const uint32_t bae = dsmem_addr(smem_addr(acc_empty), 0);
-        const bool vec = (p.N & 3) == 0;  // whole groups of four columns, 8-byte aligned
         pdl_wait();
         bool ok = true;
         uint32_t u = 0;
@@ -707,7 +699,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             uint2 old[8];
             auto load_old = [&](int i) {
                 const int b = i >= chunks ? 1 : 0, c = i - b * chunks, n = ncol + 256 * b;
-                if (!p.add || !vec || i >= items || n >= p.N) return;
+                if (!p.add || i >= items || n >= p.N) return;
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const int r = 32 * c + 4 * q + sub;
@@ -748,9 +740,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 for (int q = 0; q < 8; ++q)
                     acc[q] = *reinterpret_cast<const float4*>(stg + (4 * q + sub) * kGStageLd + 4 * c4);
                 const int n = ncol + 256 * b;
-                if (!vec) {
-                    store_rows4(p, m0 + 32 * c, sub, min(32, mend - 32 * c), n, acc);
-                } else if (n < p.N) {
+                if (n < p.N) {  // (N is a multiple of 4: whole groups of columns, 8-byte aligned)
                     uint2 o[8];
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
@@ -1269,7 +1259,7 @@ cudaError_t launch_gemm(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const 
     if (p.units <= 0) return cudaSuccess;
     if (p.paired_I && (p.splits != 1 || p.paired_I != p.N || p.bias || p.add)) return cudaErrorInvalidValue;
     if (p.pair_bn) {
-        if (p.splits != 1 || p.pair_bn < kPairMinBN || p.pair_bn > kPairMaxBN || p.pair_bn % 32)
+        if (p.splits != 1 || p.pair_bn < kPairMinBN || p.pair_bn > kPairMaxBN || p.pair_bn % 32 || p.N % 4)
             return cudaErrorInvalidValue;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(2 * std::max(1, std::min(p.units, sms / 2)));

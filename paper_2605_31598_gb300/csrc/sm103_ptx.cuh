@@ -55,15 +55,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
     return done != 0;
 }
 
-// Waits for the phase with the given parity to complete.  Returns false if
-// `limit` polls pass first (each try_wait itself blocks for a bounded time).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit)
-{
-    for (uint32_t i = 0; i < limit; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-
 // ---------------------------------------------------------------- proxies
 // Orders this thread's generic-proxy shared-memory writes before later
 // async-proxy reads (tcgen05.mma operands, TMA stores).
@@ -130,20 +121,7 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // memory operations are visible.  Both are no-ops without the launch attribute.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// ---------------------------------------------------------------- bulk stores
-// shared -> global copy of `bytes` (a multiple of 16; both addresses 16-byte
-// aligned) through the TMA engine, tracked by the issuing thread's bulk group
-__device__ __forceinline__ void bulk_store(void* gdst, const void* ssrc, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                 :: "l"(gdst), "r"(smem_addr(ssrc)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// every committed bulk store of this thread has read its shared source
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// every committed bulk store of this thread has completed
-__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
+// ---------------------------------------------------------------- bulk loads
 // global -> shared copy of `bytes` (a multiple of 16; both addresses 16-byte
 // aligned), counted on the mbarrier
 __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar)
@@ -156,16 +134,6 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap)
 {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, uint64_t* bar, int c0,
-                                            int c1)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_addr(dst)),
-        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_addr(bar)), "r"(c0), "r"(c1)
-        : "memory");
 }
 
 __device__ __forceinline__ void tma_load_4d(void* dst, const void* tmap, uint64_t* bar, int c0,
@@ -220,16 +188,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// Arrives once on `bar` when every tcgen05.mma this thread issued so far has
-// completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar)
-{
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_addr(bar))
         : "memory");
 }
 
@@ -317,6 +275,7 @@ __device__ __forceinline__ void umma_ss(uint32_t d, uint64_t a, uint64_t b, uint
 {
     if (elect_one()) umma_bf16(d, a, b, idesc, accumulate);
 }
+// arrives once on `bar` when every tcgen05.mma issued so far has completed
 __device__ __forceinline__ void commit_elect(uint32_t bar)
 {
     if (elect_one())
@@ -424,13 +383,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool a_mn_ma
            | (static_cast<uint32_t>(b_mn_major) << 16) // B major-ness
            | (static_cast<uint32_t>(N >> 3) << 17)     // N / 8
            | (static_cast<uint32_t>(M >> 4) << 24);    // M / 16
-}
-
-// Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a
-// 128-byte-swizzled tile whose rows are 128 B apart.
-__host__ __device__ constexpr uint32_t sw128_offset(uint32_t row, uint32_t chunk)
-{
-    return row * 128u + ((chunk ^ (row & 7u)) << 4);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)

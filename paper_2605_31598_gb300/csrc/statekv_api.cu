@@ -1026,11 +1026,10 @@ statekv_status statekv_block_frame(statekv_handle* h, const statekv_block_config
         gp.K = K;
         gp.pair_bn = g.pair_bn;
         gp.paired_I = paired ? pair_I : 0;
-        gp.n_tiles = paired ? (pair_I + gb.cols - 1) / gb.cols : g.n_tiles;
         gp.k_steps = g.k_steps;
         gp.kps = g.kps;
         gp.splits = g.splits;
-        gp.units = paired ? gp.n_tiles * (g.units / g.n_tiles) : g.units;
+        gp.units = paired ? (pair_I + gb.cols - 1) / gb.cols * (g.units / g.n_tiles) : g.units;
         gp.bias = static_cast<const __nv_bfloat16*>(bias);
         gp.D = paired ? D_pair : D;
         gp.add = add ? 1 : 0;

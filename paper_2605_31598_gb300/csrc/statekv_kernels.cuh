@@ -211,7 +211,7 @@ inline GemmBox gemm_box(const GemmPlan& g, bool paired)
 struct GemmParams {
     int M, N, K;
     int pair_bn;                // the plan's
-    int n_tiles, k_steps, kps, splits, units;
+    int k_steps, kps, splits, units;
     int paired_I;               // > 0: W = gate rows [0, I) then up rows [I, 2 I), D = SiLU(gate) * up
                                 // [M][I] (N = I); the W map is [2][I][K]; tile t covers output columns
                                 // [gemm_box(..).cols t, .. (t + 1)); splits = 1
@@ -219,7 +219,7 @@ struct GemmParams {
     __nv_bfloat16* D;           // [M][N]
     int add;                    // 1: D += X W^T
     float* partials;            // splits > 1: [units][2][128][128]
-    int* counters;              // splits > 1: [n_tiles * m_pairs], zero on entry, used once
+    int* counters;              // splits > 1: one per tile (the plan's `counters`), zero on entry, used once
     int32_t* status;
     unsigned long long watchdog_ns;
 };
