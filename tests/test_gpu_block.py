@@ -14,6 +14,7 @@ of the attention term.  Selections agree outside the 1e-3 band
 of the oracle's importance, and the decode caches hold the GPU's own
 rotated K/V rows bit for bit.
 """
+import ctypes
 import dataclasses
 import math
 
@@ -23,7 +24,7 @@ import torch
 
 import oracle
 from oracle import block as ob
-from paper_2605_31598_gb300 import StateKV, make_config
+from paper_2605_31598_gb300 import StateKV, make_config, statekv
 from paper_2605_31598_gb300.inputs import (BLOCKS, WORKLOADS, Shape, block_input,
                                            block_weights)
 from paper_2605_31598_gb300.statekv import block_weights_array, statekv_block_config
@@ -262,3 +263,50 @@ def test_block_paired_ctas_ragged_tiles():
     stats = {}
     worst = run_block_parity(shape, BlockShape(2112, 2112), 2, check_frames=[2], stats=stats)
     print("paired ragged block worst |dx|", worst, stats)
+
+
+class _GemmPlan(ctypes.Structure):
+    """The library's GemmPlan (csrc/statekv_kernels.cuh)."""
+    _fields_ = [(n, ctypes.c_int) for n in ("pair_bn", "n_tiles", "m_pairs", "k_steps", "kps",
+                                            "splits", "units", "counters")]
+    _fields_ += [("partial_bytes", ctypes.c_size_t)]
+
+
+def _pair_plan(rows, n, k, gate_up=False):
+    """(X rows per tile, tiles) of the CTA-pair GEMM for this product; (0, _): not on pairs."""
+    plan = statekv.lib()["_ZN7statekv9gemm_planEiiii"]  # statekv::gemm_plan(int, int, int, int)
+    plan.restype, plan.argtypes = _GemmPlan, [ctypes.c_int] * 4
+    p = plan(rows, n, k, torch.cuda.get_device_properties(0).multi_processor_count)
+    per_row = -(-(n // 2) // 256) if gate_up else p.n_tiles
+    return p.pair_bn, per_row * (p.units // p.n_tiles)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("streams,tokens,hidden,hq,hkv,d,inter,want", [
+    # the narrowest tile; 280 rows
+    (2, 140, 2048, 16, 2, 64, 5000, {"gate_up": (96, 60)}),
+    # the widest tile, whose ring has three stages, with bias, SiLU and residual
+    (11, 205, 3136, 32, 4, 64, 2048,
+     {"qkv": (160, 75), "o": (256, 63), "gate_up": (256, 72), "down": (256, 63)}),
+    # 76 pairs: a second tile per pair with the residual
+    (18, 196, 3136, 32, 4, 64, 2048,
+     {"qkv": (256, 70), "o": (192, 133), "gate_up": (192, 152), "down": (192, 133)}),
+    # a second tile per pair with bias, on the three-stage ring
+    (14, 193, 2048, 32, 8, 128, 2048,
+     {"qkv": (256, 132), "o": (160, 68), "gate_up": (160, 136), "down": (160, 68)}),
+])
+def test_block_on_cta_pairs(streams, tokens, hidden, hq, hkv, d, inter, want):
+    """Every tile width of the CTA-pair GEMM not met above, and pairs that take a second
+    tile; the plans are those the cases are for (on 152 SMs)."""
+    from paper_2605_31598_gb300.inputs import BlockShape
+
+    _need_gpu()
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        rows = streams * tokens
+        plans = {"qkv": _pair_plan(rows, (hq + 2 * hkv) * d, hidden), "o": _pair_plan(rows, hidden, hq * d),
+                 "gate_up": _pair_plan(rows, 2 * inter, hidden, True), "down": _pair_plan(rows, hidden, inter)}
+        assert {k: v for k, v in plans.items() if v[0]} == want
+    shape = Shape(hq, hkv, d, tokens, tokens + 12, 2, num_layers=1, num_streams=streams)
+    stats = {}
+    worst = run_block_parity(shape, BlockShape(hidden, inter), 2, check_frames=[2], stats=stats)
+    print(f"pairs {want} worst |dx|", worst, stats)
