@@ -1212,7 +1212,10 @@ GemmPlan gemm_plan(int M, int N, int K, int sms)
     // Pairs of CTAs, when the 128-wide tiles fill the SMs (with fewer, splitting
     // their K is faster) and rounds x cycles per K step come out lower; the
     // accumulators' read-out, which the pair does not overlap, counts as four K
-    // steps.  Only with K long enough to carry it and 128-byte aligned rows.
+    // steps, and rows are 128-byte aligned.  Below 32 K steps that count is too low
+    // where a pair takes several tiles: a layer at 8 streams of hidden 1536, MLP 8960
+    // takes 240 us on 128-wide tiles and 250 on pairs, of hidden 1984 269 and 276
+    // (with one tile per pair they would gain: two streams of 1536 132 and 127).
     if (narrow >= sms && g.k_steps >= 32 && (K % 64) == 0) {
         double best = (narrow + sms - 1) / sms * static_cast<double>(g.k_steps) * kNarrowCycles;
         for (int bn = kPairMinBN; bn <= kPairMaxBN; bn += 32) {
