@@ -12,7 +12,7 @@
 // (first in it, the wait cost 4 us of 227 at 28 layers; last, none).  (As a launch of
 // its own on a side stream the append needed two events per frame and kept the other
 // two kernels from overlapping.  Per frame, before and after: toy 17.2 and 12.1 us,
-// one 7B layer 32.5 and 28.5, four small-backbone layers 34.6 and 25.5.)
+// one 7B layer 32.5 and 27.7, four small-backbone layers 34.6 and 25.6.)
 //   1. importance of every pool member = the fixed-order sum of the attention
 //      kernel's per-query-tile partials (deterministic); with layer-level
 //      selection (App. A) the ranking score is the same sum taken over every
@@ -105,9 +105,9 @@ __device__ __forceinline__ void tiles_sum(const float* x, int MT, int stride, co
 // pool 4355 168 us a frame by twos, 110 by eights (133 was eights for every pool on
 // the 8-bit selection); 12 layers of 12 heads, pool 1257 56 and 66 us.
 constexpr int kMem = 2, kMemFewTiles = 8;
-int select_members(const SelectParams& p, int split)
+int select_members(const SelectParams& p)
 {
-    return split == 1 && (p.P & 3) != 0 && p.MT <= 4 && p.shared && p.P > 2 * kMem * kSelThreads ? kMemFewTiles : kMem;
+    return (p.P & 3) != 0 && p.MT <= 4 && p.shared && p.P > 2 * kMem * kSelThreads ? kMemFewTiles : kMem;
 }
 
 // For 4 adjacent columns c0..c0+3 (16-byte aligned): the sums of
@@ -189,9 +189,11 @@ static_assert(kBins / 4 <= kSelThreads && kBins % 128 == 0, "four bins per threa
 
 // kSplit: a cluster of p.split CTAs makes the keys of a head, each from its share of
 // the pool's columns; they meet in the first CTA's shared memory, which goes on alone.
-// kMembers: see select_members (an instantiation of its own: as a branch of one kernel
-// the second form cost the first 2 to 5%).
-template <bool kSplit, int kMembers>
+// kMembers: see select_members; Index: the append's, see append_narrow.  They are
+// instantiations of their own: as branches of one kernel, never taken, the eight-member
+// sums cost the other forms 2 to 5%, and the 64-bit append 0.6 us of a toy frame's 12.1
+// and 1.1 of the 27.7 of one 7B layer.
+template <bool kSplit, int kMembers, class Index>
 __global__ void __launch_bounds__(kSelThreads)
     state_select_gather(const SelectParams p)
 {
@@ -208,10 +210,7 @@ __global__ void __launch_bounds__(kSelThreads)
         ptx::pdl_wait();  // K, V and the counters, written before the attention kernel
         const int u = app / p.appenders;
         const int nf0 = p.frames[static_cast<size_t>(p.units.unit_abs(u)) * p.Hkv];
-        if (append_narrow(p.T, p.Hkv, p.D))
-            append_share<int>(p, u, app - u * p.appenders);
-        else
-            append_share<long long>(p, u, app - u * p.appenders);
+        append_share<Index>(p, u, app - u * p.appenders);
         finish_unit(p, u, nf0);
         return;
     }
@@ -602,8 +601,8 @@ size_t select_smem_bytes(int P, int T)
 cudaError_t select_prepare()
 {
     const int bytes = static_cast<int>(select_smem_bytes(kMaxPool, kMaxFrameTokens));
-    for (auto kernel : {state_select_gather<true, kMem>, state_select_gather<false, kMem>,
-                        state_select_gather<false, kMemFewTiles>}) {
+    for (auto kernel : {state_select_gather<true, kMem, int>, state_select_gather<false, kMem, int>,
+                        state_select_gather<false, kMemFewTiles, int>, state_select_gather<false, kMem, long long>}) {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
     }
@@ -650,9 +649,11 @@ cudaError_t launch_select(const SelectParams& p, int U, cudaStream_t st)
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = q.split > 1 ? 2 : 1;
-    const auto kernel = q.split > 1                                     ? state_select_gather<true, kMem>
-                        : select_members(p, q.split) == kMemFewTiles ? state_select_gather<false, kMemFewTiles>
-                                                                     : state_select_gather<false, kMem>;
+    // (thousands of heads, as the 64-bit append takes, are never split)
+    const auto kernel = q.split > 1                             ? state_select_gather<true, kMem, int>
+                        : !append_narrow(p.T, p.Hkv, p.D)       ? state_select_gather<false, kMem, long long>
+                        : select_members(p) == kMemFewTiles     ? state_select_gather<false, kMemFewTiles, int>
+                                                                : state_select_gather<false, kMem, int>;
     return cudaLaunchKernelEx(&cfg, kernel, q);
 }
 
