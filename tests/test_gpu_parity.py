@@ -443,3 +443,26 @@ def test_layer_selection_is_exact_with_few_query_tiles(name, monkeypatch):
     shape, frames = FEW_TILES[name]
     monkeypatch.setitem(SELECT, name, (shape, False, frames))
     test_selection_is_exact_for_the_exported_importance(name, 2)
+
+
+def test_append_with_64_bit_indexes():
+    """One frame of 4096 tokens of 16,384 KV heads of 128 (2^31 copies of 16 bytes): every
+    row is in the decode cache.  About 95 GB on the device."""
+    if torch.cuda.mem_get_info()[0] < 120e9:
+        pytest.skip("needs 120 GB of free device memory")
+    H, T, d = 16384, 4096, 128
+    eng = StateKV(make_config(Shape(H, H, d, T, 0, 1)))
+    g = torch.Generator(device="cuda")
+    g.manual_seed(0)
+    k, v = (torch.empty((1, 1, T, H, d), dtype=torch.bfloat16, device="cuda").normal_(generator=g) for _ in range(2))
+    out = torch.empty_like(k)
+    assert eng.prefill_frame(k, k, v, out) == 0
+    assert eng.sync() == 0
+    ck, cv, info = eng.cache(0, 0)
+    assert info.length == T
+    for h in range(0, H, 2048):
+        for rows, src in ((ck, k), (cv, v)):
+            assert torch.equal(rows[h:h + 2048], src[0, 0, :, h:h + 2048].transpose(0, 1)), h
+    eng.close()
+    del eng, k, v, out, ck, cv
+    torch.cuda.empty_cache()
