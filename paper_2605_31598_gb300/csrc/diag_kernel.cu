@@ -435,19 +435,27 @@ __global__ void __launch_bounds__(kDiagThreads) state_metrics_kernel(
     row_total<kCluster>(v, part, r, C, out + 6 * rowi);
 }
 
-// CTAs per row, a power of two up to 8 (the portable cluster size): no more than
-// give each 4096 entries (a batch, what its registers hold), and none added once the
-// rows alone fill the SMs twice.  Top-B of 28 rows, equal scores in brackets: 4096
-// entries 5.8 (6.5) us alone, 8.6 (9.6) on two; 8192 9.1 (10.2) on two, 9.8 (11.0) on
-// four, 8.9 (10.3) alone; 25k 42 us on one CTA per row with 8-bit digits, 19.4 (22.2)
-// on two, 15.0 (16.8) on four, 16.9 (18.0) on eight; 120 rows of 8192 11.7 (12.9) on
-// two, 17.6 (24.1) on four.  (Several jobs a launch keep the C of one, so the sums do
-// too.  The 152 SMs are written in: a call may come before any handle has read the
-// device's count, and the order of the sums should not follow it.)
+// CTAs per row, a power of two up to 8 (the portable cluster size): doubled while the
+// row's share is more than a batch (4096 entries, what a CTA's registers hold) and the
+// CTAs of all rows stay one per SM (sixteen clusters of eight, two per GPC of 19 SMs), or
+// three per SM while a share is more than eight batches.  Top-B of 28 rows, with equal
+// scores in brackets, on 1, 2, 4 and 8 CTAs a row: 4097 entries 7.5 (8.8), 8.6 (9.6), 9.3
+// (10.6), 14.0 (16.9) us; 9000 10.6 (12.5), 12.8 (14.4), 9.8 (11.1), 13.0 (16.9); 25k 24.3
+// (25.3), 21.6 (22.2), 16.4 (16.8), 17.1 (18.2); sums and metrics prefer two to one from
+// 4097 on (4097 13.7 and 11.7 us together).  8 rows of 25k 21.1, 19.4, 14.9, 12.6; 152 rows
+// of 25k 21.3, 25.9, 34.9, 55.2; 100 rows of 80k 68.8, 55.3, 46.1, 64.1.  (Several jobs a
+// launch keep the C of one, so the sums do too.  The 152 SMs are written in: a call may
+// come before any handle has read the device's count, and the order of the sums should not
+// follow it.)
 int row_cluster(int rows, long long n)
 {
+    constexpr long long kBatch = kDiagBatch * kDiagThreads, kSms = 152;
     int C = 1;
-    while (C < 8 && n / (2 * C) >= kDiagBatch * kDiagThreads && static_cast<long long>(rows) * C < 2 * 152) C *= 2;
+    while (C < 8 && n > C * kBatch) {
+        const long long ctas = 2ll * C * rows;
+        if (ctas > (n > 8 * C * kBatch ? 3 * kSms : C == 4 ? 128 : kSms)) break;
+        C *= 2;
+    }
     return C;
 }
 

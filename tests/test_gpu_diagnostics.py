@@ -225,9 +225,12 @@ def test_fused_statistics_equal_the_separate_kernels(rows, n, stride):
 @pytest.mark.gpu
 @pytest.mark.parametrize("rows,n,stride", [
     (7, 64, 70), (400, 100, 101), (3, 511, 512), (3, 513, 513),  # warps without entries
-    (2, 4096, 4097), (5, 4097, 4100),   # one CTA: a whole batch, and one entry more
-    (5, 8191, 8200), (5, 8193, 8300),   # the last length of one CTA, then two
-    (1, 32768, 32768), (2, 32769, 32770),  # eight CTAs, a batch each, and one entry more
+    (2, 4096, 4097),                       # one CTA a row, a whole batch
+    (76, 4097, 4100), (77, 4097, 4097),    # two; one, as 77 rows of two are more than the SMs
+    (5, 8192, 8200), (5, 8193, 8300),      # two CTAs of a whole batch each, then four
+    (16, 16385, 16385), (17, 16385, 16390),  # eight, four
+    (1, 32768, 32768), (2, 32769, 32770),  # eight CTAs, a whole batch each and one entry more
+    (100, 33000, 33000),                   # two: longer than eight batches, several CTAs an SM
 ])
 def test_rows_around_the_cluster_rule(rows, n, stride):
     """The same checks at the lengths where the form or the cluster size changes."""
