@@ -46,9 +46,9 @@ KERNEL_SOURCE = os.path.join(ROOT, "paper_2605_31598_gb300", "csrc", "attn_kerne
 # first 16 hex digits of the sha256 of the attention-kernel source it was taken
 # on.  A workload or kernel source with no capture reports null.
 K1_DRAM_BYTES = {
-    ("qwen7b_stack", "887fab2e58e31b56"): 198649088,
-    ("qwen72b_stack", "887fab2e58e31b56"): 2048347648,
-    ("qwen7b_8streams", "887fab2e58e31b56"): 1729202176,
+    ("qwen7b_stack", "c286b2182a710e41"): 197721088,
+    ("qwen72b_stack", "c286b2182a710e41"): 2047845120,
+    ("qwen7b_8streams", "c286b2182a710e41"): 1727971328,
 }
 
 
